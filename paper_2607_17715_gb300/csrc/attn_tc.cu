@@ -127,6 +127,24 @@ constexpr int kSmemTiles = 2 /*Q_A, Q_B*/ + KSTAGES + VSTAGES;
 constexpr size_t kSmemBytes = 1024 /*align*/ + (size_t)TILE * kSmemTiles + 8 * NBAR + 16;
 static_assert(kSmemBytes <= 232448, "shared memory budget of one sm_100 CTA");
 
+// What depends on the head dimension D (128, or 64 in the plain kernel's instantiations
+// attn_tc64_*): a tile's bytes, its 64-channel swizzle blocks, the shared memory of a CTA.
+// kSplitP: P enters P.V as two bf16 terms, the rounded weight over the first 64 columns of
+// S_x and what the rounding left over the last 64 (relative error 2^-18 rather than 2^-9).
+// Heads of 64 channels were computed with fp32 weights on the CUDA cores and keep that
+// precision; at N = 64 the second term's MMAs cost as much as one tile's P.V does at 128.
+// Measured on 4 requests x 100 tokens x 1000 slots, 32 / 8 heads: the attend call 400 us on the
+// CUDA cores, 30.2 us here, 0.0017 off the 64-bit result either way (64 CTAs of 9 key tiles:
+// bound by the softmax chain of a CTA and its start, not by the tensor cores).
+template <int D>
+struct Geo {
+    static constexpr int kTile = BN * D * 2;
+    static constexpr int kBlocks = D / 64;
+    static constexpr bool kSplitP = D == 64;
+    static constexpr size_t kSmem = 1024 + (size_t)kTile * kSmemTiles + 8 * NBAR + 16;
+};
+static_assert(Geo<HD>::kTile == TILE && Geo<HD>::kSmem == kSmemBytes, "the fused kernel's layout");
+
 struct TcParams {                // CUtensorMap members carry their own alignment
     CUtensorMap tm_q;        // q_rot   [Lq*Btot][Sq'][Hq][128] box {64, G, TQ, 1}; Sq' = sq_pitch
     CUtensorMap tm_k;        // cache K [L*rows][Hkv][128]      box {64, 1, 128}
@@ -273,6 +291,12 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&v)[16
         : "memory");
 }
 
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&v)[8]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr),
+                 "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+                 : "memory");
+}
+
 __device__ __forceinline__ void tmem_ld_wait() {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
@@ -344,11 +368,12 @@ __device__ __forceinline__ void sts128_(uint32_t a, const uint4& v) {
 // KV head, pair) unit writes its normalised fp32 partial and log2-domain lse, then both softmax
 // warpgroups meet (named barrier 4); one thread releases the partials (a GPU-scope fence) and
 // takes a ticket.  In the CTA that takes the last one, warpgroup A merges every row of the
-// pair as attn_combine_kernel does: 32 threads a row, 4 channels each, eight splits' lse and
+// pair as attn_combine_kernel does: D / 4 threads a row, 4 channels each, eight splits' lse and
 // output slices loaded before any is used; lse = log2 sum_s 2^lse_s,
 // O = sum_s 2^(lse_s - lse) O_s.  Then the counter goes back to zero for the next launch.  No
 // thread waits on another CTA.  At most kMaxMergeSplits splits (the host merges by launch
 // beyond that).
+template <int D>
 __device__ __forceinline__ void split_merge(const TcParams& P, uint32_t sBar, int x, int r, int t0, int l,
                                             int b, int hk) {
     __threadfence();
@@ -373,8 +398,8 @@ __device__ __forceinline__ void split_merge(const TcParams& P, uint32_t sBar, in
     const int64_t part_rows = (int64_t)P.lq * P.batch_total * P.sq * P.hq;
     const int ns = P.n_split;
 #pragma unroll 1
-    for (int it = r; it < (rows_a + rows_b) * 32; it += BM) {
-        const int row = it >> 5, c4 = it & 31;
+    for (int it = r; it < (rows_a + rows_b) * (D / 4); it += BM) {
+        const int row = it / (D / 4), c4 = it % (D / 4);
         const int xr = row < rows_a ? 0 : 1, rr = row - xr * rows_a;
         const int t = (xr ? t0b : t0a) + rr / G, g = rr - (rr / G) * G;
         const int64_t row_id = (((int64_t)l * P.batch_total + b) * P.sq_pitch + t) * P.hq + hk * G + g;
@@ -399,7 +424,7 @@ __device__ __forceinline__ void split_merge(const TcParams& P, uint32_t sBar, in
                 o[i] = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (s0 + i < ns) {
                     ls[i] = __ldcg(P.part_lse + (int64_t)(s0 + i) * part_rows + lse_id);
-                    o[i] = __ldcg(reinterpret_cast<const float4*>(P.part_o + ((int64_t)(s0 + i) * part_rows + row_id) * HD) + c4);
+                    o[i] = __ldcg(reinterpret_cast<const float4*>(P.part_o + ((int64_t)(s0 + i) * part_rows + row_id) * D) + c4);
                 }
             }
 #pragma unroll
@@ -416,7 +441,7 @@ __device__ __forceinline__ void split_merge(const TcParams& P, uint32_t sBar, in
         uint2 pk;
         pk.x = pack_bf16(acc.x * inv, acc.y * inv);
         pk.y = pack_bf16(acc.z * inv, acc.w * inv);
-        *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(P.out) + row_id * HD + c4 * 4) = pk;
+        *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(P.out) + row_id * D + c4 * 4) = pk;
         if (P.lse != nullptr && c4 == 0) P.lse[lse_id] = (mx + log2f(wsum)) * 0.69314718055994531f;
     }
     if (r == 0) P.tickets[unit] = 0u;
@@ -501,7 +526,7 @@ __device__ __forceinline__ PairSpan pair_span(const TcParams& P, int pr, int sp,
 // kSif: the plain kernel over extraction C2 rows (TcParams::sif_k), its own instantiation.
 // kKpp: the plain kernel's decode instantiation, whose pairs with one query tile split their
 // key tiles between the two warpgroups (kpp: this pair does).
-template <bool kMerge, bool kSif = false, bool kKpp = false>
+template <bool kMerge, bool kSif = false, bool kKpp = false, int D = HD>
 __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, uint32_t sBar, int x,
                                             int quad, int lane, int t0, int l, int bl, int b,
                                             int hk, int sp, const PairSpan& span, uint32_t sf_base,
@@ -516,7 +541,7 @@ __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, u
     const int r = quad * 32 + lane;                 // row = TMEM lane
     const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
     const uint32_t colS = kColS + (uint32_t)x * BN;  // S_x, and P_x over its first 64 columns
-    const uint32_t colO = kColO + (uint32_t)x * HD;
+    const uint32_t colO = kColO + (uint32_t)x * D;
     const int t_row = min(t0 + r / G, P.sq - 1);    // rows past the suffix mirror its end
     const int lim = s_r + t_row;                    // last key this row may see
     const float sc = P.scale_log2;
@@ -581,7 +606,7 @@ __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, u
         // S_x(j) complete implies the P_x.V before it complete: O_x is current and may be scaled
         if (i >= 1 && __any_sync(0xffffffffu, resc)) {
 #pragma unroll 1
-            for (int c = 0; c < 8; ++c) {
+            for (int c = 0; c < D / 16; ++c) {
                 uint32_t ov[16];
                 tmem_ld16(tmem + lane_addr + colO + c * 16, ov);
                 tmem_ld_wait();
@@ -596,19 +621,29 @@ __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, u
         // P_j (bf16, keys 2c and 2c+1 packed in column c) over the first half of S_x
         const uint32_t p_addr = tmem + lane_addr + colS;
         const float neg_m = -m_sub;
+        // (kSplitP: 16 keys at a time, their second terms over the last 64 columns)
+        constexpr int PW = Geo<D>::kSplitP ? 8 : 16;       // packed words per store
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            uint32_t pk[16];
+        for (int c = 0; c < 64 / PW; ++c) {
+            uint32_t pk[PW], pl[Geo<D>::kSplitP ? PW : 1];
 #pragma unroll
-            for (int e = 0; e < 32; e += 2) {
+            for (int w = 0; w < PW; ++w) {
+                const int e = 2 * (c * PW + w);            // key of the tile
                 float a0, a1;
-                ffma2(a0, a1, __uint_as_float(sv[c][e]), __uint_as_float(sv[c][e + 1]), sc, neg_m);
+                ffma2(a0, a1, __uint_as_float(sv[e >> 5][e & 31]), __uint_as_float(sv[e >> 5][(e & 31) + 1]), sc, neg_m);
                 a0 = ex2(a0);
                 a1 = ex2(a1);
                 if (e & 2) fadd2(ps[2], ps[3], a0, a1); else fadd2(ps[0], ps[1], a0, a1);
-                pk[e >> 1] = pack_bf16(a0, a1);
+                pk[w] = pack_bf16(a0, a1);
+                if constexpr (Geo<D>::kSplitP)      // what the rounding left (exact differences)
+                    pl[w] = pack_bf16(a0 - __uint_as_float(pk[w] << 16), a1 - __uint_as_float(pk[w] & 0xffff0000u));
             }
-            tmem_st16(p_addr + (uint32_t)c * 16u, pk);
+            if constexpr (Geo<D>::kSplitP) {
+                tmem_st8(p_addr + (uint32_t)(c * PW), pk);
+                tmem_st8(p_addr + 64u + (uint32_t)(c * PW), pl);
+            } else {
+                tmem_st16(p_addr + (uint32_t)(c * PW), pk);
+            }
         }
         tmem_st_wait();
         const float sum = (ps[0] + ps[1]) + (ps[2] + ps[3]);
@@ -618,6 +653,7 @@ __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, u
         mbar_arrive(bar(B_PF + x));
     }
 
+    static_assert(!kKpp || D == HD, "the key ping-pong is the 128-channel decode kernel's");
     if (kKpp && kpp) {
         // the two halves meet: B leaves its row's (m, l) in the Q_B tile (unused with one
         // query tile), and A, once every MMA is done, folds O_B into O_A in TMEM with the
@@ -628,7 +664,7 @@ __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, u
             asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(xch), "f"(m_run), "f"(l_run) : "memory");
             asm volatile("bar.sync 4, 256;" ::: "memory");
             if constexpr (kMerge)
-                if (P.n_split > 1 && P.tickets != nullptr) split_merge(P, sBar, x, r, t0, l, b, hk);
+                if (P.n_split > 1 && P.tickets != nullptr) split_merge<D>(P, sBar, x, r, t0, l, b, hk);
             if (arrive_oe) {
                 tc_fence_before();
                 mbar_arrive(bar(B_OE));
@@ -675,9 +711,9 @@ __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, u
     const int64_t row_id = (((int64_t)l * P.batch_total + b) * P.sq_pitch + t) * P.hq + hk * G + g;
     const int64_t lse_id = (((int64_t)l * P.batch_total + b) * P.hq + hk * G + g) * P.sq_pitch + t;
     if (P.n_split == 1 && stage != 0u && n_kv > 0) {
-        const uint32_t sbase = stage + (uint32_t)x * TILE;
+        const uint32_t sbase = stage + (uint32_t)(x * Geo<D>::kTile);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 0; c < D / 32; ++c) {
             uint32_t ov[32];
             tmem_ld32(tmem + lane_addr + colO + c * 32, ov);
             tmem_ld_wait();
@@ -698,14 +734,14 @@ __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, u
             tc_fence_before();
             mbar_arrive(bar(B_OE));
         }
-        // the rows visible to the TMA engine, every row of the tile written, then one store of
-        // both 64-column halves (tokens past the suffix fall outside the map and are dropped)
+        // the rows visible to the TMA engine, every row of the tile written, then one store per
+        // 64-column block (tokens past the suffix fall outside the map and are dropped)
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         asm volatile("bar.sync %0, 128;" ::"r"(2 + x) : "memory");
         if (r == 0) {
             const int qz = l * P.batch_total + b;
             tma_store_4d(&P.tm_o, sbase, 0, hk * G, t0, qz);
-            tma_store_4d(&P.tm_o, sbase + HALF_TILE, 64, hk * G, t0, qz);
+            if constexpr (D == 128) tma_store_4d(&P.tm_o, sbase + HALF_TILE, 64, hk * G, t0, qz);
             asm volatile("cp.async.bulk.commit_group;" ::: "memory");
             // the CTA may leave once the store has read shared memory; its writes complete
             // with the grid
@@ -717,12 +753,12 @@ __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, u
         // each thread writes its own row, a full 32-byte sector per store: the lanes of a
         // warp hold rows of up to 32 different lines, so a narrower store would leave every
         // sector it touches half written
-        // (rows are 256 bytes apart, so the output's base alignment decides; the entry points
+        // (rows are 128 or 256 bytes apart, so the output's base alignment decides; the entry points
         // guarantee 16 bytes only)
-        __nv_bfloat16* orow = static_cast<__nv_bfloat16*>(P.out) + row_id * HD;
+        __nv_bfloat16* orow = static_cast<__nv_bfloat16*>(P.out) + row_id * D;
         const bool a32 = (reinterpret_cast<uintptr_t>(P.out) & 31u) == 0;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 0; c < D / 32; ++c) {
             uint32_t ov[32];
             tmem_ld32(tmem + lane_addr + colO + c * 32, ov);
             tmem_ld_wait();
@@ -748,9 +784,9 @@ __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, u
     } else {
         // partial over this split's keys: normalised O (fp32) and its log2-domain lse
         const int64_t part_rows = (int64_t)P.lq * P.batch_total * P.sq * P.hq;
-        float* orow = P.part_o + ((int64_t)sp * part_rows + row_id) * HD;
+        float* orow = P.part_o + ((int64_t)sp * part_rows + row_id) * D;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 0; c < D / 32; ++c) {
             uint32_t ov[32];
             if (n_kv > 0) {
                 tmem_ld32(tmem + lane_addr + colO + c * 32, ov);
@@ -772,7 +808,7 @@ __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, u
         if (t < P.sq)
             P.part_lse[(int64_t)sp * part_rows + lse_id] = any ? m_run + log2f(l_run) : -CUDART_INF_F;
         if constexpr (kMerge)
-            if (P.tickets != nullptr) split_merge(P, sBar, x, r, t0, l, b, hk);
+            if (P.tickets != nullptr) split_merge<D>(P, sBar, x, r, t0, l, b, hk);
     }
     if (arrive_oe) {          // O has been read out of TMEM: the next pair may overwrite it
         tc_fence_before();
@@ -801,7 +837,7 @@ struct RingState {
 // barrier phase that says Q is in shared memory.  wait_oe: a previous pair's epilogue must
 // have read O (phase oe_par of B_OE) before this pair's first P.V overwrites it.  B_QF says
 // that every S of the pair has read Q, and B_OD at the end that O is final.
-template <bool kHasB>
+template <bool kHasB, int D = HD>
 __device__ __forceinline__ void mma_issuer(const TcParams& P, uint32_t tmem, uint32_t sQ, uint32_t sK,
                                            uint32_t sV, uint32_t sBar, int n_kv, int q_ready,
                                            uint32_t q_par, RingState& st, bool wait_oe, uint32_t oe_par,
@@ -809,31 +845,36 @@ __device__ __forceinline__ void mma_issuer(const TcParams& P, uint32_t tmem, uin
     static_assert(KSTAGES == 3 && VSTAGES == 2, "the issue schedule assumes 3 K and 2 V stages");
     auto bar = [&](int i) { return sBar + 8u * (uint32_t)i; };
     constexpr uint32_t idS = idesc_bf16(BM, BN, false);
-    constexpr uint32_t idO = idesc_bf16(BM, HD, true);
-    constexpr uint64_t kTileDesc = (uint64_t)(TILE >> 4);     // one tile in descriptor units
+    constexpr uint32_t idO = idesc_bf16(BM, D, true);
+    constexpr uint64_t kTileDesc = (uint64_t)(Geo<D>::kTile >> 4);   // one tile in descriptor units
     // descriptors of tile bases; a K step adds its byte offset / 16 to the low field
     const uint64_t dQa = sw128_desc(sQ, 16, 1024);
-    const uint64_t dQb = sw128_desc(sQ + TILE, 16, 1024);
+    const uint64_t dQb = sw128_desc(sQ + Geo<D>::kTile, 16, 1024);
     const uint64_t dK0 = sw128_desc(sK, 16, 1024);
     const uint64_t dV0 = sw128_desc(sV, HALF_TILE, 1024);
     const uint32_t tS_a = tmem + kColS, tS_b = tmem + kColS + BN;
-    const uint32_t tO_a = tmem + kColO, tO_b = tmem + kColO + HD;
+    const uint32_t tO_a = tmem + kColO, tO_b = tmem + kColO + D;
 
-    // S = Q K^T (8 K steps of 16)
+    // S = Q K^T (D / 16 K steps of 16)
     auto s_block = [&](uint64_t dq, uint64_t dk, uint32_t d) {
 #pragma unroll
-        for (int kk = 0; kk < HD / 16; ++kk) {
+        for (int kk = 0; kk < D / 16; ++kk) {
             const uint64_t off = (uint64_t)(((kk >> 2) * HALF_TILE + (kk & 3) * 32) >> 4);
             mma_bf16(d, dq + off, dk + off, idS, kk > 0 ? 1u : 0u);
         }
     };
     // O += P V with P (bf16 pairs) from TMEM: 16 keys (8 columns) per step; the first step
     // of the first block overwrites O
+    constexpr int kKeyStep = 16 * 128;      // bytes of 16 keys' rows in a 64-channel block
     auto pv_block = [&](uint32_t p, uint64_t dv, uint32_t o, uint32_t acc0) {
 #pragma unroll
         for (int kk = 0; kk < BN / 16; ++kk)
-            mma_bf16_ts(o, p + (uint32_t)kk * 8u, dv + (uint64_t)((kk * 2048) >> 4), idO,
+            mma_bf16_ts(o, p + (uint32_t)kk * 8u, dv + (uint64_t)((kk * kKeyStep) >> 4), idO,
                         kk > 0 ? 1u : acc0);
+        if constexpr (Geo<D>::kSplitP)      // the weights' second term, over the same V
+#pragma unroll
+            for (int kk = 0; kk < BN / 16; ++kk)
+                mma_bf16_ts(o, p + 64u + (uint32_t)kk * 8u, dv + (uint64_t)((kk * kKeyStep) >> 4), idO, 1u);
     };
     auto wait = [&](int i, uint32_t parity) {
         mbar_wait(bar(i), parity, P.err, abort);
@@ -1751,11 +1792,12 @@ __device__ __forceinline__ void fused_suffix_prep(const FusedTcParams& F, int ts
 // that its CTA runs in turn: a pair's Q tiles once the MMAs of the previous pair have read
 // the last ones (B_QF), and the pairs' K and V tiles in order, each as soon as its ring stage
 // is free; whichever of the three can go first goes.
-template <bool kSif>
+template <bool kSif, int D>
 __device__ __forceinline__ void plain_producer(const TcParams& P, int l, int bl, int b, int hk,
                                                int p_first, int p_count, int sp, int s_r, uint32_t sQ,
                                                uint32_t sK, uint32_t sV, uint32_t sBar,
                                                volatile uint32_t* abort) {
+    constexpr int kTile = Geo<D>::kTile;
     auto bar = [&](int i) { return sBar + 8u * (uint32_t)i; };
     const int G = P.group;
     const int qz = l * P.batch_total + b;
@@ -1771,12 +1813,12 @@ __device__ __forceinline__ void plain_producer(const TcParams& P, int l, int bl,
     while (qi < p_count || pk < p_count || pv < p_count) {
         if (qi < p_count && (qi == 0 || mbar_test(bar(B_QF), (uint32_t)(qi - 1) & 1u))) {
             const PairSpan sq = pair_span(P, p_first + qi, sp, s_r);
-            mbar_expect_tx(bar(B_Q), sq.has_b ? 2 * TILE : TILE);
+            mbar_expect_tx(bar(B_Q), sq.has_b ? 2 * kTile : kTile);
             tma_load_4d(sQ, &P.tm_q, 0, hk * G, sq.t0a, qz, bar(B_Q));
-            tma_load_4d(sQ + HALF_TILE, &P.tm_q, 64, hk * G, sq.t0a, qz, bar(B_Q));
+            if (D == 128) tma_load_4d(sQ + HALF_TILE, &P.tm_q, 64, hk * G, sq.t0a, qz, bar(B_Q));
             if (sq.has_b) {
-                tma_load_4d(sQ + TILE, &P.tm_q, 0, hk * G, sq.t0b, qz, bar(B_Q));
-                tma_load_4d(sQ + TILE + HALF_TILE, &P.tm_q, 64, hk * G, sq.t0b, qz, bar(B_Q));
+                tma_load_4d(sQ + kTile, &P.tm_q, 0, hk * G, sq.t0b, qz, bar(B_Q));
+                if (D == 128) tma_load_4d(sQ + kTile + HALF_TILE, &P.tm_q, 64, hk * G, sq.t0b, qz, bar(B_Q));
             }
             ++qi;
             idle0 = -1;
@@ -1786,9 +1828,9 @@ __device__ __forceinline__ void plain_producer(const TcParams& P, int l, int bl,
                                                        (uint32_t)((gk / KSTAGES) - 1) & 1u))) {
             const int s = gk % KSTAGES;
             const int krow = key0 + (kSif ? span_tile(sk, jk) : sk.j_base + jk) * BN;
-            mbar_expect_tx(bar(B_KF + s), TILE);
-            tma_load_3d(sK + s * TILE, &P.tm_k, 0, hk, krow, bar(B_KF + s));
-            tma_load_3d(sK + s * TILE + HALF_TILE, &P.tm_k, 64, hk, krow, bar(B_KF + s));
+            mbar_expect_tx(bar(B_KF + s), kTile);
+            tma_load_3d(sK + s * kTile, &P.tm_k, 0, hk, krow, bar(B_KF + s));
+            if (D == 128) tma_load_3d(sK + s * kTile + HALF_TILE, &P.tm_k, 64, hk, krow, bar(B_KF + s));
             ++gk;
             if (++jk == sk.n_kv) {
                 jk = 0;
@@ -1801,9 +1843,9 @@ __device__ __forceinline__ void plain_producer(const TcParams& P, int l, int bl,
                                                        (uint32_t)((gv / VSTAGES) - 1) & 1u))) {
             const int s = gv % VSTAGES;
             const int vrow = key0 + (kSif ? span_tile(sv, jv) : sv.j_base + jv) * BN;
-            mbar_expect_tx(bar(B_VF + s), TILE);
-            tma_load_3d(sV + s * TILE, &P.tm_v, 0, hk, vrow, bar(B_VF + s));
-            tma_load_3d(sV + s * TILE + HALF_TILE, &P.tm_v, 64, hk, vrow, bar(B_VF + s));
+            mbar_expect_tx(bar(B_VF + s), kTile);
+            tma_load_3d(sV + s * kTile, &P.tm_v, 0, hk, vrow, bar(B_VF + s));
+            if (D == 128) tma_load_3d(sV + s * kTile + HALF_TILE, &P.tm_v, 64, hk, vrow, bar(B_VF + s));
             ++gv;
             if (++jv == sv.n_kv) {
                 jv = 0;
@@ -1853,17 +1895,20 @@ __global__ void __launch_bounds__(256) suffix_angles_kernel(const __grid_constan
 // kernel keeps its register allocation.  kSif (plain only): extraction C2 rows
 // (TcParams::sif_k), a kernel of its own (attn_tc_sif_kernel) so that the plain kernel's code
 // stays as it is.
-template <bool kFused, bool kMulti, bool kSif, bool kKpp = false>
+// D: head dimension (64 in the plain and the SIF kernel only).
+template <bool kFused, bool kMulti, bool kSif, bool kKpp = false, int D = HD>
 __device__ __forceinline__ void attn_tc_body(const typename KernelParams<kFused>::type& KP) {
+    static_assert(D == HD || (!kFused && !kKpp), "64 channels: the plain and SIF kernels");
+    constexpr int kTile = Geo<D>::kTile;
     const TcParams& P = tc_params(KP);
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                ~uintptr_t(1023));
     const uint32_t sQ = smem_u32(smem);             // Q_A, then Q_B
-    const uint32_t sK = sQ + 2 * TILE;
-    const uint32_t sV = sK + KSTAGES * TILE;
-    const uint32_t sBar = sV + VSTAGES * TILE;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + (size_t)TILE * kSmemTiles + 8 * NBAR);
+    const uint32_t sK = sQ + 2 * kTile;
+    const uint32_t sV = sK + KSTAGES * kTile;
+    const uint32_t sBar = sV + VSTAGES * kTile;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + (size_t)kTile * kSmemTiles + 8 * NBAR);
     volatile uint32_t* abort = tmem_slot + 1;      // set by the first wait that gives up
     auto bar = [&](int i) { return sBar + 8u * (uint32_t)i; };
 
@@ -1908,7 +1953,7 @@ __device__ __forceinline__ void attn_tc_body(const typename KernelParams<kFused>
         const int key0 = (int)((int64_t)(P.layer0 + l) * P.rows + P.req[bl].row_base);
         const int row = key0 + (kSif ? span_tile(ps0, 0) : j_base) * BN;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
+        for (int h = 0; h < Geo<D>::kBlocks; ++h) {
             tma_prefetch_4d(&P.tm_q, 64 * h, hk * G, t0a, qz);
             if (has_b) tma_prefetch_4d(&P.tm_q, 64 * h, hk * G, t0b, qz);
             tma_prefetch_3d(&P.tm_k, 64 * h, hk, row);
@@ -1983,7 +2028,7 @@ __device__ __forceinline__ void attn_tc_body(const typename KernelParams<kFused>
                     if (p_count > 1)
                         fused_rest_producer(KP, l, bl, b, hk, p_count, s_r, n_kv, sQ, sK, sV, sBar, abort);
             } else {
-                plain_producer<kSif>(P, l, bl, b, hk, p_first, p_count, sp, s_r, sQ, sK, sV, sBar, abort);
+                plain_producer<kSif, D>(P, l, bl, b, hk, p_first, p_count, sp, s_r, sQ, sK, sV, sBar, abort);
             }
         } else if (warp == 1 && lane == 0 && n_kv > 0) {
             // ------------------------------------------------------------ MMA issuer
@@ -2007,11 +2052,11 @@ __device__ __forceinline__ void attn_tc_body(const typename KernelParams<kFused>
                     const PairSpan ps = pi == 0 ? ps0 : pair_span(P, p_first + pi, sp, s_r);
                     const uint32_t q_par = (uint32_t)pi & 1u, oe_par = (uint32_t)(pi - 1) & 1u;
                     if (ps.has_b)
-                        mma_issuer<true>(P, tmem, sQ, sK, sV, sBar, ps.n_kv, B_Q, q_par, st, pi > 0, oe_par, abort);
+                        mma_issuer<true, D>(P, tmem, sQ, sK, sV, sBar, ps.n_kv, B_Q, q_par, st, pi > 0, oe_par, abort);
                     else if (kKpp && ps.n_kv >= 2 && pi == p_count - 1)   // key tiles ping-pong
                         mma_issuer_kpp(P, tmem, sQ, sK, sV, sBar, ps.n_kv, B_Q, q_par, st, pi > 0, oe_par, abort);
                     else
-                        mma_issuer<false>(P, tmem, sQ, sK, sV, sBar, ps.n_kv, B_Q, q_par, st, pi > 0, oe_par, abort);
+                        mma_issuer<false, D>(P, tmem, sQ, sK, sV, sBar, ps.n_kv, B_Q, q_par, st, pi > 0, oe_par, abort);
                 }
             }
         } else if (warp == 2 && lane == 0 && n_kv > 0 && writer) {
@@ -2066,7 +2111,7 @@ __device__ __forceinline__ void attn_tc_body(const typename KernelParams<kFused>
                 // warpgroups take alternate key tiles (mma_issuer_kpp) and merge at the end
                 const bool kpp = kKpp && !ps.has_b && ps.n_kv >= 2 && pi == p_count - 1;
                 if (x == 0 || ps.has_b || kpp) {
-                    softmax_tile<true, kSif, kKpp>(P, tmem, sBar, x, warp & 3, lane, x && !kpp ? ps.t0b : ps.t0a, l, bl,
+                    softmax_tile<true, kSif, kKpp, D>(P, tmem, sBar, x, warp & 3, lane, x && !kpp ? ps.t0b : ps.t0a, l, bl,
                                  b, hk, sp, ps, done, (uint32_t)pi & 1u, p_count > 1, abort,
                                  pi == p_count - 1 ? sQ : 0u, kpp);
                     done += kpp ? (uint32_t)((ps.n_kv + 1 - x) / 2) : (uint32_t)ps.n_kv;
@@ -2108,6 +2153,14 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_sif_kernel(const __grid_c
     attn_tc_body<false, false, true>(KP);
 }
 
+// Heads of 64 channels: the plain kernel, and extraction C2 rows.
+__global__ void __launch_bounds__(kThreads, 1) attn_tc64_kernel(const __grid_constant__ TcParams KP) {
+    attn_tc_body<false, false, false, false, 64>(KP);
+}
+__global__ void __launch_bounds__(kThreads, 1) attn_tc64_sif_kernel(const __grid_constant__ TcParams KP) {
+    attn_tc_body<false, false, true, false, 64>(KP);
+}
+
 // Decode steps (AttnParams::key_pingpong): the plain kernel whose last pair, when it has one
 // query tile, splits its key tiles between the two softmax warpgroups.
 __global__ void __launch_bounds__(kThreads, 1) attn_tc_decode_kernel(const __grid_constant__ TcParams KP) {
@@ -2115,9 +2168,10 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_decode_kernel(const __gri
 }
 
 // The kernel of an instantiation.
-template <bool kFused, bool kMulti, bool kSif, bool kKpp = false>
+template <bool kFused, bool kMulti, bool kSif, bool kKpp = false, int D = HD>
 const void* tc_kernel_fn() {
-    if constexpr (kSif) return reinterpret_cast<const void*>(&attn_tc_sif_kernel);
+    if constexpr (D == 64) return reinterpret_cast<const void*>(kSif ? &attn_tc64_sif_kernel : &attn_tc64_kernel);
+    else if constexpr (kSif) return reinterpret_cast<const void*>(&attn_tc_sif_kernel);
     else if constexpr (kKpp) return reinterpret_cast<const void*>(&attn_tc_decode_kernel);
     else return reinterpret_cast<const void*>(&attn_tc_kernel<kFused, kMulti>);
 }
@@ -2234,7 +2288,11 @@ cudaError_t launch_attn_combine(const AttnParams& a, cudaStream_t s) {
 }
 
 bool attn_tc_supported(int dtype, int d, int hq, int hkv) {
-    if (dtype != kDtypeBf16 || d != HD || hkv < 1 || hq % hkv) return false;
+    return d == HD && attn_tc_takes(dtype, d, hq, hkv);
+}
+
+bool attn_tc_takes(int dtype, int d, int hq, int hkv) {
+    if (dtype != kDtypeBf16 || (d != HD && d != 64) || hkv < 1 || hq % hkv) return false;
     const int g = hq / hkv;
     return g == 1 || g == 2 || g == 4 || g == 8 || g == 16;
 }
@@ -2243,19 +2301,19 @@ namespace {
 
 // Host-side preparation shared by the plain and the fused launch: function attributes once
 // per process, the register-split guard, the tensor maps and the scalar parameters.
-template <bool kFused, bool kMulti = false, bool kSif = false, bool kKpp = false>
+template <bool kFused, bool kMulti = false, bool kSif = false, bool kKpp = false, int D = HD>
 cudaError_t prepare_tc(const AttnParams& a, TcParams& p, dim3& grid) {
     constexpr int threads = kFused ? kThreadsFused : kThreads;
     constexpr int high = kFused ? kRegsHighFused : kRegsHigh;
     constexpr int low_total = kFused ? 128 * (kRegsLowFused + kRegsLoadFused) : 128 * kRegsLow;
     // once per process (one device per context; function-local statics: thread-safe)
     static const cudaError_t smem_err = cudaFuncSetAttribute(
-        tc_kernel_fn<kFused, kMulti, kSif, kKpp>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+        tc_kernel_fn<kFused, kMulti, kSif, kKpp, D>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Geo<D>::kSmem);
     if (smem_err != cudaSuccess) return smem_err;
     {   // the register split must not ask for more than the launch holds
         static const int launch_regs = []() {
             cudaFuncAttributes fa{};
-            return cudaFuncGetAttributes(&fa, tc_kernel_fn<kFused, kMulti, kSif, kKpp>()) == cudaSuccess ? fa.numRegs : -1;
+            return cudaFuncGetAttributes(&fa, tc_kernel_fn<kFused, kMulti, kSif, kKpp, D>()) == cudaSuccess ? fa.numRegs : -1;
         }();
         if (launch_regs < 0) return cudaErrorInvalidDeviceFunction;
         if (launch_regs * threads < low_total + 256 * high) return cudaErrorInvalidConfiguration;
@@ -2265,20 +2323,20 @@ cudaError_t prepare_tc(const AttnParams& a, TcParams& p, dim3& grid) {
     std::memset(&p, 0, sizeof(p));
     const int G = a.hq / a.hkv;
     const int tq = BM / G;
-    {   // Q: q_rot [Lq*Btot][Sq'][Hq][128] -> dims (d, Hq, Sq, Lq*Btot); tokens past Sq read 0
-        const cuuint64_t dims[4] = {HD, (cuuint64_t)a.hq, (cuuint64_t)a.sq,
+    {   // Q: q_rot [Lq*Btot][Sq'][Hq][d] -> dims (d, Hq, Sq, Lq*Btot); tokens past Sq read 0
+        const cuuint64_t dims[4] = {D, (cuuint64_t)a.hq, (cuuint64_t)a.sq,
                                     (cuuint64_t)a.lq * a.batch_total};
-        const cuuint64_t str[3] = {(cuuint64_t)HD * 2, (cuuint64_t)a.hq * HD * 2,
-                                   (cuuint64_t)pitch * a.hq * HD * 2};
+        const cuuint64_t str[3] = {(cuuint64_t)D * 2, (cuuint64_t)a.hq * D * 2,
+                                   (cuuint64_t)pitch * a.hq * D * 2};
         const cuuint32_t box[4] = {64, (cuuint32_t)G, (cuuint32_t)tq, 1};
         if (!encode(&p.tm_q, a.q_rot, 4, dims, str, box)) return cudaErrorInvalidValue;
         // out has q's layout: its 128-row tiles leave through the same boxes
         if (!encode(&p.tm_o, a.out, 4, dims, str, box)) return cudaErrorInvalidValue;
     }
-    {   // K, V: cache [L*rows][Hkv][128] -> dims (d, Hkv, L*rows); layer0 + lq <= L
+    {   // K, V: cache [L*rows][Hkv][d] -> dims (d, Hkv, L*rows); layer0 + lq <= L
         const int64_t lrows = (int64_t)(a.layer0 + a.lq) * a.rows;
-        const cuuint64_t dims[3] = {HD, (cuuint64_t)a.hkv, (cuuint64_t)lrows};
-        const cuuint64_t str[2] = {(cuuint64_t)HD * 2, (cuuint64_t)a.hkv * HD * 2};
+        const cuuint64_t dims[3] = {D, (cuuint64_t)a.hkv, (cuuint64_t)lrows};
+        const cuuint64_t str[2] = {(cuuint64_t)D * 2, (cuuint64_t)a.hkv * D * 2};
         const cuuint32_t box[3] = {64, 1, (cuuint32_t)BN};
         if (!encode(&p.tm_k, a.cache_k, 3, dims, str, box)) return cudaErrorInvalidValue;
         if (!encode(&p.tm_v, a.cache_v, 3, dims, str, box)) return cudaErrorInvalidValue;
@@ -2341,45 +2399,49 @@ cudaError_t prepare_tc(const AttnParams& a, TcParams& p, dim3& grid) {
 
 }  // namespace
 
-cudaError_t preload_attn_tc_kernels() {
+cudaError_t preload_attn_tc_kernels(int d) {
     cudaFuncAttributes fa{};
-    return cudaFuncGetAttributes(&fa, attn_tc_kernel<false>);
+    return d == 64 ? cudaFuncGetAttributes(&fa, attn_tc64_kernel) : cudaFuncGetAttributes(&fa, attn_tc_kernel<false>);
 }
 
-cudaError_t launch_attn_tc(const AttnParams& a, cudaStream_t s, Hook before) {
-    (void)cudaGetLastError();   // report this launch's error only, not a stale one
+namespace {
+
+template <bool kSif, bool kKpp, int D>
+cudaError_t launch_plain(const AttnParams& a, cudaStream_t s, Hook before) {
     TcParams p;
     dim3 grid;
-    if (a.sif_k > 0) {          // extraction C2 rows: their own instantiation, launched plainly
-        cudaError_t e = prepare_tc<false, false, true>(a, p, grid);
-        if (e != cudaSuccess) return e;
-        before();
-        attn_tc_sif_kernel<<<grid, kThreads, kSmemBytes, s>>>(p);
-        return cudaGetLastError();
-    }
-    cudaError_t e = a.key_pingpong ? prepare_tc<false, false, false, true>(a, p, grid) : prepare_tc<false>(a, p, grid);
+    cudaError_t e = prepare_tc<false, false, kSif, kKpp, D>(a, p, grid);
     if (e != cudaSuccess) return e;
     before();
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = Geo<D>::kSmem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
     if (a.dependent) {          // starts while the kernel before it runs (the producer waits)
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = grid;
-        cfg.blockDim = dim3(kThreads);
-        cfg.dynamicSmemBytes = kSmemBytes;
-        cfg.stream = s;
-        cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        e = a.key_pingpong ? cudaLaunchKernelEx(&cfg, attn_tc_decode_kernel, p)
-                           : cudaLaunchKernelEx(&cfg, attn_tc_kernel<false>, p);
-        if (e != cudaSuccess) return e;
-    } else if (a.key_pingpong) {
-        attn_tc_decode_kernel<<<grid, kThreads, kSmemBytes, s>>>(p);
-    } else {
-        attn_tc_kernel<false><<<grid, kThreads, kSmemBytes, s>>>(p);
     }
-    return cudaGetLastError();
+    void* args[1] = {&p};
+    e = cudaLaunchKernelExC(&cfg, tc_kernel_fn<false, false, kSif, kKpp, D>(), args);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_attn_tc(const AttnParams& a, cudaStream_t s, Hook before) {
+    (void)cudaGetLastError();   // report this launch's error only, not a stale one
+    if (a.d == 64) {
+        if (a.key_pingpong) return cudaErrorInvalidValue;
+        return a.sif_k > 0 ? launch_plain<true, false, 64>(a, s, before) : launch_plain<false, false, 64>(a, s, before);
+    }
+    if (a.d != HD) return cudaErrorInvalidValue;
+    // extraction C2 rows and decode steps: their own instantiations
+    if (a.sif_k > 0) return launch_plain<true, false, HD>(a, s, before);
+    return a.key_pingpong ? launch_plain<false, true, HD>(a, s, before) : launch_plain<false, false, HD>(a, s, before);
 }
 
 namespace {

@@ -315,7 +315,7 @@ c2kv_status c2kv_create(const c2kv_config* cfg, void* stream, c2kv_ctx** out) {
             // c2kv_attend_noalloc's scratch array and kernels, reserved now rather than at
             // its first call (lazy module loading)
             const bool tc = f.attn_impl != C2KV_ATTN_SIMT &&
-                            c2kv::attn_tc_supported(f.dtype, f.head_dim, f.n_q_heads, f.n_kv_heads);
+                            c2kv::attn_tc_takes(f.dtype, f.head_dim, f.n_q_heads, f.n_kv_heads);
             e = c2kv::noalloc_prepare(f.dtype, f.head_dim, tc, &c->noalloc_scratch);
         }
         if (e == cudaSuccess) {
@@ -785,8 +785,8 @@ cudaError_t attend_run(c2kv_ctx* c, c2kv_cache* cache, int32_t layer0, int32_t l
     const int32_t B = cache->batch;
     const bool use_tc =
         c->cfg.attn_impl != C2KV_ATTN_SIMT &&
-        c2kv::attn_tc_supported(c->cfg.dtype, c->cfg.head_dim, c->cfg.n_q_heads, c->cfg.n_kv_heads);
-    if (fused && (!use_tc || layer0 != 0 || lq != c->cfg.layers || B > c2kv::kMaxReq))
+        c2kv::attn_tc_takes(c->cfg.dtype, c->cfg.head_dim, c->cfg.n_q_heads, c->cfg.n_kv_heads);
+    if (fused && (!use_tc || c->cfg.head_dim != 128 || layer0 != 0 || lq != c->cfg.layers || B > c2kv::kMaxReq))
         return cudaErrorInvalidValue;
 
     // scratch: the suffix queries after RoPE (the attention kernels' Q operand); the fused
@@ -853,6 +853,7 @@ cudaError_t attend_run(c2kv_ctx* c, c2kv_cache* cache, int32_t layer0, int32_t l
         a.sq = n_suffix;
         a.hq = c->cfg.n_q_heads;
         a.hkv = c->cfg.n_kv_heads;
+        a.d = c->cfg.head_dim;
         a.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)c->cfg.head_dim));
         a.n_split = n_split;
         a.pairs_per_cta = c->cfg.attn_pairs;
@@ -1423,6 +1424,7 @@ c2kv_status c2kv_decode(c2kv_ctx* c, c2kv_cache* cache, int32_t layer, const voi
                 a.sq = 1;
                 a.hq = hq;
                 a.hkv = hkv;
+                a.d = d;
                 a.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)d));
                 a.n_split = n_split;
                 a.pairs_per_cta = c->cfg.attn_pairs;

@@ -15,7 +15,7 @@
 // context dtype like every cached activation).  The masked attention then takes one of two
 // routes.
 //
-// Tensor cores (bf16, d = 128, the group sizes attn_tc_kernel takes).  The mask splits into
+// Tensor cores (bf16, the group sizes attn_tc_kernel takes).  The mask splits into
 // pieces the suffix-attention kernel already computes:
 //   1. document rows: plain causal attention over document keys 0..t, i.e. a "suffix" of n
 //      tokens over an empty prefix;
@@ -26,7 +26,7 @@
 // Both are launches of attn_tc_kernel with a token pitch of n + m, so they read and write
 // the extraction layout in place.
 //
-// CUDA cores (fp32, d = 64, other group sizes): extract_attn_kernel runs every row with fp32
+// CUDA cores (fp32, other group sizes): extract_attn_kernel runs every row with fp32
 // accumulation: one CTA holds RB packed query rows (row r = t * G + g: token t, query head
 // h_kv * G + g) of one (layer, KV head), stages K/V tiles of KT keys in shared memory, and
 // skips the tiles none of its rows can see.
@@ -220,9 +220,9 @@ __global__ void __launch_bounds__(XNW * 32) extract_attn_kernel(const __grid_con
     }
 }
 
+template <int D>
 cudaError_t launch_tc(const ExtractParams& p, cudaStream_t s, cudaStream_t s2, cudaEvent_t fork,
                       cudaEvent_t join) {
-    constexpr int D = 128;
     extract_rope_kernel<__nv_bfloat16, D / 2 / Vec16<__nv_bfloat16>::N>
         <<<dim3((unsigned)p.n_all, (unsigned)p.lq), 256, 0, s>>>(p);
     cudaError_t e = cudaGetLastError();
@@ -241,6 +241,7 @@ cudaError_t launch_tc(const ExtractParams& p, cudaStream_t s, cudaStream_t s2, c
     a.sq_pitch = p.n_all;
     a.hq = p.hq;
     a.hkv = p.hkv;
+    a.d = D;
     a.scale_log2 = p.scale_log2;
     a.n_split = 1;
     a.pairs_per_cta = p.pairs_per_cta;
@@ -294,14 +295,15 @@ cudaError_t launch_typed(const ExtractParams& p, cudaStream_t s) {
 
 }  // namespace
 
-bool extract_uses_tc(int dtype, int d, int hq, int hkv) { return attn_tc_supported(dtype, d, hq, hkv); }
+bool extract_uses_tc(int dtype, int d, int hq, int hkv) { return attn_tc_takes(dtype, d, hq, hkv); }
 
 cudaError_t launch_extract(const ExtractParams& p, int dtype, int d, cudaStream_t s, cudaStream_t s2,
                            cudaEvent_t fork, cudaEvent_t join) {
     (void)cudaGetLastError();   // report this launch's error only, not a stale one
     if (p.n_all < 1 || p.lq < 1) return cudaSuccess;
     if (p.lq > 65535 || p.hkv > 65535) return cudaErrorInvalidValue;
-    if (extract_uses_tc(dtype, d, p.hq, p.hkv)) return launch_tc(p, s, s2, fork, join);
+    if (extract_uses_tc(dtype, d, p.hq, p.hkv))
+        return d == 64 ? launch_tc<64>(p, s, s2, fork, join) : launch_tc<128>(p, s, s2, fork, join);
     if (dtype == kDtypeF32 && d == 64) return launch_typed<float, 64>(p, s);
     if (dtype == kDtypeF32 && d == 128) return launch_typed<float, 128>(p, s);
     if (dtype == kDtypeBf16 && d == 64) return launch_typed<__nv_bfloat16, 64>(p, s);

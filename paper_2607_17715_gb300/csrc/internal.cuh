@@ -141,6 +141,7 @@ struct AttnParams {
                              // (tensor-core kernel only, and only with n_split == 1)
     int32_t hq;
     int32_t hkv;
+    int32_t d;               // head_dim (the tensor-core kernel's choice of instantiation)
     float scale_log2;        // log2(e) / sqrt(d)
     int32_t n_split;         // key-range splits per work unit (1 = write O directly)
     float* part_o;           // n_split > 1: [n_split][Lq][Btot][Sq][Hq][d] fp32, normalised
@@ -252,8 +253,11 @@ bool encode_tensor_map(CUtensorMap* tm, CUtensorMapDataType type, int rank, cons
                        const cuuint64_t* dims, const cuuint64_t* strides_bytes, const cuuint32_t* box,
                        CUtensorMapSwizzle swizzle);
 
-// Tensor-core attention (attn_tc.cu).
+// Tensor-core attention (attn_tc.cu).  attn_tc_takes: the plain kernel and its SIF form take
+// the head layout (bf16, d 64 or 128); attn_tc_supported: so do the fused and decode kernels
+// and C2KV_ATTN_TC (d 128).
 bool attn_tc_supported(int dtype, int d, int hq, int hkv);
+bool attn_tc_takes(int dtype, int d, int hq, int hkv);
 cudaError_t launch_attn_tc(const AttnParams& p, cudaStream_t s, Hook before = {});
 // Merge n_split partial (O, lse) over disjoint key ranges into out (bf16) and lse (attn_tc.cu).
 cudaError_t launch_attn_combine(const AttnParams& p, cudaStream_t s);
@@ -308,7 +312,7 @@ cudaError_t launch_attn_fused(cudaStream_t s, Hook before = {});
 // takes no device memory.
 cudaError_t preload_suffix_kernels(int dtype, int d);      // kv_kernels.cu
 cudaError_t preload_attn_simt_kernels(int dtype, int d);   // attn_simt.cu
-cudaError_t preload_attn_tc_kernels();                     // attn_tc.cu
+cudaError_t preload_attn_tc_kernels(int d);                // attn_tc.cu
 // The device address of c2kv_attend_noalloc's fixed scratch array on the current device, its
 // module loaded, with every kernel that call can launch (noalloc.cu); called by c2kv_create.
 cudaError_t noalloc_prepare(int dtype, int d, bool tc, void** scratch);

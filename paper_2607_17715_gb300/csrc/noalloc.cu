@@ -51,7 +51,7 @@ cudaError_t noalloc_prepare(int dtype, int d, bool tc, void** scratch) {
     void* p = nullptr;
     cudaError_t e = cudaGetSymbolAddress(&p, g_attend_scratch);
     if (e == cudaSuccess) e = preload_suffix_kernels(dtype, d);
-    if (e == cudaSuccess) e = tc ? preload_attn_tc_kernels() : preload_attn_simt_kernels(dtype, d);
+    if (e == cudaSuccess) e = tc ? preload_attn_tc_kernels(d) : preload_attn_simt_kernels(dtype, d);
     if (e != cudaSuccess) return e;
     *scratch = p;
     return cudaSuccess;
@@ -103,7 +103,7 @@ extern "C" c2kv_status c2kv_attend_noalloc(c2kv_ctx* ctx, c2kv_cache* cache, int
     void* const q_rot = v.noalloc_scratch;
     cudaError_t e = cudaSuccess;
     const bool use_tc = v.attn_impl != C2KV_ATTN_SIMT &&
-                        c2kv::attn_tc_supported(v.dtype, v.head_dim, v.n_q_heads, v.n_kv_heads);
+                        c2kv::attn_tc_takes(v.dtype, v.head_dim, v.n_q_heads, v.n_kv_heads);
     for (int32_t b0 = 0; e == cudaSuccess && b0 < B; b0 += c2kv::kMaxReq) {
         const int32_t nb = B - b0 < c2kv::kMaxReq ? B - b0 : c2kv::kMaxReq;
         c2kv::SuffixParams s{};
@@ -147,6 +147,7 @@ extern "C" c2kv_status c2kv_attend_noalloc(c2kv_ctx* ctx, c2kv_cache* cache, int
         a.sq = n_suffix;
         a.hq = v.n_q_heads;
         a.hkv = v.n_kv_heads;
+        a.d = v.head_dim;
         a.scale_log2 = (float)(1.4426950408889634 / __builtin_sqrt((double)v.head_dim));
         a.pairs_per_cta = v.attn_pairs;
         for (int32_t i = 0; i < nb; ++i) a.req[i] = s.req[i];

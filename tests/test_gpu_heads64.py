@@ -1,0 +1,81 @@
+"""bf16 heads of 64 channels on the tensor cores: the suffix attention and the extraction
+attention against the oracle and against the CUDA-core kernel, at the edges of the query and key
+tiles (128 packed rows, 128 keys), over the group sizes and key-range splits."""
+import numpy as np
+import pytest
+import torch
+
+import synth
+from tests import _gpu_helpers as H
+from tests.test_gpu_extract import _extract_case
+from tests.test_gpu_parity import _attend_case
+
+pytestmark = pytest.mark.gpu
+
+D64 = synth.scaled(synth.workload("llama8b"), layers=1, head_dim=64, chunks_per_request=2, pool_chunks=2)
+
+
+@pytest.mark.parametrize("hq,hkv,sq,tokens,k", [
+    (4, 1, 1, 64, 1),        # one row tile, keys end one past a tile (2 x 64 slots + 1)
+    (4, 1, 32, 256, 4),      # exactly one 128-row tile
+    (4, 1, 33, 252, 4),      # one token past it
+    (8, 2, 64, 300, 10),     # exactly a pair of tiles
+    (8, 2, 65, 300, 10),     # a second pair of one token
+    (2, 2, 129, 64, 4),      # G = 1: a tile past one pair's half
+    (32, 2, 17, 97, 16),     # G = 16: eight tokens a tile
+    (16, 2, 47, 2048, 1),    # 4096 slots, G = 8
+])
+def test_attend(hq, hkv, sq, tokens, k):
+    _attend_case(synth.scaled(D64, n_q_heads=hq, n_kv_heads=hkv, chunk_tokens=tokens, ratio_k=k), n_suffix=sq)
+
+
+@pytest.mark.parametrize("split", [2, 5, 16])
+def test_attend_splits(split):
+    # three key tiles: with more splits some are empty, and they merge in the kernel
+    _attend_case(synth.scaled(D64, chunk_tokens=64, chunks_per_request=1, pool_chunks=1), n_suffix=300,
+                 attn_split=split)
+
+
+def test_attend_layer_of_a_batch():
+    wl = synth.scaled(synth.workload("batched"), head_dim=64, layers=3, batch=3, chunks_per_request=4,
+                      pool_chunks=32, n_suffix=70)
+    _attend_case(wl, layer=1)
+
+
+@pytest.mark.parametrize("n,k", [(512, 4), (128, 1), (129, 16), (33, 4), (1, 1), (700, 10)])
+def test_extract(n, k):
+    _extract_case(D64, n, k, layers=2 if n < 200 else 1)
+
+
+def test_weights_keep_more_than_bf16():
+    """The tensor-core kernel's weights enter P.V as two bf16 terms, so its output is off the
+    CUDA-core kernel's (fp32 weights) by at most a rounding flip of the bf16 output (2^-8 of the
+    value) and, per unit weight, 2^-17 of the largest value; four times that covers the two
+    kernels' fp32 sums.  Weights of one bf16 term would be off by 2^-9 of it."""
+    c2kv = H.lib()
+    wl = synth.scaled(D64, n_suffix=50, chunks_per_request=4, pool_chunks=4)
+    (ids, offs), = synth.requests(wl)
+    chunks = H.oracle_chunks_meanpool(wl, ids)
+    q, ks, vs = (H.to_dev(x, wl) for x in synth.suffix(wl))
+    outs = []
+    for impl in (c2kv.ATTN_AUTO, c2kv.ATTN_SIMT):
+        ctx = H.make_ctx(wl, pool_slots=4 * 128 + 16, attn_impl=impl)
+        try:
+            dev = H.load_stored(ctx, wl, chunks)
+            cache = c2kv.c2kv_compose(ctx, [0, len(ids)], [dev[c] for c in ids], offs, suffix_capacity=50)
+            out = torch.full_like(q, float("nan"))
+            c2kv.c2kv_attend(ctx, cache, -1, q, ks, vs, 50, out)
+            c2kv.c2kv_sync(ctx)
+            outs.append(out.double().cpu().numpy())
+        finally:
+            c2kv.c2kv_destroy(ctx)
+    vmax = max(float(vs.abs().max()), max(float(np.abs(c[1]).max()) for c in chunks.values()))
+    allowed = 2.0 ** -8 * np.abs(outs[1]) + 4 * 2.0 ** -17 * vmax
+    assert (np.abs(outs[0] - outs[1]) <= allowed).all(), float((np.abs(outs[0] - outs[1]) - allowed).max())
+
+
+def test_forced_tensor_cores_stay_refused():
+    c2kv = H.lib()
+    with pytest.raises(c2kv.C2KVError) as e:
+        H.make_ctx(D64, pool_slots=64, attn_impl=c2kv.ATTN_TC)
+    assert e.value.status == c2kv.ERR_UNSUPPORTED
