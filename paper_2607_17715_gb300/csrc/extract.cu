@@ -27,22 +27,15 @@
 // the extraction layout in place.
 //
 // CUDA cores (fp32, other group sizes): extract_attn_kernel runs every row with fp32
-// accumulation: one CTA holds RB packed query rows (row r = t * G + g: token t, query head
-// h_kv * G + g) of one (layer, KV head), stages K/V tiles of KT keys in shared memory, and
-// skips the tiles none of its rows can see.
-#include <math_constants.h>
+// accumulation through attention_core (attn_core.cuh): packed row r = t * G + g is token t,
+// query head h_kv * G + g, and the tiles that none of a CTA's rows can see are skipped.
+#include <algorithm>
 
-#include "internal.cuh"
+#include "attn_core.cuh"
 #include "rope.cuh"
-#include "vec16.cuh"
 
 namespace c2kv {
 namespace {
-
-constexpr int XRB = 16;   // query rows per CTA
-constexpr int XKT = 32;   // keys per staged tile (one per lane)
-constexpr int XNW = 4;    // warps per CTA
-constexpr int XRPW = XRB / XNW;
 
 // Extraction position of token t of an (n, k) chunk.
 __device__ __forceinline__ int extract_pos(int t, int n, int k) {
@@ -50,15 +43,6 @@ __device__ __forceinline__ int extract_pos(int t, int n, int k) {
     const int j = t - n;
     const int end = (j + 1) * k < n ? (j + 1) * k : n;
     return end - 1;
-}
-
-// Whether token tq may attend to token tk under the SIF mask.
-__device__ __forceinline__ bool sif_visible(int tq, int tk, int n, int k) {
-    if (tq < n) return tk <= tq;                               // document: causal, no C2 tokens
-    const int j = tq - n;
-    if (tk >= n) return tk - n <= j;                           // C2 tokens c_0 .. c_j
-    const int blk = tk / k;
-    return blk == j || blk == 0;                               // its block and the sink block
 }
 
 template <typename T, int VPH>
@@ -94,130 +78,69 @@ __global__ void __launch_bounds__(256) extract_rope_kernel(const __grid_constant
     }
 }
 
-template <typename T>
-__device__ __forceinline__ float ldx(const T* p) { return static_cast<float>(*p); }
-template <>
-__device__ __forceinline__ float ldx<__nv_bfloat16>(const __nv_bfloat16* p) { return __bfloat162float(*p); }
-
+// The rows of one (layer, KV head) under the SIF mask, for attention_core.
 template <typename T, int D>
-__global__ void __launch_bounds__(XNW * 32) extract_attn_kernel(const __grid_constant__ ExtractParams P) {
-    __shared__ float qs[XRB][D];
-    __shared__ float ks[XKT][D + 1];
-    __shared__ float vs[XKT][D];
-    const int G = P.hq / P.hkv;
-    const int l = blockIdx.z;
-    const int hk = blockIdx.y;
-    const int row0 = blockIdx.x * XRB;
-    const int nrows = P.n_all * G;
-    const int n = P.n, k = P.ratio;
-    const T* qr = static_cast<const T*>(P.q_rot);
-
-    for (int i = threadIdx.x; i < XRB * D; i += XNW * 32) {
-        const int r = i / D, c = i - (i / D) * D;
-        const int pr = row0 + r;
-        float val = 0.f;
-        if (pr < nrows) {
-            const int t = pr / G, g = pr - (pr / G) * G;
-            val = ldx(qr + (((int64_t)l * P.n_all + t) * P.hq + hk * G + g) * D + c);
-        }
-        qs[r][c] = val;
+struct SifJob {
+    const ExtractParams& p;
+    int l, hk, g_heads;
+    int row0, t0, t1;                 // this CTA's first packed row, first and last token
+    int nrows, nkeys;
+    int doc_end;                      // document keys its document rows see: [0, doc_end)
+    int blk_lo, blk_hi, sink;         // document keys its C2 rows see: [0, sink) and within [blk_lo, blk_hi)
+    const T *k, *v;
+    int64_t stride;
+    float scale_log2;
+    __device__ int64_t row_off(int r) const {
+        const int t = r / g_heads, g = r - t * g_heads;
+        return (((int64_t)l * p.n_all + t) * p.hq + hk * g_heads + g) * D;
     }
-
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    float m[XRPW], lsum[XRPW], acc[XRPW][D / 32];
-#pragma unroll
-    for (int rr = 0; rr < XRPW; ++rr) {
-        m[rr] = -CUDART_INF_F;
-        lsum[rr] = 0.f;
-#pragma unroll
-        for (int c = 0; c < D / 32; ++c) acc[rr][c] = 0.f;
+    __device__ const T* q_row(int r) const { return static_cast<const T*>(p.q_rot) + row_off(r); }
+    __device__ T* out_row(int r) const { return static_cast<T*>(p.out) + row_off(r); }
+    __device__ float* lse_at(int r) const {
+        if (p.lse == nullptr) return nullptr;
+        const int t = r / g_heads, g = r - t * g_heads;
+        return p.lse + ((int64_t)l * p.hq + hk * g_heads + g) * p.n_all + t;
     }
-    // key ranges some row of this CTA may see: causal document keys up to the last document
-    // row, and for C2 rows c_ja .. c_jb the sink block, their blocks and c_0 .. c_jb
-    const int tq0 = row0 / G;
-    const int tq1 = min(P.n_all - 1, (row0 + XRB - 1) / G);
-    const int doc_end = tq0 < n ? min(tq1, n - 1) + 1 : 0;
-    const bool has_c2 = tq1 >= n;
-    const int ja = max(tq0 - n, 0), jb = tq1 - n;
-    const int sink_end = min(k, n);
-    const int blk_lo = ja * k, blk_hi = has_c2 ? min((jb + 1) * k, n) : 0;
-    const int c2_end = has_c2 ? n + jb + 1 : 0;
-    auto tile_needed = [&](int k0) {
-        const int k1 = k0 + XKT;
+    __device__ bool needed(int k0, int k1) const {
         if (k0 < doc_end) return true;
-        if (!has_c2) return false;
-        return k0 < sink_end || (k1 > blk_lo && k0 < blk_hi) || (k1 > n && k0 < c2_end);
-    };
-    const int nkeys = has_c2 ? c2_end : doc_end;
-    const int64_t row_stride = (int64_t)P.hkv * D;
-    const T* kb = static_cast<const T*>(P.k_rot) + ((int64_t)l * P.n_all * P.hkv + hk) * D;
-    const T* vb = static_cast<const T*>(P.v) + ((int64_t)l * P.n_all * P.hkv + hk) * D;
-    const float sc = P.scale_log2;
-
-    for (int k0 = 0; k0 < nkeys; k0 += XKT) {
-        if (!tile_needed(k0)) continue;                        // the same for the whole CTA
-        __syncthreads();
-        for (int i = threadIdx.x; i < XKT * D; i += XNW * 32) {
-            const int r = i / D, c = i - (i / D) * D;
-            float kv = 0.f, vv = 0.f;
-            if (k0 + r < nkeys) {
-                kv = ldx(kb + (int64_t)(k0 + r) * row_stride + c);
-                vv = ldx(vb + (int64_t)(k0 + r) * row_stride + c);
-            }
-            ks[r][c] = kv;
-            vs[r][c] = vv;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int rr = 0; rr < XRPW; ++rr) {
-            const int r = warp + XNW * rr;
-            const int pr = row0 + r;
-            if (pr >= nrows) continue;                           // warp-uniform
-            const int tq = pr / G;
-            const int tk = k0 + lane;
-            float s = -CUDART_INF_F;
-            if (tk < nkeys && sif_visible(tq, tk, n, k)) {
-                float dot = 0.f;
-#pragma unroll 16
-                for (int c = 0; c < D; ++c) dot = fmaf(qs[r][c], ks[lane][c], dot);
-                s = dot * sc;
-            }
-            float mx = s;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-            const float m_new = fmaxf(m[rr], mx);
-            if (m_new == -CUDART_INF_F) continue;                // warp-uniform: nothing visible yet
-            const float p = (s == -CUDART_INF_F) ? 0.f : exp2f(s - m_new);
-            const float alpha = exp2f(m[rr] - m_new);
-            float ps = p;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) ps += __shfl_xor_sync(0xffffffffu, ps, o);
-            lsum[rr] = lsum[rr] * alpha + ps;
-#pragma unroll
-            for (int c = 0; c < D / 32; ++c) acc[rr][c] *= alpha;
-            for (int jk = 0; jk < XKT; ++jk) {
-                const float pj = __shfl_sync(0xffffffffu, p, jk);
-#pragma unroll
-                for (int c = 0; c < D / 32; ++c) acc[rr][c] = fmaf(pj, vs[jk][lane + 32 * c], acc[rr][c]);
-            }
-            m[rr] = m_new;
-        }
+        if (t1 < p.n) return false;                              // document rows only
+        return k0 < sink || (k1 > blk_lo && k0 < blk_hi) || k1 > p.n;
     }
-
-    T* out = static_cast<T*>(P.out);
-#pragma unroll
-    for (int rr = 0; rr < XRPW; ++rr) {
-        const int pr = row0 + warp + XNW * rr;
-        if (pr >= nrows) continue;
-        const int t = pr / G, g = pr - (pr / G) * G;
-        const int h = hk * G + g;
-        const float inv = 1.f / lsum[rr];                        // every row sees itself
-        const int64_t off = (((int64_t)l * P.n_all + t) * P.hq + h) * D;
-#pragma unroll
-        for (int c = 0; c < D / 32; ++c) out[off + lane + 32 * c] = static_cast<T>(acc[rr][c] * inv);
-        if (P.lse != nullptr && lane == 0)
-            P.lse[((int64_t)l * P.hq + h) * P.n_all + t] = (m[rr] + log2f(lsum[rr])) * 0.69314718055994531f;
+    __device__ bool whole(int, int k1) const { return t1 < p.n && k1 - 1 <= t0; }
+    __device__ int row(int r) const { return r / g_heads; }               // its token
+    __device__ bool sees(int t, int key) const {
+        const int n = p.n;
+        if (t < n) return key <= t;                              // document: causal, no C2 tokens
+        const int j = t - n;
+        if (key >= n) return key - n <= j;                       // C2 tokens c_0 .. c_j
+        return key < p.ratio || (int64_t)key >= (int64_t)j * p.ratio && (int64_t)key < ((int64_t)j + 1) * p.ratio;
     }
+};
+
+template <typename T, int D, int RT>
+__global__ void __launch_bounds__(kCoreThreads, core_ctas(D, RT)) extract_attn_kernel(const __grid_constant__ ExtractParams P, int ns) {
+    extern __shared__ __align__(16) uint8_t core_smem[];
+    SifJob<T, D> j{P};
+    j.l = blockIdx.z;
+    j.hk = blockIdx.y;
+    j.g_heads = P.hq / P.hkv;
+    // last rows first: under the causal mask they see the most keys
+    j.row0 = (int)((gridDim.x - 1 - blockIdx.x) / (unsigned)ns) * 16 * RT;
+    j.nrows = P.n_all * j.g_heads;
+    j.t0 = j.row0 / j.g_heads;
+    j.t1 = min(P.n_all - 1, (j.row0 + 16 * RT - 1) / j.g_heads);
+    const int n = P.n, ja = max(j.t0 - n, 0), jb = j.t1 - n;
+    const bool c2 = j.t1 >= n;
+    j.doc_end = j.t0 < n ? min(j.t1, n - 1) + 1 : 0;
+    j.sink = c2 ? min(P.ratio, n) : 0;
+    j.blk_lo = c2 ? min((int64_t)ja * P.ratio, (int64_t)n) : 0;
+    j.blk_hi = c2 ? min(((int64_t)jb + 1) * P.ratio, (int64_t)n) : 0;
+    j.nkeys = c2 ? n + jb + 1 : j.doc_end;
+    j.stride = (int64_t)P.hkv * D;
+    j.k = static_cast<const T*>(P.k_rot) + ((int64_t)j.l * P.n_all * P.hkv + j.hk) * D;
+    j.v = static_cast<const T*>(P.v) + ((int64_t)j.l * P.n_all * P.hkv + j.hk) * D;
+    j.scale_log2 = P.scale_log2;
+    attention_core<T, D, RT>(j, j.row0, ns, (int)(blockIdx.x % (unsigned)ns), core_smem);   // (the cluster rank)
 }
 
 template <int D>
@@ -281,16 +204,48 @@ cudaError_t launch_tc(const ExtractParams& p, cudaStream_t s, cudaStream_t s2, c
     return e;
 }
 
+template <typename T, int D, int RT>
+const CoreKernel<D, RT>& ready() {
+    static const CoreKernel<D, RT> k(reinterpret_cast<const void*>(&extract_attn_kernel<T, D, RT>), core_sms());
+    return k;
+}
+
+template <typename T, int D, int RT>
+cudaError_t launch_rt(const ExtractParams& p, int ns, bool alone, cudaStream_t s) {
+    const int64_t gx = ((int64_t)p.n_all * (p.hq / p.hkv) + 16 * RT - 1) / (16 * RT) * ns;
+    if (gx > 0x7fffffffLL) return cudaErrorInvalidValue;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)gx, (unsigned)p.hkv, (unsigned)p.lq);
+    cfg.blockDim = dim3(kCoreThreads);
+    cfg.dynamicSmemBytes = alone ? kCoreAlone : Core<D, RT>::kSmem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    if (ns > 1) {
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)ns;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+    }
+    return cudaLaunchKernelEx(&cfg, extract_attn_kernel<T, D, RT>, p, ns);
+}
+
 template <typename T, int D>
 cudaError_t launch_typed(const ExtractParams& p, cudaStream_t s) {
     constexpr int VPH = D / 2 / Vec16<T>::N;
     extract_rope_kernel<T, VPH><<<dim3((unsigned)p.n_all, (unsigned)p.lq), 256, 0, s>>>(p);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const int G = p.hq / p.hkv;
-    const dim3 grid((unsigned)((p.n_all * G + XRB - 1) / XRB), (unsigned)p.hkv, (unsigned)p.lq);
-    extract_attn_kernel<T, D><<<grid, XNW * 32, 0, s>>>(p);
-    return cudaGetLastError();
+    const CoreKernel<D, 4>& large = ready<T, D, 4>();
+    const CoreKernel<D, 1>& small = ready<T, D, 1>();
+    if (large.err != cudaSuccess || small.err != cudaSuccess) return large.err != cudaSuccess ? large.err : small.err;
+    // (the causal rows see half of the keys on average)
+    const CorePlan plan = core_plan((int64_t)p.n_all * (p.hq / p.hkv), (int64_t)p.hkv * p.lq, (p.n_all + 1) / 2, D,
+                                    [&](bool sm, int ns, bool alone) {
+                                        return sm ? small.slots[alone][ns] : large.slots[alone][ns];
+                                    });
+    return plan.small ? launch_rt<T, D, 1>(p, plan.ns, plan.alone, s) : launch_rt<T, D, 4>(p, plan.ns, plan.alone, s);
 }
 
 }  // namespace
