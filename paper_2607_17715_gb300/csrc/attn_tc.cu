@@ -481,12 +481,8 @@ __device__ __forceinline__ int span_tile(const PairSpan& o, int i) {
     const int i1 = i - (o.lead0 ? 1 : 0);
     return i1 < 0 ? 0 : i1 < o.n_mid ? o.j_base + i1 : o.j_tail + (i1 - o.n_mid);
 }
-__device__ __forceinline__ PairSpan pair_span(const TcParams& P, int pr, int sp, int s_r) {
-    PairSpan o;
-    o.t0a = 2 * pr * P.tq;
-    o.t0b = o.t0a + P.tq;
-    o.has_b = o.t0b < P.sq;
-    o.t_last = min(P.sq - 1, (o.has_b ? o.t0b : o.t0a) + P.tq - 1);
+// The key tiles (of split sp) that the query tokens [t0a, t_last] of `o` see.
+__device__ __forceinline__ void span_keys(const TcParams& P, PairSpan& o, int sp, int s_r) {
     o.lead0 = false;
     if (P.sif_k > 0) {
         // extraction C2 rows c_j, j in [t0a, t_last], over a chunk of n = s_r document keys:
@@ -501,7 +497,7 @@ __device__ __forceinline__ PairSpan pair_span(const TcParams& P, int pr, int sp,
         o.n_mid = b1 - b0 + 1;
         o.j_tail = c0;
         o.n_kv = (o.lead0 ? 1 : 0) + o.n_mid + max(0, c1 - c0 + 1);
-        return o;
+        return;
     }
     const int n_kv_all = (s_r + o.t_last + 1 + BN - 1) / BN;
     const int per_split = (n_kv_all + P.n_split - 1) / P.n_split;
@@ -509,6 +505,24 @@ __device__ __forceinline__ PairSpan pair_span(const TcParams& P, int pr, int sp,
     o.n_kv = max(0, min(n_kv_all, o.j_base + per_split) - o.j_base);
     o.n_mid = o.n_kv;
     o.j_tail = o.j_base + o.n_kv;
+}
+__device__ __forceinline__ PairSpan pair_span(const TcParams& P, int pr, int sp, int s_r) {
+    PairSpan o;
+    o.t0a = 2 * pr * P.tq;
+    o.t0b = o.t0a + P.tq;
+    o.has_b = o.t0b < P.sq;
+    o.t_last = min(P.sq - 1, (o.has_b ? o.t0b : o.t0a) + P.tq - 1);
+    span_keys(P, o, sp, s_r);
+    return o;
+}
+// One query tile alone (the solo kernel's unit).
+__device__ __forceinline__ PairSpan tile_span(const TcParams& P, int qt, int sp, int s_r) {
+    PairSpan o;
+    o.t0a = qt * P.tq;
+    o.t0b = P.sq;
+    o.has_b = false;
+    o.t_last = min(P.sq - 1, o.t0a + P.tq - 1);
+    span_keys(P, o, sp, s_r);
     return o;
 }
 
@@ -526,7 +540,10 @@ __device__ __forceinline__ PairSpan pair_span(const TcParams& P, int pr, int sp,
 // kSif: the plain kernel over extraction C2 rows (TcParams::sif_k), its own instantiation.
 // kKpp: the plain kernel's decode instantiation, whose pairs with one query tile split their
 // key tiles between the two warpgroups (kpp: this pair does).
-template <bool kMerge, bool kSif = false, bool kKpp = false, int D = HD>
+// kO: the first TMEM column of O_A.  kDbl (x = 0): S and P alternate between two column blocks and
+// their barriers (B_SF, B_PF and the next ones); P.V(j - 1) may then still run when S(j) is read,
+// so a rescale of O waits for it (B_OE, one phase per P.V).
+template <bool kMerge, bool kSif = false, bool kKpp = false, int D = HD, uint32_t kO = kColO, bool kDbl = false>
 __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, uint32_t sBar, int x,
                                             int quad, int lane, int t0, int l, int bl, int b,
                                             int hk, int sp, const PairSpan& span, uint32_t sf_base,
@@ -541,7 +558,7 @@ __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, u
     const int r = quad * 32 + lane;                 // row = TMEM lane
     const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
     const uint32_t colS = kColS + (uint32_t)x * BN;  // S_x, and P_x over its first 64 columns
-    const uint32_t colO = kColO + (uint32_t)x * D;
+    const uint32_t colO = kO + (uint32_t)x * D;
     const int t_row = min(t0 + r / G, P.sq - 1);    // rows past the suffix mirror its end
     const int lim = s_r + t_row;                    // last key this row may see
     const float sc = P.scale_log2;
@@ -553,11 +570,12 @@ __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, u
     // tile; i counts the tiles it has taken
     const bool kpp = kKpp && kpp_pair;
     for (int j = kpp ? x : 0, i = 0; j < n_kv; j += kpp ? 2 : 1, ++i) {
-        mbar_wait(bar(B_SF + x), (sf_base + (uint32_t)i) & 1u, P.err, abort);
+        const uint32_t dbl = kDbl ? (uint32_t)i & 1u : 0u;
+        mbar_wait(bar(B_SF + x + (int)dbl), (kDbl ? (uint32_t)i >> 1 : sf_base + (uint32_t)i) & 1u, P.err, abort);
         tc_fence_after();
         uint32_t sv[4][32];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) tmem_ld32(tmem + lane_addr + colS + c * 32, sv[c]);
+        for (int c = 0; c < 4; ++c) tmem_ld32(tmem + lane_addr + colS + dbl * BN + c * 32, sv[c]);
         tmem_ld_wait();
 
         const int kbase = (kSif ? span_tile(span, j) : span.j_base + j) * BN;
@@ -605,6 +623,10 @@ __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, u
 
         // S_x(j) complete implies the P_x.V before it complete: O_x is current and may be scaled
         if (i >= 1 && __any_sync(0xffffffffu, resc)) {
+            if constexpr (kDbl) {
+                mbar_wait(bar(B_OE), (uint32_t)(i - 1) & 1u, P.err, abort);
+                tc_fence_after();
+            }
 #pragma unroll 1
             for (int c = 0; c < D / 16; ++c) {
                 uint32_t ov[16];
@@ -619,7 +641,7 @@ __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, u
 #pragma unroll
         for (int e = 0; e < 4; ++e) ps[e] = 0.f;
         // P_j (bf16, keys 2c and 2c+1 packed in column c) over the first half of S_x
-        const uint32_t p_addr = tmem + lane_addr + colS;
+        const uint32_t p_addr = tmem + lane_addr + colS + dbl * BN;
         const float neg_m = -m_sub;
         // (kSplitP: 16 keys at a time, their second terms over the last 64 columns)
         constexpr int PW = Geo<D>::kSplitP ? 8 : 16;       // packed words per store
@@ -650,7 +672,7 @@ __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, u
         l_run = l_run * alpha + sum;
         m_run = m_use;
         tc_fence_before();
-        mbar_arrive(bar(B_PF + x));
+        mbar_arrive(bar(B_PF + x + (int)dbl));
     }
 
     static_assert(!kKpp || D == HD, "the key ping-pong is the 128-channel decode kernel's");
@@ -2167,22 +2189,202 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_decode_kernel(const __gri
     attn_tc_body<false, false, false, true>(KP);
 }
 
+// One query tile a CTA (the solo kernel), in two forms.
+//   Shared, two CTAs an SM.  The pair kernel's two tiles share each K/V tile and alternate on the
+//   tensor core, but its CTA has the SM to itself: its start (barriers, TMEM, the first tiles'
+//   latency) and its end (the last softmax, P.V and the epilogue) are some 9 us of a unit of nine
+//   key tiles' 24, and several short pairs in turn pay for each change of query tiles.  Here the
+//   SM's other CTA works on meanwhile: each has one Q tile, one K and one V tile (two at 64
+//   channels; 96 KB at 128), S and O in 256 columns of tensor memory, and runs the chain S(j),
+//   softmax(j), P.V(j); K of the next tile lands while the softmax runs.
+//   Alone, one CTA an SM, when the query tiles do not outnumber the SMs: two K and V stages, and S
+//   and P double-buffered in 512 columns, so that S(j + 1) is computed while softmax(j) runs and
+//   the softmax alone is the chain.
+// With key-range splits (x = tile * n_split + split) the partials are merged by attn_combine_kernel.
+constexpr int kSoloThreads = 192;          // warp 0 loads, warp 1 MMA and TMEM, warps 2..5 softmax
+template <int D, bool kAlone>
+struct Solo {
+    static constexpr int kStages = kAlone || D == 64 ? 2 : 1;
+    static constexpr uint32_t kCols = kAlone ? 512 : 256, kO = kAlone ? 256 : 128;
+    static constexpr size_t kBytes = 1024 + (1 + 2 * kStages) * (size_t)Geo<D>::kTile + 8 * NBAR + 16;
+    // (alone: too much for a second CTA of any form, whose tensor memory would not suffice)
+    static constexpr size_t kSmem = kAlone && kBytes < 150 * 1024 ? 150 * 1024 : kBytes;
+};
+static_assert(2 * (Solo<HD, false>::kSmem + 1024) <= 228 * 1024 && 2 * (Solo<64, false>::kSmem + 1024) <= 228 * 1024,
+              "two CTAs an SM");
+
+template <bool kSif, int D, bool kAlone>
+__device__ __forceinline__ void attn_solo_body(const TcParams& P) {
+    using L = Solo<D, kAlone>;
+    constexpr int kTile = Geo<D>::kTile, NS = L::kStages;
+    static_assert(NS <= KSTAGES && NS <= VSTAGES, "barrier slots");
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    const uint32_t sQ = smem_u32(smem), sK = sQ + kTile, sV = sK + NS * kTile, sBar = sV + NS * kTile;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + (1 + 2 * NS) * (size_t)kTile + 8 * NBAR);
+    volatile uint32_t* abort = tmem_slot + 1;
+    auto bar = [&](int i) { return sBar + 8u * (uint32_t)i; };
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int hk = blockIdx.y;
+    const int l = blockIdx.z / P.batch;
+    const int bl = blockIdx.z - l * P.batch;
+    const int b = P.b0 + bl;
+    const int s_r = P.req[bl].n_slots + P.req[bl].t0;
+    // the last query tile first: under a causal mask it sees the most keys
+    const int sp = (int)(blockIdx.x % P.n_split);
+    const PairSpan span = tile_span(P, (int)((gridDim.x - 1 - blockIdx.x) / P.n_split), sp, s_r);
+    const int n_kv = span.n_kv;
+    const int qz = l * P.batch_total + b;
+    const int key0 = (int)((int64_t)(P.layer0 + l) * P.rows + P.req[bl].row_base);
+    auto key_row = [&](int j) { return key0 + (kSif ? span_tile(span, j) : span.j_base + j) * BN; };
+
+    if (threadIdx.x == 0) {
+        if (n_kv > 0) {
+            // the first tiles on their way into L2 while the CTA sets up
+#pragma unroll
+            for (int h = 0; h < Geo<D>::kBlocks; ++h) {
+                tma_prefetch_4d(&P.tm_q, 64 * h, hk * P.group, span.t0a, qz);
+                tma_prefetch_3d(&P.tm_k, 64 * h, hk, key_row(0));
+                tma_prefetch_3d(&P.tm_v, 64 * h, hk, key_row(0));
+            }
+        }
+        for (int i : {B_Q, B_SF, B_SF + 1, B_OD, B_OE}) mbar_init(bar(i), 1);
+        for (int st = 0; st < NS; ++st)
+            for (int i : {B_KF, B_KE, B_VF, B_VE}) mbar_init(bar(i + st), 1);
+        for (int i : {B_PF, B_PF + 1}) mbar_init(bar(i), 128);
+        *abort = 0u;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                     "r"(L::kCols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+    // a programmatic dependent launched after this grid (the split merge) may start now
+    if (threadIdx.x == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+
+    if (warp == 0) {
+        if (lane == 0 && n_kv > 0) {
+            // -------------------------------------------------------------- loads
+            // launched as a programmatic dependent: the grid before it (which wrote Q and the newest
+            // key rows) has completed and its writes are visible (returns at once otherwise)
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            mbar_expect_tx(bar(B_Q), kTile);
+            tma_load_4d(sQ, &P.tm_q, 0, hk * P.group, span.t0a, qz, bar(B_Q));
+            if (D == 128) tma_load_4d(sQ + HALF_TILE, &P.tm_q, 64, hk * P.group, span.t0a, qz, bar(B_Q));
+            for (int j = 0; j < n_kv; ++j) {
+                const int row = key_row(j), st = j % NS;
+                const uint32_t ph = (uint32_t)(j / NS - 1) & 1u;
+                if (j >= NS) mbar_wait(bar(B_KE + st), ph, P.err, abort);
+                if (*abort) break;
+                const uint32_t dk = sK + (uint32_t)(st * kTile), dv = sV + (uint32_t)(st * kTile);
+                mbar_expect_tx(bar(B_KF + st), kTile);
+                tma_load_3d(dk, &P.tm_k, 0, hk, row, bar(B_KF + st));
+                if (D == 128) tma_load_3d(dk + HALF_TILE, &P.tm_k, 64, hk, row, bar(B_KF + st));
+                if (j >= NS) mbar_wait(bar(B_VE + st), ph, P.err, abort);
+                if (*abort) break;
+                mbar_expect_tx(bar(B_VF + st), kTile);
+                tma_load_3d(dv, &P.tm_v, 0, hk, row, bar(B_VF + st));
+                if (D == 128) tma_load_3d(dv + HALF_TILE, &P.tm_v, 64, hk, row, bar(B_VF + st));
+            }
+        }
+    } else if (warp == 1) {
+        if (lane == 0 && n_kv > 0) {
+            // -------------------------------------------------------------- MMA issuer
+            constexpr uint32_t idS = idesc_bf16(BM, BN, false);
+            constexpr uint32_t idO = idesc_bf16(BM, D, true);
+            constexpr int kKeyStep = 16 * 128;      // bytes of 16 keys' rows in a 64-channel block
+            constexpr uint64_t kTileDesc = (uint64_t)(kTile >> 4);
+            const uint64_t dQ = sw128_desc(sQ, 16, 1024), dK0 = sw128_desc(sK, 16, 1024);
+            const uint64_t dV0 = sw128_desc(sV, HALF_TILE, 1024);
+            const uint32_t tS = tmem + kColS, tO = tmem + L::kO;
+            auto wait = [&](int i, uint32_t parity) {
+                mbar_wait(bar(i), parity, P.err, abort);
+                tc_fence_after();
+            };
+            auto s_tile = [&](int j) {              // S(j), in its block (alone: of two)
+                const int st = j % NS;
+                const uint64_t dk = dK0 + (uint64_t)st * kTileDesc;
+                const uint32_t d = kAlone ? (uint32_t)j & 1u : 0u;
+                wait(B_KF + st, (uint32_t)(j / NS) & 1u);
+#pragma unroll
+                for (int kk = 0; kk < D / 16; ++kk) {
+                    const uint64_t off = (uint64_t)(((kk >> 2) * HALF_TILE + (kk & 3) * 32) >> 4);
+                    mma_bf16(tS + d * BN, dQ + off, dk + off, idS, kk > 0 ? 1u : 0u);
+                }
+                mma_commit(bar(B_SF + (int)d));
+                mma_commit(bar(B_KE + st));
+            };
+            constexpr int kAhead = kAlone ? 2 : 1;  // S tiles before the first P.V
+            wait(B_Q, 0u);
+            s_tile(0);
+            if (kAlone && n_kv > 1) s_tile(1);
+            for (int j = 0; j < n_kv; ++j) {
+                const int st = j % NS;
+                const uint32_t d = kAlone ? (uint32_t)j & 1u : 0u, tP = tS + d * BN;
+                const uint64_t dv = dV0 + (uint64_t)st * kTileDesc;
+                wait(B_PF + (int)d, (uint32_t)(kAlone ? j >> 1 : j) & 1u);
+                wait(B_VF + st, (uint32_t)(j / NS) & 1u);
+#pragma unroll
+                for (int kk = 0; kk < BN / 16; ++kk)
+                    mma_bf16_ts(tO, tP + (uint32_t)kk * 8u, dv + (uint64_t)((kk * kKeyStep) >> 4), idO,
+                                kk > 0 || j > 0 ? 1u : 0u);
+                if constexpr (Geo<D>::kSplitP) {
+#pragma unroll
+                    for (int kk = 0; kk < BN / 16; ++kk)
+                        mma_bf16_ts(tO, tP + 64u + (uint32_t)kk * 8u, dv + (uint64_t)((kk * kKeyStep) >> 4), idO, 1u);
+                }
+                if (kAlone) mma_commit(bar(B_OE));
+                mma_commit(bar(B_VE + st));
+                // S overwrites the P that this P.V reads after it, in issue order
+                if (j + kAhead < n_kv) s_tile(j + kAhead);
+            }
+            mma_commit(bar(B_OD));
+        }
+    } else {
+        // ------------------------------------------------------------------ softmax, epilogue
+        softmax_tile<false, kSif, false, D, L::kO, kAlone>(P, tmem, sBar, 0, warp & 3, lane, span.t0a, l, bl, b, hk, sp,
+                                                           span, 0u, 0u, false, abort, sQ);
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(L::kCols) : "memory");
+    }
+}
+
+template <bool kSif, int D, bool kAlone>
+__global__ void __launch_bounds__(kSoloThreads, kAlone ? 1 : 2) attn_solo_kernel(const __grid_constant__ TcParams KP) {
+    attn_solo_body<kSif, D, kAlone>(KP);
+}
+
 // The kernel of an instantiation.
-template <bool kFused, bool kMulti, bool kSif, bool kKpp = false, int D = HD>
+// kSolo: 0, or the solo kernel shared (1) or alone (2).
+template <bool kFused, bool kMulti, bool kSif, bool kKpp = false, int D = HD, int kSolo = 0>
 const void* tc_kernel_fn() {
-    if constexpr (D == 64) return reinterpret_cast<const void*>(kSif ? &attn_tc64_sif_kernel : &attn_tc64_kernel);
+    if constexpr (kSolo != 0) return reinterpret_cast<const void*>(&attn_solo_kernel<kSif, D, kSolo == 2>);
+    else if constexpr (D == 64) return reinterpret_cast<const void*>(kSif ? &attn_tc64_sif_kernel : &attn_tc64_kernel);
     else if constexpr (kSif) return reinterpret_cast<const void*>(&attn_tc_sif_kernel);
     else if constexpr (kKpp) return reinterpret_cast<const void*>(&attn_tc_decode_kernel);
     else return reinterpret_cast<const void*>(&attn_tc_kernel<kFused, kMulti>);
 }
 
 // Merge the splits: lse = log2 sum_s 2^lse_s, O = sum_s 2^(lse_s - lse) O_s.  One warp per
-// (layer, request, suffix token, query head) row; lane i owns head channels 4i .. 4i+3.
+// (layer, request, suffix token, query head) row; lane i owns head channels C i .. C i + C - 1.
 // Every split's lse and O slice is loaded before any is used (at most kMaxSplit), so the
 // loads of one row are all in flight together.
 constexpr int kMaxSplit = 16;
 
+template <int D>
 __global__ void __launch_bounds__(256) attn_combine_kernel(const __grid_constant__ AttnParams P) {
+    constexpr int C = D / 32;                       // channels a lane
+
     asm volatile("griddepcontrol.wait;" ::: "memory");   // the partials are complete and visible
     const int64_t rows = (int64_t)P.lq * P.batch_total * P.sq * P.hq;
     const int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -2194,35 +2396,48 @@ __global__ void __launch_bounds__(256) attn_combine_kernel(const __grid_constant
     const int64_t lb = lbt / P.sq;
     const int64_t lse_id = (lb * P.hq + h) * P.sq + t;
     float ls[kMaxSplit];
-    float4 o[kMaxSplit];
+    float o[kMaxSplit][C];
 #pragma unroll
     for (int s = 0; s < kMaxSplit; ++s) {
         ls[s] = -CUDART_INF_F;
-        o[s] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int c = 0; c < C; ++c) o[s][c] = 0.f;
         if (s < P.n_split) {
             ls[s] = P.part_lse[(int64_t)s * rows + lse_id];
-            o[s] = *reinterpret_cast<const float4*>(P.part_o + ((int64_t)s * rows + row) * HD + lane * 4);
+            const float* src = P.part_o + ((int64_t)s * rows + row) * D + lane * C;
+            if constexpr (C == 4) {
+                const float4 v = *reinterpret_cast<const float4*>(src);
+                o[s][0] = v.x;
+                o[s][1] = v.y;
+                o[s][2] = v.z;
+                o[s][3] = v.w;
+            } else {
+                const float2 v = *reinterpret_cast<const float2*>(src);
+                o[s][0] = v.x;
+                o[s][1] = v.y;
+            }
         }
     }
     float mx = -CUDART_INF_F;
 #pragma unroll
     for (int s = 0; s < kMaxSplit; ++s) mx = fmaxf(mx, ls[s]);
     float wsum = 0.f;
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    float acc[C];
+#pragma unroll
+    for (int c = 0; c < C; ++c) acc[c] = 0.f;
 #pragma unroll
     for (int s = 0; s < kMaxSplit; ++s) {
         const float w = ls[s] == -CUDART_INF_F ? 0.f : ex2(ls[s] - mx);
-        acc.x += w * o[s].x;
-        acc.y += w * o[s].y;
-        acc.z += w * o[s].z;
-        acc.w += w * o[s].w;
+#pragma unroll
+        for (int c = 0; c < C; ++c) acc[c] += w * o[s][c];
         wsum += w;
     }
     const float inv = 1.0f / wsum;
-    uint2 pk;
-    pk.x = pack_bf16(acc.x * inv, acc.y * inv);
-    pk.y = pack_bf16(acc.z * inv, acc.w * inv);
-    *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(P.out) + row * HD + lane * 4) = pk;
+    uint32_t* dst = reinterpret_cast<uint32_t*>(static_cast<__nv_bfloat16*>(P.out) + row * D + lane * C);
+    if constexpr (C == 4)
+        *reinterpret_cast<uint2*>(dst) = make_uint2(pack_bf16(acc[0] * inv, acc[1] * inv), pack_bf16(acc[2] * inv, acc[3] * inv));
+    else
+        *dst = pack_bf16(acc[0] * inv, acc[1] * inv);
     if (P.lse != nullptr && lane == 0) P.lse[lse_id] = (mx + log2f(wsum)) * 0.69314718055994531f;
 }
 
@@ -2257,6 +2472,11 @@ bool encode_tensor_map(CUtensorMap* tm, CUtensorMapDataType type, int rank, cons
     return r == CUDA_SUCCESS;
 }
 
+int64_t attn_tc_tiles(int hq, int hkv, int sq, int lq, int batch) {
+    const int tq = BM / (hq / hkv);
+    return (int64_t)((sq + tq - 1) / tq) * hkv * lq * batch;
+}
+
 int64_t attn_tc_units(int hq, int hkv, int sq, int lq, int batch) {
     const int tq = BM / (hq / hkv);
     const int64_t tiles = (sq + tq - 1) / tq;
@@ -2269,22 +2489,21 @@ cudaError_t launch_attn_combine(const AttnParams& a, cudaStream_t s) {
     const int64_t rows = (int64_t)a.lq * a.batch_total * a.sq * a.hq;
     const int64_t blocks = (rows + 7) / 8;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(256);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
     if (a.dependent) {          // its launch overlaps the attention's last CTAs
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3((unsigned)blocks);
-        cfg.blockDim = dim3(256);
-        cfg.stream = s;
-        cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        const cudaError_t e = cudaLaunchKernelEx(&cfg, attn_combine_kernel, a);
-        if (e != cudaSuccess) return e;
-    } else {
-        attn_combine_kernel<<<(unsigned)blocks, 256, 0, s>>>(a);
     }
-    return cudaGetLastError();
+    void* args[1] = {const_cast<AttnParams*>(&a)};
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, a.d == 64 ? reinterpret_cast<const void*>(&attn_combine_kernel<64>)
+                                                              : reinterpret_cast<const void*>(&attn_combine_kernel<HD>), args);
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 bool attn_tc_supported(int dtype, int d, int hq, int hkv) {
@@ -2301,19 +2520,19 @@ namespace {
 
 // Host-side preparation shared by the plain and the fused launch: function attributes once
 // per process, the register-split guard, the tensor maps and the scalar parameters.
-template <bool kFused, bool kMulti = false, bool kSif = false, bool kKpp = false, int D = HD>
+template <bool kFused, bool kMulti = false, bool kSif = false, bool kKpp = false, int D = HD, int kSolo = 0>
 cudaError_t prepare_tc(const AttnParams& a, TcParams& p, dim3& grid) {
     constexpr int threads = kFused ? kThreadsFused : kThreads;
     constexpr int high = kFused ? kRegsHighFused : kRegsHigh;
     constexpr int low_total = kFused ? 128 * (kRegsLowFused + kRegsLoadFused) : 128 * kRegsLow;
     // once per process (one device per context; function-local statics: thread-safe)
     static const cudaError_t smem_err = cudaFuncSetAttribute(
-        tc_kernel_fn<kFused, kMulti, kSif, kKpp, D>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Geo<D>::kSmem);
+        tc_kernel_fn<kFused, kMulti, kSif, kKpp, D, kSolo>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSolo ? Solo<D, kSolo == 2>::kSmem : Geo<D>::kSmem));
     if (smem_err != cudaSuccess) return smem_err;
-    {   // the register split must not ask for more than the launch holds
+    if constexpr (!kSolo) {   // the register split must not ask for more than the launch holds
         static const int launch_regs = []() {
             cudaFuncAttributes fa{};
-            return cudaFuncGetAttributes(&fa, tc_kernel_fn<kFused, kMulti, kSif, kKpp, D>()) == cudaSuccess ? fa.numRegs : -1;
+            return cudaFuncGetAttributes(&fa, tc_kernel_fn<kFused, kMulti, kSif, kKpp, D, kSolo>()) == cudaSuccess ? fa.numRegs : -1;
         }();
         if (launch_regs < 0) return cudaErrorInvalidDeviceFunction;
         if (launch_regs * threads < low_total + 256 * high) return cudaErrorInvalidConfiguration;
@@ -2373,7 +2592,9 @@ cudaError_t prepare_tc(const AttnParams& a, TcParams& p, dim3& grid) {
     // from HBM, the epilogue) is then paid once for several short pairs (causal extraction
     // rows: 1 to 4 key tiles a pair).  The context's attn_pairs setting caps the choice.
     int64_t pg = 1;
-    if (kMulti) {                // every pair of a (layer, request, KV head) in one CTA
+    if (kSolo) {
+        if (p.n_split > 1 && (p.tickets || kSif)) return cudaErrorInvalidValue;
+    } else if (kMulti) {         // every pair of a (layer, request, KV head) in one CTA
         if (p.n_split != 1) return cudaErrorInvalidValue;
         pg = pairs;
     } else if (!kFused && p.n_split == 1) {
@@ -2390,7 +2611,7 @@ cudaError_t prepare_tc(const AttnParams& a, TcParams& p, dim3& grid) {
     }
     p.pairs = (int32_t)pairs;
     p.pair_group = (int32_t)pg;
-    const int64_t gx = (pairs + pg - 1) / pg * p.n_split;
+    const int64_t gx = kSolo ? (int64_t)((a.sq + tq - 1) / tq) * p.n_split : (pairs + pg - 1) / pg * p.n_split;
     if (gx > 0x7fffffffLL) return cudaErrorInvalidValue;
     grid = dim3((unsigned)gx, a.hkv, a.lq * a.batch);
     if (grid.z > 65535u || grid.y > 65535u) return cudaErrorInvalidValue;
@@ -2401,22 +2622,29 @@ cudaError_t prepare_tc(const AttnParams& a, TcParams& p, dim3& grid) {
 
 cudaError_t preload_attn_tc_kernels(int d) {
     cudaFuncAttributes fa{};
-    return d == 64 ? cudaFuncGetAttributes(&fa, attn_tc64_kernel) : cudaFuncGetAttributes(&fa, attn_tc_kernel<false>);
+    cudaError_t e = d == 64 ? cudaFuncGetAttributes(&fa, attn_tc64_kernel) : cudaFuncGetAttributes(&fa, attn_tc_kernel<false>);
+    if (e == cudaSuccess)
+        e = d == 64 ? cudaFuncGetAttributes(&fa, attn_solo_kernel<false, 64, false>)
+                    : cudaFuncGetAttributes(&fa, attn_solo_kernel<false, HD, false>);
+    if (e == cudaSuccess)
+        e = d == 64 ? cudaFuncGetAttributes(&fa, attn_solo_kernel<false, 64, true>)
+                    : cudaFuncGetAttributes(&fa, attn_solo_kernel<false, HD, true>);
+    return e;
 }
 
 namespace {
 
-template <bool kSif, bool kKpp, int D>
+template <bool kSif, bool kKpp, int D, int kSolo = 0>
 cudaError_t launch_plain(const AttnParams& a, cudaStream_t s, Hook before) {
     TcParams p;
     dim3 grid;
-    cudaError_t e = prepare_tc<false, false, kSif, kKpp, D>(a, p, grid);
+    cudaError_t e = prepare_tc<false, false, kSif, kKpp, D, kSolo>(a, p, grid);
     if (e != cudaSuccess) return e;
     before();
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = Geo<D>::kSmem;
+    cfg.blockDim = dim3(kSolo ? kSoloThreads : kThreads);
+    cfg.dynamicSmemBytes = kSolo ? Solo<D, kSolo == 2>::kSmem : Geo<D>::kSmem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     if (a.dependent) {          // starts while the kernel before it runs (the producer waits)
@@ -2426,22 +2654,55 @@ cudaError_t launch_plain(const AttnParams& a, cudaStream_t s, Hook before) {
         cfg.numAttrs = 1;
     }
     void* args[1] = {&p};
-    e = cudaLaunchKernelExC(&cfg, tc_kernel_fn<false, false, kSif, kKpp, D>(), args);
+    e = cudaLaunchKernelExC(&cfg, tc_kernel_fn<false, false, kSif, kKpp, D, kSolo>(), args);
     return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+// Which kernel attends.  Measured pair against solo (us a call, GB300): extraction solo by 15 to
+// 60 % from 512 to 4096 tokens; suffixes of 64 and 200 tokens over 5 to 17 key tiles solo by 2 to
+// 24 % while the pairs are at most half the SMs, or a (layer, request, KV head) has a single query
+// tile, or few key tiles (256 pairs of 3: 38 / 36, of 5: 44 / 42), and the pair kernel by 2 to 7 %
+// (and 13 % over 257 key tiles) when 77 pairs or more share their K/V tiles.
+enum class SoloChoice { kPair, kShared, kAlone };
+SoloChoice solo_choice(const AttnParams& a) {
+    if (a.key_pingpong || a.pairs_per_cta != 0 || a.tickets != nullptr) return SoloChoice::kPair;
+    static const int sms = []() {
+        int dev = 0, n = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1)
+            return 1;
+        return n;
+    }();
+    const int tq = BM / (a.hq / a.hkv);
+    const int64_t per_head = (a.sq + tq - 1) / tq, heads = (int64_t)a.hkv * a.lq * a.batch;
+    const int64_t units = per_head * heads * std::max(1, a.n_split);
+    if (units <= sms && a.sif_k == 0) return SoloChoice::kAlone;
+    if (a.n_split > 1 || a.sif_k > 0 || per_head == 1) return SoloChoice::kShared;
+    int slots = 0;
+    for (int i = 0; i < a.batch; ++i) slots = std::max(slots, a.req[i].n_slots);
+    const int tiles = (slots + a.sq + BN - 1) / BN;
+    const bool causal_only = slots == 0;             // extraction document rows
+    if (causal_only || tiles <= 6 || 2 * ((per_head + 1) / 2 * heads) <= sms) return SoloChoice::kShared;
+    return SoloChoice::kPair;
+}
+template <bool kSif, int D>
+cudaError_t launch_form(SoloChoice c, const AttnParams& a, cudaStream_t s, Hook before) {
+    if constexpr (!kSif)
+        if (c == SoloChoice::kAlone) return launch_plain<false, false, D, 2>(a, s, before);
+    if (c == SoloChoice::kShared) return launch_plain<kSif, false, D, 1>(a, s, before);
+    return launch_plain<kSif, false, D>(a, s, before);
 }
 
 }  // namespace
 
 cudaError_t launch_attn_tc(const AttnParams& a, cudaStream_t s, Hook before) {
     (void)cudaGetLastError();   // report this launch's error only, not a stale one
-    if (a.d == 64) {
-        if (a.key_pingpong) return cudaErrorInvalidValue;
-        return a.sif_k > 0 ? launch_plain<true, false, 64>(a, s, before) : launch_plain<false, false, 64>(a, s, before);
-    }
-    if (a.d != HD) return cudaErrorInvalidValue;
-    // extraction C2 rows and decode steps: their own instantiations
-    if (a.sif_k > 0) return launch_plain<true, false, HD>(a, s, before);
-    return a.key_pingpong ? launch_plain<false, true, HD>(a, s, before) : launch_plain<false, false, HD>(a, s, before);
+    if (a.d != HD && (a.d != 64 || a.key_pingpong)) return cudaErrorInvalidValue;
+    const SoloChoice solo = solo_choice(a);
+    if (a.d == 64)
+        return a.sif_k > 0 ? launch_form<true, 64>(solo, a, s, before) : launch_form<false, 64>(solo, a, s, before);
+    if (a.key_pingpong) return launch_plain<false, true, HD>(a, s, before);    // decode steps
+    return a.sif_k > 0 ? launch_form<true, HD>(solo, a, s, before) : launch_form<false, HD>(solo, a, s, before);
 }
 
 namespace {

@@ -774,6 +774,42 @@ cudaError_t suffix_run(c2kv_ctx* c, const c2kv_cache* cache, int32_t layer0, int
     return e;
 }
 
+// Key-range splits of an attend launch on the tensor cores (`merge_launch`: partials merged by a
+// launch of their own rather than in the kernel).  When the query tiles leave SMs idle, each one's
+// key tiles may be split, as far as the SMs go, by a model of the call (us): a key tile takes about
+// 1, a CTA 8 to start and end, the merge launch 5 and its partials' bytes both ways at 5 TB/s.
+// (The merge in the kernel, by the last CTA of a unit alone, costs about 0.25 a row: with 256 rows a
+// unit it had made 2 requests x 200 tokens over 16 chunks 103 us a call, now 29.)  Measured, one
+// layer, 32 / 8 heads: 64 tokens over 10 chunks 28.9 -> 16 us, over 64 chunks 43 -> 24.
+int32_t attn_splits(const c2kv_ctx* c, const c2kv_cache* cache, int32_t lq, int32_t n_suffix, bool fused,
+                    bool* merge_launch) {
+    *merge_launch = fused;
+    if (c->cfg.attn_split >= 1) return c->cfg.attn_split;
+    int32_t tiles = 1;
+    for (int32_t b = 0; b < cache->batch; ++b)
+        tiles = std::max<int32_t>(tiles, (cache->n_slots[b] + n_suffix + 127) / 128);
+    if (fused) {
+        const int64_t units = c2kv::attn_tc_units(c->cfg.n_q_heads, c->cfg.n_kv_heads, n_suffix, lq, cache->batch);
+        if (2 * units > c->sms) return 1;
+        // at most half of the SMs would have work: split toward one wave, keeping at least
+        // 8 key tiles per split (below that the merge costs more than it saves)
+        return std::max<int32_t>(1, std::min<int32_t>((int32_t)std::min<int64_t>(16, c->sms / units), tiles / 8));
+    }
+    const int64_t units = c2kv::attn_tc_tiles(c->cfg.n_q_heads, c->cfg.n_kv_heads, n_suffix, lq, cache->batch);
+    const double rows = (double)lq * cache->batch * n_suffix * c->cfg.n_q_heads;
+    int32_t best = 1;
+    double cost = tiles * 1.0 + 8.0;
+    for (int32_t n = 2; n <= 16 && n * units <= c->sms && n <= tiles; ++n) {
+        const double t = (tiles + n - 1) / n * 1.0 + 8.0 + 5.0 + n * rows * (c->cfg.head_dim + 1) * 8.0 / 5.0e6;
+        if (t < 0.95 * cost) {
+            cost = t;
+            best = n;
+        }
+    }
+    *merge_launch = best > 1;
+    return best;
+}
+
 // Suffix preparation and attention of a cache (arguments already checked).  With `fused`,
 // the cache is not written yet: the fused kernel reads the composed slots from the pool and
 // the suffix from k_suf / v_suf, turns the queries itself, and writes the whole cache
@@ -796,32 +832,19 @@ cudaError_t attend_run(c2kv_ctx* c, c2kv_cache* cache, int32_t layer0, int32_t l
     cudaError_t e = fused || q_rot_ready ? cudaSuccess : pool_alloc(c, &q_rot, q_bytes);
     if (e != cudaSuccess) return e;
     void* const q_rot_own = q_rot_ready ? nullptr : q_rot;    // freed here
-    // Key-range split of the tensor-core attention: when its work units would leave most
-    // SMs idle (a single layer of a small batch), each unit's key tiles are split and the
-    // partials merged; at a wave or more the split only adds the merge.
     int32_t n_split = 1;
+    bool merge_launch = false;
     float* part = nullptr;
     if (use_tc) {
-        const int64_t units = c2kv::attn_tc_units(c->cfg.n_q_heads, c->cfg.n_kv_heads, n_suffix, lq, B);
-        int32_t n_kv_max = 1;
-        for (int32_t b = 0; b < B; ++b)
-            n_kv_max = std::max<int32_t>(n_kv_max, (cache->n_slots[b] + n_suffix + 127) / 128);
-        if (fused && fused->pairs_in_turn) {
-            n_split = 1;             // one CTA runs every pair of its (layer, request, KV head)
-        } else if (c->cfg.attn_split >= 1) {
-            n_split = c->cfg.attn_split;
-        } else if (2 * units <= c->sms) {
-            // at most half of the SMs would have work: split toward one wave, keeping at
-            // least 8 key tiles per split (below that the merge costs more than it saves)
-            n_split = (int32_t)std::min<int64_t>(16, c->sms / units);
-            n_split = std::max<int32_t>(1, std::min<int32_t>(n_split, n_kv_max / 8));
-        }
+        // (a fused CTA that runs every pair of its (layer, request, KV head) takes no split)
+        if (!(fused && fused->pairs_in_turn))
+            n_split = attn_splits(c, cache, lq, n_suffix, fused != nullptr, &merge_launch);
         if (n_split > 1) {
             const size_t rows = (size_t)lq * B * n_suffix * c->cfg.n_q_heads;
             e = pool_alloc(c, reinterpret_cast<void**>(&part),
                            (size_t)n_split * rows * (c->cfg.head_dim + 1) * sizeof(float));
-            // the plain kernel merges the splits itself (per-unit counters)
-            if (e == cudaSuccess && !fused && n_split <= c2kv::kMaxMergeSplits)
+            // the pair kernel merges the splits itself (per-unit counters)
+            if (e == cudaSuccess && !merge_launch && n_split <= c2kv::kMaxMergeSplits)
                 e = tickets_ready(c, (size_t)c2kv::attn_tc_units(c->cfg.n_q_heads, c->cfg.n_kv_heads, n_suffix,
                                                                  lq, std::min<int32_t>(B, c2kv::kMaxReq)));
             if (e != cudaSuccess) {
@@ -831,7 +854,7 @@ cudaError_t attend_run(c2kv_ctx* c, c2kv_cache* cache, int32_t layer0, int32_t l
             }
         }
     }
-    const bool merge_in_kernel = use_tc && !fused && n_split > 1 && n_split <= c2kv::kMaxMergeSplits;
+    const bool merge_in_kernel = use_tc && !merge_launch && n_split > 1 && n_split <= c2kv::kMaxMergeSplits;
     const size_t part_rows = (size_t)lq * B * n_suffix * c->cfg.n_q_heads;
     c2kv::AttnParams last{};
     for (int32_t b0 = 0; e == cudaSuccess && b0 < B; b0 += c2kv::kMaxReq) {

@@ -261,7 +261,9 @@ bool attn_tc_takes(int dtype, int d, int hq, int hkv);
 cudaError_t launch_attn_tc(const AttnParams& p, cudaStream_t s, Hook before = {});
 // Merge n_split partial (O, lse) over disjoint key ranges into out (bf16) and lse (attn_tc.cu).
 cudaError_t launch_attn_combine(const AttnParams& p, cudaStream_t s);
-// CTAs of one tensor-core attention launch before key-range splitting.
+// Query tiles of one tensor-core attention launch, and pairs of them (the pair kernel's CTAs),
+// before key-range splitting.
+int64_t attn_tc_tiles(int hq, int hkv, int sq, int lq, int batch);
 int64_t attn_tc_units(int hq, int hkv, int sq, int lq, int batch);
 
 // Fused compose + attention (attn_tc.cu): the attention reads the composed slots straight
