@@ -163,6 +163,7 @@ struct TcParams {                // CUtensorMap members carry their own alignmen
     float* part_lse;
     uint32_t* tickets;       // null, or per-unit counters: the last split merges (plain kernel)
     int32_t sif_k;           // 0, or extraction C2 rows with ratio k (plain kernel, one split)
+    const float2* q_cs;      // null, or (solo kernel) the queries are before RoPE: AttnParams::q_cs
     ReqParam req[kMaxReq];
 };
 
@@ -2213,6 +2214,63 @@ struct Solo {
 static_assert(2 * (Solo<HD, false>::kSmem + 1024) <= 228 * 1024 && 2 * (Solo<64, false>::kSmem + 1024) <= 228 * 1024,
               "two CTAs an SM");
 
+// The queries of a solo CTA turned in shared memory (TcParams::q_cs): the softmax warps (ts =
+// 0..127), which have nothing else to do until the first S, take item (token, chunk pair q = ts %
+// NQ): its 8 frequencies' (cos, sin) from the table, fetched while Q lands, then chunk pair q of the
+// token's G query rows (the rope kernel's rounding).  Then the MMA issuer is told (B_QR).
+template <int D>
+__device__ __forceinline__ void solo_turn_queries(const TcParams& P, int ts, const PairSpan& span, uint32_t sQ,
+                                                  uint32_t sBar, volatile uint32_t* abort) {
+    constexpr int NQ = D / 16, STEP = 128 / NQ;   // chunk pairs a row (8 channels each half); tokens a pass
+    const int G = P.group, q = ts % NQ;
+    auto angles = [&](int tt, float2 (&cc)[4], float2 (&ss)[4]) {
+        const float4* t = reinterpret_cast<const float4*>(P.q_cs + (int64_t)tt * (D / 2) + 8 * q);
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+            const float4 v = __ldg(t + w);
+            cc[w] = make_float2(v.x, v.z);
+            ss[w] = make_float2(v.y, v.w);
+        }
+    };
+    auto turn = [&](int tt, const float2 (&cc)[4], const float2 (&ss)[4]) {
+#pragma unroll 2
+        for (int g = 0; g < G; ++g) {
+            const int r = (tt - span.t0a) * G + g;
+            // channels 8 q .. of a 64-channel block and their partners, in the other block (128
+            // channels) or four chunks on (64)
+            const uint32_t a0 = sQ + sw_off(r, q);
+            const uint32_t a1 = D == 128 ? a0 + HALF_TILE : sQ + sw_off(r, q + 4);
+            const uint4 xv = lds128(a0), yv = lds128(a1);
+            const uint32_t xw[4] = {xv.x, xv.y, xv.z, xv.w}, yw[4] = {yv.x, yv.y, yv.z, yv.w};
+            uint32_t xo[4], yo[4];
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+                float2 gx, gy;
+                rotate2(bf2_to_f2(xw[w]), bf2_to_f2(yw[w]), cc[w], ss[w], gx, gy);
+                xo[w] = f2_to_bf2(gx.x, gx.y);
+                yo[w] = f2_to_bf2(gy.x, gy.y);
+            }
+            sts128(a0, make_uint4(xo[0], xo[1], xo[2], xo[3]));
+            sts128(a1, make_uint4(yo[0], yo[1], yo[2], yo[3]));
+        }
+    };
+    // two tokens' angles in flight together
+    const int tt0 = span.t0a + ts / NQ;
+    float2 c0[4], s0[4], c1[4], s1[4];
+    if (tt0 <= span.t_last) angles(tt0, c0, s0);
+    if (tt0 + STEP <= span.t_last) angles(tt0 + STEP, c1, s1);
+    mbar_wait(sBar + 8u * B_Q, 0u, P.err, abort);
+    if (tt0 <= span.t_last) turn(tt0, c0, s0);
+    if (tt0 + STEP <= span.t_last) turn(tt0 + STEP, c1, s1);
+#pragma unroll 1
+    for (int tt = tt0 + 2 * STEP; tt <= span.t_last; tt += STEP) {
+        angles(tt, c0, s0);
+        turn(tt, c0, s0);
+    }
+    fence_proxy_async();
+    mbar_arrive(sBar + 8u * B_QR);
+}
+
 template <bool kSif, int D, bool kAlone>
 __device__ __forceinline__ void attn_solo_body(const TcParams& P) {
     using L = Solo<D, kAlone>;
@@ -2251,7 +2309,7 @@ __device__ __forceinline__ void attn_solo_body(const TcParams& P) {
         for (int i : {B_Q, B_SF, B_SF + 1, B_OD, B_OE}) mbar_init(bar(i), 1);
         for (int st = 0; st < NS; ++st)
             for (int i : {B_KF, B_KE, B_VF, B_VE}) mbar_init(bar(i + st), 1);
-        for (int i : {B_PF, B_PF + 1}) mbar_init(bar(i), 128);
+        for (int i : {B_PF, B_PF + 1, B_QR}) mbar_init(bar(i), 128);
         *abort = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -2321,7 +2379,7 @@ __device__ __forceinline__ void attn_solo_body(const TcParams& P) {
                 mma_commit(bar(B_KE + st));
             };
             constexpr int kAhead = kAlone ? 2 : 1;  // S tiles before the first P.V
-            wait(B_Q, 0u);
+            wait(P.q_cs != nullptr ? B_QR : B_Q, 0u);
             s_tile(0);
             if (kAlone && n_kv > 1) s_tile(1);
             for (int j = 0; j < n_kv; ++j) {
@@ -2348,6 +2406,7 @@ __device__ __forceinline__ void attn_solo_body(const TcParams& P) {
         }
     } else {
         // ------------------------------------------------------------------ softmax, epilogue
+        if (P.q_cs != nullptr && n_kv > 0) solo_turn_queries<D>(P, (int)threadIdx.x - 64, span, sQ, sBar, abort);
         softmax_tile<false, kSif, false, D, L::kO, kAlone>(P, tmem, sBar, 0, warp & 3, lane, span.t0a, l, bl, b, hk, sp,
                                                            span, 0u, 0u, false, abort, sQ);
     }
@@ -2581,6 +2640,8 @@ cudaError_t prepare_tc(const AttnParams& a, TcParams& p, dim3& grid) {
     p.part_lse = a.part_lse;
     p.tickets = kFused || p.n_split == 1 || p.n_split > kMaxMergeSplits ? nullptr : a.tickets;
     p.sif_k = a.sif_k;
+    p.q_cs = a.q_cs;
+    if (a.q_cs != nullptr && !kSolo) return cudaErrorInvalidValue;
 
     if (kSif != (a.sif_k > 0) || a.sif_k < 0 || (kSif && (kFused || p.n_split != 1))) return cudaErrorInvalidValue;
     if (kKpp != (a.key_pingpong != 0) || (kKpp && (kFused || kSif))) return cudaErrorInvalidValue;

@@ -1527,7 +1527,11 @@ c2kv_status c2kv_extract_attention(c2kv_ctx* c, int32_t n_layers, const void* q,
         if ((int64_t)n_tokens + m > 0x7fffffffLL / 128) return fail(c, C2KV_ERR_ARG, "extract: chunk too long");
         const int32_t n_all = (int32_t)(n_tokens + m);
         const int32_t hq = c->cfg.n_q_heads, hkv = c->cfg.n_kv_heads;
-        const size_t qb = (size_t)n_layers * n_all * hq * d * c->eb;
+        // the turned queries, or the angles from which the attention turns them
+        const bool turn_q = c2kv::extract_uses_tc(c->cfg.dtype, d, hq, hkv) &&
+                            c2kv::extract_turns_queries(c->cfg.attn_pairs);
+        const size_t qb = turn_q ? (size_t)n_all * (d / 2) * sizeof(float2)
+                                 : (size_t)n_layers * n_all * hq * d * c->eb;
         const size_t kb = (size_t)n_layers * n_all * hkv * d * c->eb;
         void* q_rot = nullptr;
         void* k_rot = nullptr;
@@ -1543,7 +1547,8 @@ c2kv_status c2kv_extract_attention(c2kv_ctx* c, int32_t n_layers, const void* q,
         p.q = q;
         p.k = k;
         p.v = v;
-        p.q_rot = q_rot;
+        p.q_rot = turn_q ? nullptr : q_rot;
+        p.q_cs = turn_q ? static_cast<float2*>(q_rot) : nullptr;
         p.k_rot = k_rot;
         p.out = out;
         p.lse = lse;

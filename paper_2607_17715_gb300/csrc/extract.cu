@@ -12,8 +12,8 @@
 // it is read as the first block, [0, min(k, n)).
 //
 // extract_rope_kernel turns Q and K to those positions (fp32 arithmetic, stored in the
-// context dtype like every cached activation).  The masked attention then takes one of two
-// routes.
+// context dtype like every cached activation), or extract_rope_k_kernel K alone where the attention
+// turns the queries itself.  The masked attention then takes one of two routes.
 //
 // Tensor cores (bf16, the group sizes attn_tc_kernel takes).  The mask splits into
 // pieces the suffix-attention kernel already computes:
@@ -75,6 +75,52 @@ __global__ void __launch_bounds__(256) extract_rope_kernel(const __grid_constant
         T* dst = static_cast<T*>(is_q ? P.q_rot : P.k_rot) + off;
         st16(dst, V::pack(gx));
         st16(dst + HALF, V::pack(gy));
+    }
+}
+
+// K alone, and the table of every token's (cos, sin) from which the solo attention kernel turns its
+// query tiles in shared memory.  Turning Q here read and wrote four fifths of the tensors' bytes
+// (Q is Hq / Hkv times K): 68 us of the 32-layer call on 512 + 128 tokens, against 49 us for those
+// bytes at the rate of HBM; the call went from 226 to 200 us.  A CTA takes kRopeTokens tokens of one layer, each thread one (token, head,
+// vector pair) at a time, its loads issued before the angles are formed.
+constexpr int kRopeTokens = 4;
+template <typename T, int VPH>
+__global__ void __launch_bounds__(256) extract_rope_k_kernel(const __grid_constant__ ExtractParams P) {
+    using V = Vec16<T>;
+    constexpr int E = V::N, HALF = VPH * E, D = 2 * HALF;
+    __shared__ float2 cs[kRopeTokens * HALF];
+    const int t0 = blockIdx.x * kRopeTokens, l = blockIdx.y;
+    const int nt = min(kRopeTokens, P.n_all - t0);
+    const int items = nt * P.hkv * VPH;
+    const int64_t base = ((int64_t)l * P.n_all + t0) * P.hkv * D;      // the tokens' rows are contiguous
+    const T* src = static_cast<const T*>(P.k) + base;
+    T* dst = static_cast<T*>(P.k_rot) + base;
+    auto offset = [&](int p) { return (int64_t)(p / VPH) * D + (p % VPH) * E; };
+    uint4 a{}, b{};
+    int p = threadIdx.x;
+    if (p < items) {
+        a = ld16(src + offset(p));
+        b = ld16(src + offset(p) + HALF);
+    }
+    for (int e = threadIdx.x; e < nt * HALF; e += blockDim.x) {
+        const int t = t0 + e / HALF;
+        const float2 v = turn_cs(P.rope.turn[e % HALF], extract_pos(t, P.n, P.ratio));
+        cs[e] = v;
+        if (l == 0) P.q_cs[(int64_t)t0 * HALF + e] = v;
+    }
+    __syncthreads();
+    while (p < items) {
+        float x[E], y[E], gx[E], gy[E];
+        V::unpack(a, x);
+        V::unpack(b, y);
+        rotate<E>(x, y, cs + p / (P.hkv * VPH) * HALF + p % VPH * E, gx, gy);
+        st16(dst + offset(p), V::pack(gx));
+        st16(dst + offset(p) + HALF, V::pack(gy));
+        p += blockDim.x;
+        if (p < items) {
+            a = ld16(src + offset(p));
+            b = ld16(src + offset(p) + HALF);
+        }
     }
 }
 
@@ -146,8 +192,13 @@ __global__ void __launch_bounds__(kCoreThreads, core_ctas(D, RT)) extract_attn_k
 template <int D>
 cudaError_t launch_tc(const ExtractParams& p, cudaStream_t s, cudaStream_t s2, cudaEvent_t fork,
                       cudaEvent_t join) {
-    extract_rope_kernel<__nv_bfloat16, D / 2 / Vec16<__nv_bfloat16>::N>
-        <<<dim3((unsigned)p.n_all, (unsigned)p.lq), 256, 0, s>>>(p);
+    constexpr int VPH = D / 2 / Vec16<__nv_bfloat16>::N;
+    const bool turn_q = p.q_rot == nullptr;
+    if (turn_q)
+        extract_rope_k_kernel<__nv_bfloat16, VPH>
+            <<<dim3((unsigned)((p.n_all + kRopeTokens - 1) / kRopeTokens), (unsigned)p.lq), 256, 0, s>>>(p);
+    else
+        extract_rope_kernel<__nv_bfloat16, VPH><<<dim3((unsigned)p.n_all, (unsigned)p.lq), 256, 0, s>>>(p);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int m = p.n_all - p.n;
@@ -178,7 +229,9 @@ cudaError_t launch_tc(const ExtractParams& p, cudaStream_t s, cudaStream_t s2, c
         sc = s2;
     }
     // 1. document rows over document keys 0..t
-    a.q_rot = p.q_rot;
+    const void* const q = turn_q ? p.q : p.q_rot;
+    a.q_rot = q;
+    a.q_cs = turn_q ? p.q_cs : nullptr;
     a.out = p.out;
     a.lse = p.lse;
     a.sq = p.n;
@@ -189,7 +242,8 @@ cudaError_t launch_tc(const ExtractParams& p, cudaStream_t s, cudaStream_t s2, c
     // that c_j sees c_0 .. c_j causally; the kernel's SIF mode keeps, of the document keys,
     // the sink block and B(j), and visits only their key tiles
     const int64_t c2_off = (int64_t)p.n * p.hq * D;
-    a.q_rot = static_cast<const __nv_bfloat16*>(p.q_rot) + c2_off;
+    a.q_rot = static_cast<const __nv_bfloat16*>(q) + c2_off;
+    a.q_cs = turn_q ? p.q_cs + (int64_t)p.n * (D / 2) : nullptr;
     a.out = static_cast<__nv_bfloat16*>(p.out) + c2_off;
     a.lse = p.lse != nullptr ? p.lse + p.n : nullptr;
     a.sq = m;
@@ -252,11 +306,16 @@ cudaError_t launch_typed(const ExtractParams& p, cudaStream_t s) {
 
 bool extract_uses_tc(int dtype, int d, int hq, int hkv) { return attn_tc_takes(dtype, d, hq, hkv); }
 
+// (the context's attn_pairs asks for the pair kernel, which takes turned queries)
+bool extract_turns_queries(int pairs_per_cta) { return pairs_per_cta == 0; }
+
 cudaError_t launch_extract(const ExtractParams& p, int dtype, int d, cudaStream_t s, cudaStream_t s2,
                            cudaEvent_t fork, cudaEvent_t join) {
     (void)cudaGetLastError();   // report this launch's error only, not a stale one
     if (p.n_all < 1 || p.lq < 1) return cudaSuccess;
     if (p.lq > 65535 || p.hkv > 65535) return cudaErrorInvalidValue;
+    if (!p.q_rot != (extract_uses_tc(dtype, d, p.hq, p.hkv) && extract_turns_queries(p.pairs_per_cta)))
+        return cudaErrorInvalidValue;
     if (extract_uses_tc(dtype, d, p.hq, p.hkv))
         return d == 64 ? launch_tc<64>(p, s, s2, fork, join) : launch_tc<128>(p, s, s2, fork, join);
     if (dtype == kDtypeF32 && d == 64) return launch_typed<float, 64>(p, s);

@@ -164,6 +164,9 @@ struct AttnParams {
                              // document tokens, suffix token j is C2 token c_j, and of the
                              // document keys row j sees only the sink block [0, min(k, n)) and
                              // its own block [jk, min((j+1)k, n)); n_split must be 1
+    const float2* q_cs;      // tensor-core solo kernel: null, or q_rot holds the queries before
+                             // RoPE and token t turns by row t of this table [sq][d / 2] of (cos,
+                             // sin) (the same for every request of the launch)
     ReqParam req[kMaxReq];
 };
 
@@ -224,7 +227,8 @@ struct ExtractParams {
     const void* q;           // [Lq][n_all][Hq][d] pre-RoPE
     const void* k;           // [Lq][n_all][Hkv][d] pre-RoPE
     const void* v;           // [Lq][n_all][Hkv][d]
-    void* q_rot;             // scratch, shaped like q
+    void* q_rot;             // scratch, shaped like q; null: the attention turns the queries
+    float2* q_cs;            // q_rot null: scratch [n_all][d / 2], (cos, sin) at each token's position
     void* k_rot;             // scratch, shaped like k
     void* out;               // [Lq][n_all][Hq][d]
     float* lse;              // [Lq][Hq][n_all] or null
@@ -246,6 +250,8 @@ cudaError_t launch_extract(const ExtractParams& p, int dtype, int d, cudaStream_
 // Whether launch_extract takes the tensor-core route; otherwise every row runs on the CUDA
 // cores.
 bool extract_uses_tc(int dtype, int d, int hq, int hkv);
+// Whether the tensor-core route turns the queries in the attention (q_rot null, q_cs given).
+bool extract_turns_queries(int pairs_per_cta);
 
 // Tiled tensor map for TMA (cuTensorMapEncodeTiled through the runtime's driver entry point);
 // false when the driver refuses it (attn_tc.cu).
