@@ -7,6 +7,7 @@ fallback: if the compiled library is missing, importing this module fails.
 """
 from __future__ import annotations
 
+import array
 import ctypes
 import os
 
@@ -126,8 +127,19 @@ def _ptr(x):
 
 
 def _i32(arr):
+    """The values as int32 memory that the first result keeps, and its pointer."""
     if arr is None:
         return None, None
+    if type(arr) in (list, tuple) and arr:
+        # a short list costs numpy some 3 us, an int array 0.5; it refuses what does not fit too.
+        # Anything but integers (floats, nested lists) is numpy's to convert
+        try:
+            a = array.array("i", arr)
+        except TypeError:
+            pass
+        else:
+            p = (ctypes.c_int32 * len(a)).from_buffer(a)
+            return p, p
     a = np.ascontiguousarray(np.asarray(arr, dtype=np.int32))
     return a, a.ctypes.data_as(_P32)
 
@@ -214,11 +226,10 @@ def c2kv_cache_info(cache) -> dict:
     d = c2kv_cache_desc()
     _check(_lib.c2kv_cache_info(cache, ctypes.byref(d)))
     b = d.batch
-    return dict(batch=b, layers=d.layers, rows=d.rows, k=d.k, v=d.v, pos=d.pos,
-                row_base=np.ctypeslib.as_array(d.row_base, (b,)).copy(),
-                n_slots=np.ctypeslib.as_array(d.n_slots, (b,)).copy(),
-                l_req=np.ctypeslib.as_array(d.l_req, (b,)).copy(),
-                capacity=np.ctypeslib.as_array(d.capacity, (b,)).copy(),
+    i32_b = ctypes.c_int32 * b
+    host = {f: np.frombuffer(i32_b.from_address(ctypes.addressof(getattr(d, f).contents)), np.int32).copy()
+            for f in ("row_base", "n_slots", "l_req", "capacity")}
+    return dict(batch=b, layers=d.layers, rows=d.rows, k=d.k, v=d.v, pos=d.pos, **host,
                 suffix_capacity=d.suffix_capacity)
 
 

@@ -672,7 +672,8 @@ cudaError_t compose_launch(c2kv_ctx* c, const c2kv_cache* cache, const std::vect
         }
         const int32_t ts = bulk ? compose_bulk_tile_slots(c, occ, g0, g1, n_layers)
                                 : compose_tile_slots(c, slots, n_layers, max_ctas);
-        c2kv::ComposeParams pr{};
+        c2kv::ComposeParams pr;             // (its occurrences are written as far as n_occ: 24 KB)
+        static_cast<c2kv::ComposeHead&>(pr) = c2kv::ComposeHead{};
         pr.pool_k = c->pool_k;
         pr.pool_v = c->pool_v;
         pr.out_k = cache->k;
