@@ -414,7 +414,8 @@ const char* c2kv_last_error(const c2kv_ctx* ctx);
  */
 #define C2KV_PROF_COMPOSE  0
 #define C2KV_PROF_COMPRESS 1
-#define C2KV_PROF_SUFFIX   2   /* suffix RoPE + append + pad zeroing */
+#define C2KV_PROF_SUFFIX   2   /* suffix RoPE + append + pad zeroing (the tensor-core decode
+                                  kernel does these itself: no launch of this kind) */
 #define C2KV_PROF_ATTN     3   /* the attention kernel alone */
 #define C2KV_PROF_COMBINE  4   /* merge of key-range splits (when attention was split) */
 #define C2KV_PROF_DECODE   5   /* decode attention (with the merge of its splits) */

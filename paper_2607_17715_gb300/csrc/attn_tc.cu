@@ -112,11 +112,11 @@ constexpr int B_VE = B_VF + VSTAGES;     // + stage: V stage free (both P.V fini
 constexpr int B_SF = B_VE + VSTAGES;     // + tile: S_x(j) complete (and every MMA before it)
 constexpr int B_PF = B_SF + 2;           // + tile: P_x(j) written (and O_x corrected)
 constexpr int B_OD = B_PF + 2;           // every MMA finished: O_A, O_B final
-constexpr int B_KL = B_OD + 1;           // + stage (fused): the TMA part of a K tile landed
-constexpr int B_VL = B_KL + KSTAGES;     // + stage (fused): the TMA part of a V tile landed
+constexpr int B_KL = B_OD + 1;           // + stage (fused; decode: the last tile): the TMA part of a K tile landed
+constexpr int B_VL = B_KL + KSTAGES;     // + stage (fused; decode: the last tile): the TMA part of a V tile landed
 constexpr int B_KW = B_VL + VSTAGES;     // + stage (fused): K' of the stage's tile stored to the cache
 constexpr int B_VW = B_KW + KSTAGES;     // + stage (fused): V of the stage's tile stored
-constexpr int B_QR = B_VW + VSTAGES;     // (fused) Q turned in shared memory
+constexpr int B_QR = B_VW + VSTAGES;     // (fused, decode) Q turned in shared memory
 constexpr int B_SK = B_QR + 1;           // (fused) the suffix rows' K' turned into the cache
 constexpr int B_QF = B_SK + 1;           // every MMA of a pair has read its Q tiles
 constexpr int B_OE = B_QF + 1;           // a pair's epilogue has read O (pairs run in turn)
@@ -191,16 +191,34 @@ struct FusedTcParams {
     FusedOcc occ[kMaxFusedOcc];
 };
 
-template <bool kFused>
+// A decode step's launch (attn_tc_decode_kernel): t.tm_q covers the queries before RoPE, and the
+// kernel appends the new token's key and value rows itself.
+struct DecodeTcParams {
+    TcParams t;
+    const void* k_new;       // [Lq][Btot][Hkv][128], K before RoPE
+    const void* v_new;
+    void* cache_k;           // [L][rows][Hkv][128]
+    void* cache_v;
+    int32_t* pos;            // [rows]
+    uint32_t pad_mask[kMaxReq / 32];   // request i: zero the rows after the new one in its key tile
+    RopeTurns rope;
+};
+
+template <bool kFused, bool kKpp = false>
 struct KernelParams {
     using type = TcParams;
 };
 template <>
-struct KernelParams<true> {
+struct KernelParams<true, false> {
     using type = FusedTcParams;
+};
+template <>
+struct KernelParams<false, true> {
+    using type = DecodeTcParams;
 };
 __device__ __forceinline__ const TcParams& tc_params(const TcParams& p) { return p; }
 __device__ __forceinline__ const TcParams& tc_params(const FusedTcParams& p) { return p.t; }
+__device__ __forceinline__ const TcParams& tc_params(const DecodeTcParams& p) { return p.t; }
 
 // ------------------------------------------------------------------ tcgen05 wrappers
 
@@ -977,7 +995,7 @@ __device__ __forceinline__ void mma_issuer(const TcParams& P, uint32_t tmem, uin
     if (kHasB) st.pb += (uint32_t)n_kv;
 }
 
-// The MMA issuer for a pair with one query tile (tile A) and n_kv >= 2 key tiles, the key tiles
+// The MMA issuer for a pair with one query tile (tile A) and n_kv >= 1 key tiles, the key tiles
 // split between the two halves of TMEM: tiles 0, 2, 4, ... go to (S_A, O_A), tiles 1, 3, 5, ...
 // to (S_B, O_B), and the two softmax warpgroups each run an online softmax over their half, so
 // that one half's softmax overlaps the other's MMAs as two query tiles' do (warpgroup A merges
@@ -1017,7 +1035,7 @@ __device__ __forceinline__ void mma_issuer_kpp(const TcParams& P, uint32_t tmem,
     };
     wait(q_ready, q_par);
     s_next(0);
-    s_next(1);
+    if (n_kv > 1) s_next(1);
     uint32_t pa = st.pa, pb = st.pb;   // P phases of each half completed before this pair
 #pragma unroll 1
     for (int j = 0; j < n_kv; ++j) {
@@ -1814,11 +1832,12 @@ __device__ __forceinline__ void fused_suffix_prep(const FusedTcParams& F, int ts
 // The plain kernel's TMA producer (one thread) for the pairs [p_first, p_first + p_count)
 // that its CTA runs in turn: a pair's Q tiles once the MMAs of the previous pair have read
 // the last ones (B_QF), and the pairs' K and V tiles in order, each as soon as its ring stage
-// is free; whichever of the three can go first goes.
-template <bool kSif, int D>
+// is free; whichever of the three can go first goes.  append (decode): the last key tile is
+// decode_append's to pass on.
+template <bool kSif, int D, bool kKpp>
 __device__ __forceinline__ void plain_producer(const TcParams& P, int l, int bl, int b, int hk,
                                                int p_first, int p_count, int sp, int s_r, uint32_t sQ,
-                                               uint32_t sK, uint32_t sV, uint32_t sBar,
+                                               uint32_t sK, uint32_t sV, uint32_t sBar, bool append,
                                                volatile uint32_t* abort) {
     constexpr int kTile = Geo<D>::kTile;
     auto bar = [&](int i) { return sBar + 8u * (uint32_t)i; };
@@ -1851,9 +1870,10 @@ __device__ __forceinline__ void plain_producer(const TcParams& P, int l, int bl,
                                                        (uint32_t)((gk / KSTAGES) - 1) & 1u))) {
             const int s = gk % KSTAGES;
             const int krow = key0 + (kSif ? span_tile(sk, jk) : sk.j_base + jk) * BN;
-            mbar_expect_tx(bar(B_KF + s), kTile);
-            tma_load_3d(sK + s * kTile, &P.tm_k, 0, hk, krow, bar(B_KF + s));
-            if (D == 128) tma_load_3d(sK + s * kTile + HALF_TILE, &P.tm_k, 64, hk, krow, bar(B_KF + s));
+            const uint32_t full = bar(kKpp && append && jk == sk.n_kv - 1 ? B_KL : B_KF + s);
+            mbar_expect_tx(full, kTile);
+            tma_load_3d(sK + s * kTile, &P.tm_k, 0, hk, krow, full);
+            if (D == 128) tma_load_3d(sK + s * kTile + HALF_TILE, &P.tm_k, 64, hk, krow, full);
             ++gk;
             if (++jk == sk.n_kv) {
                 jk = 0;
@@ -1866,9 +1886,10 @@ __device__ __forceinline__ void plain_producer(const TcParams& P, int l, int bl,
                                                        (uint32_t)((gv / VSTAGES) - 1) & 1u))) {
             const int s = gv % VSTAGES;
             const int vrow = key0 + (kSif ? span_tile(sv, jv) : sv.j_base + jv) * BN;
-            mbar_expect_tx(bar(B_VF + s), kTile);
-            tma_load_3d(sV + s * kTile, &P.tm_v, 0, hk, vrow, bar(B_VF + s));
-            if (D == 128) tma_load_3d(sV + s * kTile + HALF_TILE, &P.tm_v, 64, hk, vrow, bar(B_VF + s));
+            const uint32_t full = bar(kKpp && append && jv == sv.n_kv - 1 ? B_VL : B_VF + s);
+            mbar_expect_tx(full, kTile);
+            tma_load_3d(sV + s * kTile, &P.tm_v, 0, hk, vrow, full);
+            if (D == 128) tma_load_3d(sV + s * kTile + HALF_TILE, &P.tm_v, 64, hk, vrow, full);
             ++gv;
             if (++jv == sv.n_kv) {
                 jv = 0;
@@ -1912,6 +1933,114 @@ __global__ void __launch_bounds__(256) suffix_angles_kernel(const __grid_constan
     }
 }
 
+// A decode CTA's queries: the softmax warps (ts = 0..255) form the angles of the new token's
+// position in `tab` and turn the G live rows of the query tile in shared memory, then tell the MMA
+// issuer (B_QR).  The suffix kernel's angles and rounding.
+__device__ __forceinline__ void decode_turn_queries(const DecodeTcParams& X, int ts, int64_t pos, uint32_t sQ,
+                                                    float2* tab, uint32_t sBar, volatile uint32_t* abort) {
+    const TcParams& P = X.t;
+    if (ts < HD / 2) tab[ts] = turn_cs(X.rope.turn[ts], pos);
+    asm volatile("bar.sync 5, 256;" ::: "memory");
+    mbar_wait(sBar + 8u * B_Q, 0u, P.err, abort);
+    const int g = ts >> 3, q = ts & 7;
+    if (g < P.group) {
+        const uint32_t a0 = sQ + sw_off(g, q);
+        const uint4 xv = lds128(a0), yv = lds128(a0 + HALF_TILE);
+        const uint32_t xw[4] = {xv.x, xv.y, xv.z, xv.w}, yw[4] = {yv.x, yv.y, yv.z, yv.w};
+        uint32_t xo[4], yo[4];
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+            const float2 e0 = tab[8 * q + 2 * w], e1 = tab[8 * q + 2 * w + 1];
+            float2 gx, gy;
+            rotate2(bf2_to_f2(xw[w]), bf2_to_f2(yw[w]), make_float2(e0.x, e1.x), make_float2(e0.y, e1.y), gx, gy);
+            xo[w] = f2_to_bf2(gx.x, gx.y);
+            yo[w] = f2_to_bf2(gy.x, gy.y);
+        }
+        sts128(a0, make_uint4(xo[0], xo[1], xo[2], xo[3]));
+        sts128(a0 + HALF_TILE, make_uint4(yo[0], yo[1], yo[2], yo[3]));
+    }
+    fence_proxy_async();
+    mbar_arrive(sBar + 8u * B_QR);
+}
+
+// The new token's key and value rows (one warp of the CTA whose key tiles end with theirs): turned
+// and written to the cache (with the row's position, and zeros after it up to the tile's edge when
+// nothing finite is there yet), and, once the tile has landed, written into it in shared memory (the
+// copy engine may have read the cache before or after): the tile's loads complete barriers of their
+// own (B_KL, B_VL), and this warp then fills the stage's for the MMA issuer.  It takes a kernel of
+// its own (3.5 us, then the attention's start behind it) out of every step: 16 requests of 1163 keys
+// 20.7 -> 18.5 us, one of 131k keys 91.8 -> 89.6.
+__device__ __forceinline__ void decode_append(const DecodeTcParams& X, int lane, int l, int bl, int b, int hk, int n_kv,
+                                              int64_t pos, uint32_t sK, uint32_t sV, float2* tab, uint32_t sBar,
+                                              volatile uint32_t* abort) {
+    using bf = __nv_bfloat16;
+    const TcParams& P = X.t;
+    const ReqParam& rq = P.req[bl];
+    const int row = rq.n_slots + rq.t0, rt = row % BN;      // the new row, in the request and in its tile
+    const bool pad = (X.pad_mask[bl >> 5] >> (bl & 31)) & 1u;
+    const int64_t src = (((int64_t)l * P.batch_total + b) * P.hkv + hk) * HD;
+    const int64_t stride = (int64_t)P.hkv * HD;
+    const int64_t dst = (((int64_t)(P.layer0 + l) * P.rows + rq.row_base + row) * P.hkv + hk) * HD;
+    bf* const ck = static_cast<bf*>(X.cache_k) + dst;
+    bf* const cv = static_cast<bf*>(X.cache_v) + dst;
+    uint4 a = make_uint4(0u, 0u, 0u, 0u), o = a;
+    const int q = lane & 7, c = lane - 8;                   // lanes 0..7: K's chunk pair q; 8..23: V's chunk c
+    if (lane < 8) {
+        a = ld16(static_cast<const bf*>(X.k_new) + src + 8 * q);
+        o = ld16(static_cast<const bf*>(X.k_new) + src + 64 + 8 * q);
+    } else if (c < 16) {
+        a = ld16(static_cast<const bf*>(X.v_new) + src + 8 * c);
+    }
+    for (int i = lane; i < HD / 2; i += 32) tab[i] = turn_cs(X.rope.turn[i], pos);
+    __syncwarp();
+    if (lane < 8) {
+        const uint32_t xw[4] = {a.x, a.y, a.z, a.w}, yw[4] = {o.x, o.y, o.z, o.w};
+        uint32_t xo[4], yo[4];
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+            const float2 e0 = tab[8 * q + 2 * w], e1 = tab[8 * q + 2 * w + 1];
+            float2 gx, gy;
+            rotate2(bf2_to_f2(xw[w]), bf2_to_f2(yw[w]), make_float2(e0.x, e1.x), make_float2(e0.y, e1.y), gx, gy);
+            xo[w] = f2_to_bf2(gx.x, gx.y);
+            yo[w] = f2_to_bf2(gy.x, gy.y);
+        }
+        a = make_uint4(xo[0], xo[1], xo[2], xo[3]);
+        o = make_uint4(yo[0], yo[1], yo[2], yo[3]);
+        st16(ck + 8 * q, a);
+        st16(ck + 64 + 8 * q, o);
+    } else if (c < 16) {
+        st16(cv + 8 * c, a);
+    }
+    if (lane == 24 && l == 0 && hk == 0) X.pos[rq.row_base + row] = (int32_t)pos;
+    const uint4 z = make_uint4(0u, 0u, 0u, 0u);
+    if (pad)
+        for (int i = lane; i < (BN - 1 - rt) * 16; i += 32) {
+            const int64_t off = (int64_t)(1 + (i >> 4)) * stride + (i & 15) * 8;
+            st16(ck + off, z);
+            st16(cv + off, z);
+        }
+    auto patch = [&](uint32_t tile, bool is_k) {
+        if (is_k && lane < 8) {
+            sts128(tile + sw_off(rt, q), a);
+            sts128(tile + HALF_TILE + sw_off(rt, q), o);
+        } else if (!is_k && lane >= 8 && c < 16) {
+            sts128(tile + (uint32_t)((c >> 3) * HALF_TILE) + sw_off(rt, c & 7), a);
+        }
+        if (pad)
+            for (int i = lane; i < (BN - 1 - rt) * 16; i += 32)
+                sts128(tile + (uint32_t)(((i >> 3) & 1) * HALF_TILE) + sw_off(rt + 1 + (i >> 4), i & 7), z);
+        fence_proxy_async();
+        __syncwarp();
+    };
+    const int ks = (n_kv - 1) % KSTAGES, vs = (n_kv - 1) % VSTAGES;
+    mbar_wait(sBar + 8u * (uint32_t)B_KL, 0u, P.err, abort);
+    patch(sK + (uint32_t)(ks * TILE), true);
+    if (lane == 0) mbar_arrive(sBar + 8u * (uint32_t)(B_KF + ks));
+    mbar_wait(sBar + 8u * (uint32_t)B_VL, 0u, P.err, abort);
+    patch(sV + (uint32_t)(vs * TILE), false);
+    if (lane == 0) mbar_arrive(sBar + 8u * (uint32_t)(B_VF + vs));
+}
+
 // kFused: compose + suffix preparation + attention; kMulti (fused only): the CTA runs every
 // pair of query tiles of its (layer, request, KV head), the last pair first (it composes the
 // cache), the others from the cache.  A separate instantiation, so that the one-pair fused
@@ -1920,7 +2049,7 @@ __global__ void __launch_bounds__(256) suffix_angles_kernel(const __grid_constan
 // stays as it is.
 // D: head dimension (64 in the plain and the SIF kernel only).
 template <bool kFused, bool kMulti, bool kSif, bool kKpp = false, int D = HD>
-__device__ __forceinline__ void attn_tc_body(const typename KernelParams<kFused>::type& KP) {
+__device__ __forceinline__ void attn_tc_body(const typename KernelParams<kFused, kKpp>::type& KP) {
     static_assert(D == HD || (!kFused && !kKpp), "64 channels: the plain and SIF kernels");
     constexpr int kTile = Geo<D>::kTile;
     const TcParams& P = tc_params(KP);
@@ -1966,6 +2095,8 @@ __device__ __forceinline__ void attn_tc_body(const typename KernelParams<kFused>
     const bool has_b = ps0.has_b;
     const int j_base = ps0.j_base;
     const int n_kv = ps0.n_kv;
+    // decode: this CTA's key tiles end with the new token's
+    const bool append = kKpp && n_kv > 0 && j_base + n_kv - 1 == s_r / BN;
 
     if (!kFused && threadIdx.x == 0 && n_kv > 0) {
         // the first pair's Q tiles and first key tile on their way into L2 while the CTA sets
@@ -2051,7 +2182,8 @@ __device__ __forceinline__ void attn_tc_body(const typename KernelParams<kFused>
                     if (p_count > 1)
                         fused_rest_producer(KP, l, bl, b, hk, p_count, s_r, n_kv, sQ, sK, sV, sBar, abort);
             } else {
-                plain_producer<kSif, D>(P, l, bl, b, hk, p_first, p_count, sp, s_r, sQ, sK, sV, sBar, abort);
+                plain_producer<kSif, D, kKpp>(P, l, bl, b, hk, p_first, p_count, sp, s_r, sQ, sK, sV, sBar, append,
+                                              abort);
             }
         } else if (warp == 1 && lane == 0 && n_kv > 0) {
             // ------------------------------------------------------------ MMA issuer
@@ -2076,8 +2208,8 @@ __device__ __forceinline__ void attn_tc_body(const typename KernelParams<kFused>
                     const uint32_t q_par = (uint32_t)pi & 1u, oe_par = (uint32_t)(pi - 1) & 1u;
                     if (ps.has_b)
                         mma_issuer<true, D>(P, tmem, sQ, sK, sV, sBar, ps.n_kv, B_Q, q_par, st, pi > 0, oe_par, abort);
-                    else if (kKpp && ps.n_kv >= 2 && pi == p_count - 1)   // key tiles ping-pong
-                        mma_issuer_kpp(P, tmem, sQ, sK, sV, sBar, ps.n_kv, B_Q, q_par, st, pi > 0, oe_par, abort);
+                    else if (kKpp)                                        // key tiles ping-pong (one pair)
+                        mma_issuer_kpp(P, tmem, sQ, sK, sV, sBar, ps.n_kv, B_QR, q_par, st, pi > 0, oe_par, abort);
                     else
                         mma_issuer<false, D>(P, tmem, sQ, sK, sV, sBar, ps.n_kv, B_Q, q_par, st, pi > 0, oe_par, abort);
                 }
@@ -2087,6 +2219,11 @@ __device__ __forceinline__ void attn_tc_body(const typename KernelParams<kFused>
             if constexpr (kFused)
                 fused_writer(KP, l, bl, hk, j_base, n_kv, sK, sV, sBar, kMulti && p_count > 1, abort);
         } else if (warp == 3 && n_kv > 0) {
+            // ------------------------------------------------------------ new row (decode)
+            if constexpr (kKpp)
+                if (append)
+                    decode_append(KP, lane, l, bl, b, hk, n_kv, (int64_t)P.req[bl].l_req + P.req[bl].t0, sK, sV,
+                                  reinterpret_cast<float2*>(smem + TILE + 8192), sBar, abort);
             // ------------------------------------------------------------ V loader (fused)
             if constexpr (kFused)
                 fused_v_loader(KP, lane, l, bl, hk, j_base, n_kv, kMulti ? n_all : n_kv, sV, sBar, abort);
@@ -2130,9 +2267,13 @@ __device__ __forceinline__ void attn_tc_body(const typename KernelParams<kFused>
             uint32_t done = 0u;     // S_x tiles of the earlier pairs
             for (int pi = 0; pi < p_count; ++pi) {
                 const PairSpan ps = pi == 0 ? ps0 : pair_span(P, p_first + pi, sp, s_r);
-                // one query tile over two or more key tiles (the CTA's last pair): the two
-                // warpgroups take alternate key tiles (mma_issuer_kpp) and merge at the end
-                const bool kpp = kKpp && !ps.has_b && ps.n_kv >= 2 && pi == p_count - 1;
+                // a decode step's one query tile: the two warpgroups take alternate key tiles
+                // (mma_issuer_kpp) and merge at the end
+                const bool kpp = kKpp && ps.n_kv >= 1;
+                if constexpr (kKpp)
+                    if (kpp)
+                        decode_turn_queries(KP, (int)threadIdx.x - 128, (int64_t)P.req[bl].l_req + P.req[bl].t0, sQ,
+                                            reinterpret_cast<float2*>(smem + TILE + 4096), sBar, abort);
                 if (x == 0 || ps.has_b || kpp) {
                     softmax_tile<true, kSif, kKpp, D>(P, tmem, sBar, x, warp & 3, lane, x && !kpp ? ps.t0b : ps.t0a, l, bl,
                                  b, hk, sp, ps, done, (uint32_t)pi & 1u, p_count > 1, abort,
@@ -2168,7 +2309,7 @@ __device__ __forceinline__ void attn_tc_body(const typename KernelParams<kFused>
 
 template <bool kFused, bool kMulti = false>
 __global__ void __launch_bounds__(kFused ? kThreadsFused : kThreads, 1)
-    attn_tc_kernel(const __grid_constant__ typename KernelParams<kFused>::type KP) {
+    attn_tc_kernel(const __grid_constant__ typename KernelParams<kFused, false>::type KP) {
     attn_tc_body<kFused, kMulti, false>(KP);
 }
 
@@ -2186,7 +2327,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc64_sif_kernel(const __grid
 
 // Decode steps (AttnParams::key_pingpong): the plain kernel whose last pair, when it has one
 // query tile, splits its key tiles between the two softmax warpgroups.
-__global__ void __launch_bounds__(kThreads, 1) attn_tc_decode_kernel(const __grid_constant__ TcParams KP) {
+__global__ void __launch_bounds__(kThreads, 1) attn_tc_decode_kernel(const __grid_constant__ DecodeTcParams KP) {
     attn_tc_body<false, false, false, true>(KP);
 }
 
@@ -2644,7 +2785,7 @@ cudaError_t prepare_tc(const AttnParams& a, TcParams& p, dim3& grid) {
     if (a.q_cs != nullptr && !kSolo) return cudaErrorInvalidValue;
 
     if (kSif != (a.sif_k > 0) || a.sif_k < 0 || (kSif && (kFused || p.n_split != 1))) return cudaErrorInvalidValue;
-    if (kKpp != (a.key_pingpong != 0) || (kKpp && (kFused || kSif))) return cudaErrorInvalidValue;
+    if (kKpp != (a.key_pingpong != 0) || (kKpp && (kFused || kSif || a.sq != 1))) return cudaErrorInvalidValue;
     if (a.batch < 1 || a.batch > kMaxReq) return cudaErrorInvalidValue;
     std::memcpy(p.req, a.req, sizeof(ReqParam) * (size_t)a.batch);
     const int64_t pairs = ((a.sq + tq - 1) / tq + 1) / 2;
@@ -2695,11 +2836,11 @@ cudaError_t preload_attn_tc_kernels(int d) {
 
 namespace {
 
-template <bool kSif, bool kKpp, int D, int kSolo = 0>
+template <bool kSif, int D, int kSolo = 0>
 cudaError_t launch_plain(const AttnParams& a, cudaStream_t s, Hook before) {
     TcParams p;
     dim3 grid;
-    cudaError_t e = prepare_tc<false, false, kSif, kKpp, D, kSolo>(a, p, grid);
+    cudaError_t e = prepare_tc<false, false, kSif, false, D, kSolo>(a, p, grid);
     if (e != cudaSuccess) return e;
     before();
     cudaLaunchConfig_t cfg{};
@@ -2715,7 +2856,7 @@ cudaError_t launch_plain(const AttnParams& a, cudaStream_t s, Hook before) {
         cfg.numAttrs = 1;
     }
     void* args[1] = {&p};
-    e = cudaLaunchKernelExC(&cfg, tc_kernel_fn<false, false, kSif, kKpp, D, kSolo>(), args);
+    e = cudaLaunchKernelExC(&cfg, tc_kernel_fn<false, false, kSif, false, D, kSolo>(), args);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -2749,21 +2890,39 @@ SoloChoice solo_choice(const AttnParams& a) {
 template <bool kSif, int D>
 cudaError_t launch_form(SoloChoice c, const AttnParams& a, cudaStream_t s, Hook before) {
     if constexpr (!kSif)
-        if (c == SoloChoice::kAlone) return launch_plain<false, false, D, 2>(a, s, before);
-    if (c == SoloChoice::kShared) return launch_plain<kSif, false, D, 1>(a, s, before);
-    return launch_plain<kSif, false, D>(a, s, before);
+        if (c == SoloChoice::kAlone) return launch_plain<false, D, 2>(a, s, before);
+    if (c == SoloChoice::kShared) return launch_plain<kSif, D, 1>(a, s, before);
+    return launch_plain<kSif, D>(a, s, before);
 }
 
 }  // namespace
 
 cudaError_t launch_attn_tc(const AttnParams& a, cudaStream_t s, Hook before) {
     (void)cudaGetLastError();   // report this launch's error only, not a stale one
-    if (a.d != HD && (a.d != 64 || a.key_pingpong)) return cudaErrorInvalidValue;
+    if ((a.d != HD && a.d != 64) || a.key_pingpong) return cudaErrorInvalidValue;
     const SoloChoice solo = solo_choice(a);
     if (a.d == 64)
         return a.sif_k > 0 ? launch_form<true, 64>(solo, a, s, before) : launch_form<false, 64>(solo, a, s, before);
-    if (a.key_pingpong) return launch_plain<false, true, HD>(a, s, before);    // decode steps
     return a.sif_k > 0 ? launch_form<true, HD>(solo, a, s, before) : launch_form<false, HD>(solo, a, s, before);
+}
+
+cudaError_t launch_attn_tc_decode(const AttnParams& a, const DecodeAppend& d, cudaStream_t s, Hook before) {
+    (void)cudaGetLastError();   // report this launch's error only, not a stale one
+    if (!d.k_new || !d.v_new || !d.pos || a.d != HD) return cudaErrorInvalidValue;
+    DecodeTcParams p;
+    dim3 grid;
+    cudaError_t e = prepare_tc<false, false, false, true>(a, p.t, grid);
+    if (e != cudaSuccess) return e;
+    p.k_new = d.k_new;
+    p.v_new = d.v_new;
+    p.cache_k = const_cast<void*>(a.cache_k);
+    p.cache_v = const_cast<void*>(a.cache_v);
+    p.pos = d.pos;
+    std::memcpy(p.pad_mask, d.pad_mask, sizeof(p.pad_mask));
+    p.rope = d.rope;
+    before();
+    attn_tc_decode_kernel<<<grid, kThreads, kSmemBytes, s>>>(p);
+    return cudaGetLastError();
 }
 
 namespace {

@@ -1367,9 +1367,10 @@ c2kv_status c2kv_decode(c2kv_ctx* c, c2kv_cache* cache, int32_t layer, const voi
         }
         const int32_t keys_per_split = (n_keys_max + n_split - 1) / n_split;
 
+        // the turned queries (the tensor-core kernel turns them, and appends the new rows, itself)
         const size_t q_bytes = (size_t)lq * B * hq * d * c->eb;
         void* q_rot = nullptr;
-        cudaError_t e = pool_alloc(c, &q_rot, q_bytes);
+        cudaError_t e = use_tc ? cudaSuccess : pool_alloc(c, &q_rot, q_bytes);
         if (e != cudaSuccess) return cuda_fail(c, e, "decode: scratch allocation");
         float* part = nullptr;
         const size_t rows_all = (size_t)lq * B * hq;
@@ -1388,7 +1389,6 @@ c2kv_status c2kv_decode(c2kv_ctx* c, c2kv_cache* cache, int32_t layer, const voi
         // the next 128-row edge must hold finite values (masked keys weigh zero, but 0 * NaN is
         // not zero), so each request's are zeroed once, when not written or zeroed before
         std::vector<int32_t> edge(B), pad_from(B);
-        bool any_pad = false;
         for (int32_t b = 0; b < B; ++b) {
             const int64_t next = (int64_t)cache->n_slots[b] + steps[b] + 1;
             edge[b] = (int32_t)std::min<int64_t>((next + kTileRows - 1) / kTileRows * kTileRows, cache->capacity[b]);
@@ -1396,44 +1396,15 @@ c2kv_status c2kv_decode(c2kv_ctx* c, c2kv_cache* cache, int32_t layer, const voi
             for (int32_t l = layer0; use_tc && l < layer0 + lq; ++l)
                 need = need || cache->clean_to[(size_t)l * B + b] < edge[b];
             pad_from[b] = need ? (int32_t)next : (int32_t)((next + kTileRows - 1) / kTileRows * kTileRows);
-            any_pad = any_pad || need;
         }
         std::vector<c2kv::ReqParam> reqs(B);
         for (int32_t b = 0; b < B; ++b)
             reqs[b] = c2kv::ReqParam{cache->row_base[b], cache->n_slots[b], cache->l_req[b], steps[b]};
         for (int32_t b0 = 0; e == cudaSuccess && b0 < B; b0 += c2kv::kMaxReq) {
             const int32_t nb = std::min<int32_t>(c2kv::kMaxReq, B - b0);
-            c2kv::SuffixParams s{};
-            s.q = q;
-            s.k = k_new;
-            s.v = v_new;
-            s.q_rot = q_rot;
-            s.cache_k = cache->k;
-            s.cache_v = cache->v;
-            s.pos = cache->pos;
-            s.rows = cache->rows;
-            s.layer0 = layer0;
-            s.lq = lq;
-            s.batch = nb;
-            s.batch_total = B;
-            s.b0 = b0;
-            s.sq = 1;
-            s.hq = hq;
-            s.hkv = hkv;
-            s.pad_rows = any_pad ? 1 : 0;
-            s.rope = c->turns;
-            for (int32_t i = 0; i < nb; ++i) {
-                s.req[i] = reqs[b0 + i];
-                s.pad_from[i] = pad_from[b0 + i];
-            }
-            {
-                ProfScope prof_suffix(c, C2KV_PROF_SUFFIX);
-                e = c2kv::launch_suffix_prep(s, c->cfg.dtype, d, c->stream);
-            }
-            if (e != cudaSuccess) break;
             if (use_tc) {
                 c2kv::AttnParams a{};
-                a.q_rot = q_rot;
+                a.q_rot = q;
                 a.cache_k = cache->k;
                 a.cache_v = cache->v;
                 a.out = out;
@@ -1460,16 +1431,46 @@ c2kv_status c2kv_decode(c2kv_ctx* c, c2kv_cache* cache, int32_t layer, const voi
                 a.tickets = in_kernel ? c->tickets : nullptr;
                 // the two softmax warpgroups take alternate key tiles of the one query tile
                 a.key_pingpong = 1;
-                // the suffix kernel's programmatic dependent, unless a trace puts events
-                // between them
-                a.dependent = c->prof ? 0 : 1;
+                a.dependent = c->prof ? 0 : 1;    // (the merge launch's)
                 for (int32_t i = 0; i < nb; ++i) a.req[i] = reqs[b0 + i];
+                c2kv::DecodeAppend ap{};
+                ap.k_new = k_new;
+                ap.v_new = v_new;
+                ap.pos = cache->pos;
+                ap.rope = c->turns;
+                for (int32_t i = 0; i < nb; ++i)
+                    if (pad_from[b0 + i] < edge[b0 + i]) ap.pad_mask[i / 32] |= 1u << (i % 32);
                 ProfScope prof_decode(c, C2KV_PROF_DECODE, true);
-                e = c2kv::launch_attn_tc(a, c->stream, prof_decode.hook());
+                e = c2kv::launch_attn_tc_decode(a, ap, c->stream, prof_decode.hook());
                 if (e == cudaSuccess && n_split > 1 && !in_kernel && b0 + nb >= B)
                     e = c2kv::launch_attn_combine(a, c->stream);
                 continue;
             }
+            c2kv::SuffixParams s{};
+            s.q = q;
+            s.k = k_new;
+            s.v = v_new;
+            s.q_rot = q_rot;
+            s.cache_k = cache->k;
+            s.cache_v = cache->v;
+            s.pos = cache->pos;
+            s.rows = cache->rows;
+            s.layer0 = layer0;
+            s.lq = lq;
+            s.batch = nb;
+            s.batch_total = B;
+            s.b0 = b0;
+            s.sq = 1;
+            s.hq = hq;
+            s.hkv = hkv;
+            s.pad_rows = 0;      // (this kernel reads no row after the new one)
+            s.rope = c->turns;
+            for (int32_t i = 0; i < nb; ++i) s.req[i] = reqs[b0 + i];
+            {
+                ProfScope prof_suffix(c, C2KV_PROF_SUFFIX);
+                e = c2kv::launch_suffix_prep(s, c->cfg.dtype, d, c->stream);
+            }
+            if (e != cudaSuccess) break;
             c2kv::DecodeParams p{};
             p.q_rot = q_rot;
             p.cache_k = cache->k;

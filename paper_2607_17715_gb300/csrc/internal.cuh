@@ -155,10 +155,9 @@ struct AttnParams {
                              // merges), or one zeroed counter per (layer, request, KV head,
                              // pair): the unit's last split merges the partials in the kernel
                              // and sets it back to zero
-    int32_t key_pingpong;    // tensor-core kernel: a pair with one query tile (a decode step's)
+    int32_t key_pingpong;    // 1: a decode step (launch_attn_tc_decode), whose one query tile
                              // splits its key tiles between the two softmax warpgroups, merged
-                             // at the end (a different rounding order: off where the result must
-                             // equal the fused kernel's bit for bit)
+                             // at the end
     int32_t sif_k;           // tensor-core kernel, extraction C2 rows (Sec. 3.3.1): 0, or the
                              // ratio k: the request's n_slots key rows are then the chunk's n
                              // document tokens, suffix token j is C2 token c_j, and of the
@@ -265,6 +264,17 @@ bool encode_tensor_map(CUtensorMap* tm, CUtensorMapDataType type, int rank, cons
 bool attn_tc_supported(int dtype, int d, int hq, int hkv);
 bool attn_tc_takes(int dtype, int d, int hq, int hkv);
 cudaError_t launch_attn_tc(const AttnParams& p, cudaStream_t s, Hook before = {});
+// A decode step on the tensor cores (AttnParams with sq 1, key_pingpong 1; its q_rot is the queries
+// before RoPE): the new token's key and value rows are appended by the same kernel.
+struct DecodeAppend {
+    const void* k_new;       // [Lq][B][Hkv][128], K before RoPE
+    const void* v_new;
+    int32_t* pos;            // [rows]
+    uint32_t pad_mask[kMaxReq / 32];   // request i of the launch: zero the rows after the new one up
+                                       // to the next 128-row boundary
+    RopeTurns rope;
+};
+cudaError_t launch_attn_tc_decode(const AttnParams& a, const DecodeAppend& d, cudaStream_t s, Hook before = {});
 // Merge n_split partial (O, lse) over disjoint key ranges into out (bf16) and lse (attn_tc.cu).
 cudaError_t launch_attn_combine(const AttnParams& p, cudaStream_t s);
 // Query tiles of one tensor-core attention launch, and pairs of them (the pair kernel's CTAs),
