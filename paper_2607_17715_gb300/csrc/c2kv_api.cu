@@ -1030,7 +1030,20 @@ cudaError_t compose_attend_pipelined(c2kv_ctx* c, c2kv_cache* cache, const std::
                                      const void* q, const void* k_suf, const void* v_suf,
                                      int32_t n_suffix, void* out, float* lse) {
     const int32_t L = c->cfg.layers;
-    const int32_t groups = std::min<int32_t>(4, L);
+    // A group costs some 25 us of its own (its copies and kernels start one after the other), and its
+    // attention hides behind the next group's reading: one for every 64 MB over the link, up to four.
+    // Measured (1 / 2 / 3 / 4 groups, us a call): 8 layers x 1280 slots, 64 suffix tokens (53 MB)
+    // 291 / 296 / 308 / 344; 4 layers 171 / 181 / 181 / 241; 32 layers (210 MB) 1090 / 1057 / 1057 /
+    // 1069; 8 layers x 5120 slots, 256 tokens (210 MB) 1187 / 1112 / 1081 / 1091; 16 layers, 512 tokens
+    // (250 MB) 1536 / 1399 / 1410 / 1411.
+    int64_t host_slots = 0;
+    for (const c2kv::OccParam& o : occ)
+        if (o.host) host_slots += o.m;
+    const double row = (double)c->cfg.head_dim * c->eb;
+    const double link_bytes =
+        row * L * (2.0 * c->cfg.n_kv_heads * (double)host_slots +
+                   2.0 * (c->cfg.n_kv_heads + c->cfg.n_q_heads) * (double)cache->batch * n_suffix);
+    const int32_t groups = std::min<int32_t>({4, L, std::max<int32_t>(1, (int32_t)std::min(4.0, link_bytes / 64e6 + 0.5))});
     const int32_t per = (L + groups - 1) / groups;
     cudaError_t e = aux_ready(c, (size_t)groups + 2);
     if (e != cudaSuccess) return e;
