@@ -2358,7 +2358,9 @@ static_assert(2 * (Solo<HD, false>::kSmem + 1024) <= 228 * 1024 && 2 * (Solo<64,
 // The queries of a solo CTA turned in shared memory (TcParams::q_cs): the softmax warps (ts =
 // 0..127), which have nothing else to do until the first S, take item (token, chunk pair q = ts %
 // NQ): its 8 frequencies' (cos, sin) from the table, fetched while Q lands, then chunk pair q of the
-// token's G query rows (the rope kernel's rounding).  Then the MMA issuer is told (B_QR).
+// token's G query rows (the rope kernel's rounding).  Then the MMA issuer is told (B_QR).  The rows
+// one at a time: two or four unrolled make the CTA's once-run code longer (32 layers x 512 tokens:
+// extraction 195.4 us rolled, 199.3 by two, 205 by four).
 template <int D>
 __device__ __forceinline__ void solo_turn_queries(const TcParams& P, int ts, const PairSpan& span, uint32_t sQ,
                                                   uint32_t sBar, volatile uint32_t* abort) {
@@ -2374,7 +2376,7 @@ __device__ __forceinline__ void solo_turn_queries(const TcParams& P, int ts, con
         }
     };
     auto turn = [&](int tt, const float2 (&cc)[4], const float2 (&ss)[4]) {
-#pragma unroll 2
+#pragma unroll 1
         for (int g = 0; g < G; ++g) {
             const int r = (tt - span.t0a) * G + g;
             // channels 8 q .. of a 64-channel block and their partners, in the other block (128
