@@ -2791,10 +2791,13 @@ cudaError_t prepare_tc(const AttnParams& a, TcParams& p, dim3& grid) {
     if (a.batch < 1 || a.batch > kMaxReq) return cudaErrorInvalidValue;
     std::memcpy(p.req, a.req, sizeof(ReqParam) * (size_t)a.batch);
     const int64_t pairs = ((a.sq + tq - 1) / tq + 1) / 2;
-    // The plain kernel runs several pairs of one (layer, request, KV head) per CTA when the
-    // launch is many waves of CTAs: each CTA's fixed cost (TMEM, barriers, the first tiles
-    // from HBM, the epilogue) is then paid once for several short pairs (causal extraction
-    // rows: 1 to 4 key tiles a pair).  The context's attn_pairs setting caps the choice.
+    // The plain kernel may run several pairs of one (layer, request, KV head) per CTA, one after the
+    // other.  A change of pair costs about as much (8 us: the last softmax, P.V and epilogue, then the
+    // next Q and softmax) as a CTA's start and end, so that this only pays where it saves a round of
+    // CTAs: the choice with the least rounds x (1.5 + pairs x (8 + 1.6 a key tile)).  Measured at 1 / 2
+    // pairs a CTA (us a call; 32 / 8 heads, 11 key tiles): 256 pairs 63.3 / 61.1, 384 89.7 / 106.4, 640
+    // (four a head) 131 / 146, 1024 204 / 220; 64 / 8 heads, 22 key tiles, 512 pairs (16 a head) 170 /
+    // 171, three in turn 228.  The context's attn_pairs setting caps the choice.
     int64_t pg = 1;
     if (kSolo) {
         if (p.n_split > 1 && (p.tickets || kSif)) return cudaErrorInvalidValue;
@@ -2809,8 +2812,18 @@ cudaError_t prepare_tc(const AttnParams& a, TcParams& p, dim3& grid) {
                 return 1;
             return n;
         }();
-        const int64_t ctas = pairs * a.hkv * a.lq * a.batch;
-        pg = std::max<int64_t>(1, std::min<int64_t>(pairs, ctas / sms));
+        const int64_t cols = (int64_t)a.hkv * a.lq * a.batch;
+        int slots = 0;
+        for (int i = 0; i < a.batch; ++i) slots = std::max(slots, a.req[i].n_slots + a.req[i].t0);
+        const double pair_us = 8.0 + 1.6 * ((slots + a.sq + BN - 1) / BN);
+        double best = 0.0;
+        for (int64_t n = 1; n <= std::min<int64_t>(pairs, 16); ++n) {
+            const double us = (double)(((pairs + n - 1) / n * cols + sms - 1) / sms) * (1.5 + (double)n * pair_us);
+            if (n == 1 || us < 0.985 * best) {
+                best = us;
+                pg = n;
+            }
+        }
         if (a.pairs_per_cta >= 1) pg = std::min<int64_t>(pairs, a.pairs_per_cta);
     }
     p.pairs = (int32_t)pairs;
