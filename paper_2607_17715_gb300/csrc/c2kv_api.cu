@@ -811,6 +811,50 @@ int32_t attn_splits(const c2kv_ctx* c, const c2kv_cache* cache, int32_t lq, int3
     return best;
 }
 
+// Whether compose_attend's fused kernel is expected to be faster than compose, then attention (one pair
+// of query tiles a head).  It is where every key tile lies within one chunk or the suffix.  A tile that
+// holds a boundary (a ragged chunk's end) costs its loaders 11.5 us rather than 2.3 (1.75 with one
+// query tile), so with such tiles a model of both (us) decides; compose moves its bytes at 6.7 TB/s.
+// Measured, fused / unfused (32 / 8 heads, 64 suffix tokens, chunks x slots): 32 layers, 10 x 128:
+// 81 / 107, 10 x 125: 270 / 107; 16 layers, 10 x 130: 132 / 61, 3 x 500: 77 / 68, 20 x 64: 132 / 61; one
+// layer, 2 requests, 10 x 125: 136 / 33.  The results are the same bits, unless the keys are split.
+bool fused_pays(const c2kv_ctx* c, const c2kv_cache* cache, const std::vector<c2kv::OccParam>& occ,
+                const int32_t* req_ptr, int32_t n_suffix) {
+    const int32_t L = c->cfg.layers, B = cache->batch, hkv = c->cfg.n_kv_heads;
+    const int64_t units = (int64_t)L * B * hkv;
+    const double rounds = (double)((units + c->sms - 1) / c->sms);
+    const bool two = c2kv::attn_tc_tiles(c->cfg.n_q_heads, hkv, n_suffix, 1, 1) > hkv;
+    const double clean_us = two ? 2.26 : 1.75, start_us = two ? 10.7 : 8.0, key_us = two ? 1.6 : 1.0;
+    bool merge = false;
+    const int32_t split = attn_splits(c, cache, L, n_suffix, true, &merge);
+    double longest = 0.0, mean = 0.0, keys = 0.0, rows = 0.0;
+    bool boundaries = false;
+    for (int32_t b = 0; b < B; ++b) {
+        const int32_t tiles = (cache->n_slots[b] + n_suffix + kTileRows - 1) / kTileRows;
+        int32_t mixed = 0, last = -1;
+        for (int32_t i = req_ptr[b]; i < req_ptr[b + 1]; ++i) {
+            const int64_t end = (int64_t)occ[i].dest_row - cache->row_base[b] + occ[i].m;
+            const int32_t tile = (int32_t)(end / kTileRows);
+            if (end % kTileRows != 0 && tile != last) {
+                ++mixed;
+                last = tile;
+            }
+        }
+        boundaries = boundaries || mixed > 0;
+        const double us = start_us + (clean_us * (tiles - mixed) + 11.5 * mixed) / split;
+        longest = std::max(longest, us);
+        mean += us / B;
+        keys += (double)tiles / B;
+        rows += cache->n_slots[b];
+    }
+    if (!boundaries) return true;
+    const double fused_us = 10.0 + std::max(longest, rounds * mean) + (split > 1 ? 8.0 : 0.0);
+    const int32_t splits = attn_splits(c, cache, L, n_suffix, false, &merge);
+    const double attn_us = splits > 1 ? keys / splits + 13.0 : rounds * (9.0 + key_us * keys);
+    const double bytes = 4.0 * L * rows * hkv * c->cfg.head_dim * c->eb;
+    return 6.0 + bytes / 6.7e6 + attn_us > 0.95 * fused_us;
+}
+
 // Suffix preparation and attention of a cache (arguments already checked).  With `fused`,
 // the cache is not written yet: the fused kernel reads the composed slots from the pool and
 // the suffix from k_suf / v_suf, turns the queries itself, and writes the whole cache
@@ -1161,7 +1205,8 @@ c2kv_status c2kv_compose_attend(c2kv_ctx* c, int32_t batch, const int32_t* req_p
         // The fused kernel takes pool-resident chunks on the tensor-core route, at most
         // kMaxFusedReq requests and at most kMaxFusedOcc occurrences; anything
         // else runs compose and then attention.  By default it runs only when one pair of
-        // query tiles covers each (layer, request, KV head).  With more pairs, forcing it
+        // query tiles covers each (layer, request, KV head), and where it is expected to be the
+        // faster (fused_pays).  With more pairs, forcing it
         // (C2KV_FUSE_ALWAYS) runs them in turn in one CTA per (layer, request, KV head), the
         // last pair first (it composes the cache), the others over the cache; with forced
         // key-range splits each pair's CTA composes its own tiles instead.  Neither beat
@@ -1182,6 +1227,7 @@ c2kv_status c2kv_compose_attend(c2kv_ctx* c, int32_t batch, const int32_t* req_p
         // PRE_ROPE slots turn by a position per slot, which the fused loaders' per-occurrence
         // angle tables do not hold: compose, then attend
         fuse = fuse && !host_chunks && c->cfg.storage == C2KV_STORAGE_LOCAL_ROPE;
+        fuse = fuse && (forced || fused_pays(c, cache, occ, req_ptr, n_suffix));
         cudaError_t e = cudaSuccess;
         // suffix tensors and outputs in pinned host memory: copied through device scratch (the
         // pipelined route does this per layer group itself)
