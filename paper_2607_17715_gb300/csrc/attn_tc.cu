@@ -130,7 +130,7 @@ static_assert(kSmemBytes <= 232448, "shared memory budget of one sm_100 CTA");
 // What depends on the head dimension D (128, or 64 in the plain kernel's instantiations
 // attn_tc64_*): a tile's bytes, its 64-channel swizzle blocks, the shared memory of a CTA.
 // kSplitP: P enters P.V as two bf16 terms, the rounded weight over the first 64 columns of
-// S_x and what the rounding left over the last 64 (relative error 2^-18 rather than 2^-9).
+// S_x and what the rounding left over the last 64 (relative error 2^-16 rather than 2^-8).
 // Heads of 64 channels were computed with fp32 weights on the CUDA cores and keep that
 // precision; at N = 64 the second term's MMAs cost as much as one tile's P.V does at 128.
 // Measured on 4 requests x 100 tokens x 1000 slots, 32 / 8 heads: the attend call 400 us on the
@@ -562,7 +562,10 @@ __device__ __forceinline__ PairSpan tile_span(const TcParams& P, int qt, int sp,
 // kO: the first TMEM column of O_A.  kDbl (x = 0): S and P alternate between two column blocks and
 // their barriers (B_SF, B_PF and the next ones); P.V(j - 1) may then still run when S(j) is read,
 // so a rescale of O waits for it (B_OE, one phase per P.V).
-template <bool kMerge, bool kSif = false, bool kKpp = false, int D = HD, uint32_t kO = kColO, bool kDbl = false>
+// kTwo: the weights as two bf16 terms (Geo::kSplitP; also a decode step that the CUDA cores would
+// compute with fp32 weights).
+template <bool kMerge, bool kSif = false, bool kKpp = false, int D = HD, uint32_t kO = kColO, bool kDbl = false,
+          bool kTwo = Geo<D>::kSplitP>
 __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, uint32_t sBar, int x,
                                             int quad, int lane, int t0, int l, int bl, int b,
                                             int hk, int sp, const PairSpan& span, uint32_t sf_base,
@@ -662,11 +665,11 @@ __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, u
         // P_j (bf16, keys 2c and 2c+1 packed in column c) over the first half of S_x
         const uint32_t p_addr = tmem + lane_addr + colS + dbl * BN;
         const float neg_m = -m_sub;
-        // (kSplitP: 16 keys at a time, their second terms over the last 64 columns)
-        constexpr int PW = Geo<D>::kSplitP ? 8 : 16;       // packed words per store
+        // (kTwo: 16 keys at a time, their second terms over the last 64 columns)
+        constexpr int PW = kTwo ? 8 : 16;       // packed words per store
 #pragma unroll
         for (int c = 0; c < 64 / PW; ++c) {
-            uint32_t pk[PW], pl[Geo<D>::kSplitP ? PW : 1];
+            uint32_t pk[PW], pl[kTwo ? PW : 1];
 #pragma unroll
             for (int w = 0; w < PW; ++w) {
                 const int e = 2 * (c * PW + w);            // key of the tile
@@ -676,10 +679,10 @@ __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, u
                 a1 = ex2(a1);
                 if (e & 2) fadd2(ps[2], ps[3], a0, a1); else fadd2(ps[0], ps[1], a0, a1);
                 pk[w] = pack_bf16(a0, a1);
-                if constexpr (Geo<D>::kSplitP)      // what the rounding left (exact differences)
+                if constexpr (kTwo)      // what the rounding left (exact differences)
                     pl[w] = pack_bf16(a0 - __uint_as_float(pk[w] << 16), a1 - __uint_as_float(pk[w] & 0xffff0000u));
             }
-            if constexpr (Geo<D>::kSplitP) {
+            if constexpr (kTwo) {
                 tmem_st8(p_addr + (uint32_t)(c * PW), pk);
                 tmem_st8(p_addr + 64u + (uint32_t)(c * PW), pl);
             } else {
@@ -1001,6 +1004,7 @@ __device__ __forceinline__ void mma_issuer(const TcParams& P, uint32_t tmem, uin
 // that one half's softmax overlaps the other's MMAs as two query tiles' do (warpgroup A merges
 // the halves at the end).  Issue order: S(0), S(1), then per key tile j: P(j).V(j), S(j + 2)
 // on the same half (in issue order after the P.V that reads the P it overwrites).
+template <bool kTwo>
 __device__ __forceinline__ void mma_issuer_kpp(const TcParams& P, uint32_t tmem, uint32_t sQ, uint32_t sK,
                                                uint32_t sV, uint32_t sBar, int n_kv, int q_ready,
                                                uint32_t q_par, RingState& st, bool wait_oe, uint32_t oe_par,
@@ -1050,6 +1054,11 @@ __device__ __forceinline__ void mma_issuer_kpp(const TcParams& P, uint32_t tmem,
         for (int kk = 0; kk < BN / 16; ++kk)
             mma_bf16_ts(x ? tO_b : tO_a, (x ? tS_b : tS_a) + (uint32_t)kk * 8u,
                         dv + (uint64_t)((kk * 2048) >> 4), idO, kk > 0 || j >= 2 ? 1u : 0u);
+        if constexpr (kTwo)               // the weights' second term, over the same V
+#pragma unroll
+            for (int kk = 0; kk < BN / 16; ++kk)
+                mma_bf16_ts(x ? tO_b : tO_a, (x ? tS_b : tS_a) + 64u + (uint32_t)kk * 8u,
+                            dv + (uint64_t)((kk * 2048) >> 4), idO, 1u);
         mma_commit(bar(B_VE + vs));
         vph ^= vs == VSTAGES - 1 ? 1u : 0u;
         vs = vs == VSTAGES - 1 ? 0 : vs + 1;
@@ -2048,7 +2057,7 @@ __device__ __forceinline__ void decode_append(const DecodeTcParams& X, int lane,
 // (TcParams::sif_k), a kernel of its own (attn_tc_sif_kernel) so that the plain kernel's code
 // stays as it is.
 // D: head dimension (64 in the plain and the SIF kernel only).
-template <bool kFused, bool kMulti, bool kSif, bool kKpp = false, int D = HD>
+template <bool kFused, bool kMulti, bool kSif, bool kKpp = false, int D = HD, bool kTwo = Geo<D>::kSplitP>
 __device__ __forceinline__ void attn_tc_body(const typename KernelParams<kFused, kKpp>::type& KP) {
     static_assert(D == HD || (!kFused && !kKpp), "64 channels: the plain and SIF kernels");
     constexpr int kTile = Geo<D>::kTile;
@@ -2209,7 +2218,7 @@ __device__ __forceinline__ void attn_tc_body(const typename KernelParams<kFused,
                     if (ps.has_b)
                         mma_issuer<true, D>(P, tmem, sQ, sK, sV, sBar, ps.n_kv, B_Q, q_par, st, pi > 0, oe_par, abort);
                     else if (kKpp)                                        // key tiles ping-pong (one pair)
-                        mma_issuer_kpp(P, tmem, sQ, sK, sV, sBar, ps.n_kv, B_QR, q_par, st, pi > 0, oe_par, abort);
+                        mma_issuer_kpp<kTwo>(P, tmem, sQ, sK, sV, sBar, ps.n_kv, B_QR, q_par, st, pi > 0, oe_par, abort);
                     else
                         mma_issuer<false, D>(P, tmem, sQ, sK, sV, sBar, ps.n_kv, B_Q, q_par, st, pi > 0, oe_par, abort);
                 }
@@ -2275,7 +2284,7 @@ __device__ __forceinline__ void attn_tc_body(const typename KernelParams<kFused,
                         decode_turn_queries(KP, (int)threadIdx.x - 128, (int64_t)P.req[bl].l_req + P.req[bl].t0, sQ,
                                             reinterpret_cast<float2*>(smem + TILE + 4096), sBar, abort);
                 if (x == 0 || ps.has_b || kpp) {
-                    softmax_tile<true, kSif, kKpp, D>(P, tmem, sBar, x, warp & 3, lane, x && !kpp ? ps.t0b : ps.t0a, l, bl,
+                    softmax_tile<true, kSif, kKpp, D, kColO, false, kTwo>(P, tmem, sBar, x, warp & 3, lane, x && !kpp ? ps.t0b : ps.t0a, l, bl,
                                  b, hk, sp, ps, done, (uint32_t)pi & 1u, p_count > 1, abort,
                                  pi == p_count - 1 ? sQ : 0u, kpp);
                     done += kpp ? (uint32_t)((ps.n_kv + 1 - x) / 2) : (uint32_t)ps.n_kv;
@@ -2327,8 +2336,10 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc64_sif_kernel(const __grid
 
 // Decode steps (AttnParams::key_pingpong): the plain kernel whose last pair, when it has one
 // query tile, splits its key tiles between the two softmax warpgroups.
+// kTwo: weights of two bf16 terms.
+template <bool kTwo>
 __global__ void __launch_bounds__(kThreads, 1) attn_tc_decode_kernel(const __grid_constant__ DecodeTcParams KP) {
-    attn_tc_body<false, false, false, true>(KP);
+    attn_tc_body<false, false, false, true, HD, kTwo>(KP);
 }
 
 // One query tile a CTA (the solo kernel), in two forms.
@@ -2573,7 +2584,7 @@ const void* tc_kernel_fn() {
     if constexpr (kSolo != 0) return reinterpret_cast<const void*>(&attn_solo_kernel<kSif, D, kSolo == 2>);
     else if constexpr (D == 64) return reinterpret_cast<const void*>(kSif ? &attn_tc64_sif_kernel : &attn_tc64_kernel);
     else if constexpr (kSif) return reinterpret_cast<const void*>(&attn_tc_sif_kernel);
-    else if constexpr (kKpp) return reinterpret_cast<const void*>(&attn_tc_decode_kernel);
+    else if constexpr (kKpp) return reinterpret_cast<const void*>(&attn_tc_decode_kernel<false>);
     else return reinterpret_cast<const void*>(&attn_tc_kernel<kFused, kMulti>);
 }
 
@@ -2924,6 +2935,11 @@ cudaError_t launch_attn_tc(const AttnParams& a, cudaStream_t s, Hook before) {
 cudaError_t launch_attn_tc_decode(const AttnParams& a, const DecodeAppend& d, cudaStream_t s, Hook before) {
     (void)cudaGetLastError();   // report this launch's error only, not a stale one
     if (!d.k_new || !d.v_new || !d.pos || a.d != HD) return cudaErrorInvalidValue;
+    if (d.two_terms) {
+        static const cudaError_t smem_err = cudaFuncSetAttribute(
+            attn_tc_decode_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+        if (smem_err != cudaSuccess) return smem_err;
+    }
     DecodeTcParams p;
     dim3 grid;
     cudaError_t e = prepare_tc<false, false, false, true>(a, p.t, grid);
@@ -2936,7 +2952,10 @@ cudaError_t launch_attn_tc_decode(const AttnParams& a, const DecodeAppend& d, cu
     std::memcpy(p.pad_mask, d.pad_mask, sizeof(p.pad_mask));
     p.rope = d.rope;
     before();
-    attn_tc_decode_kernel<<<grid, kThreads, kSmemBytes, s>>>(p);
+    if (d.two_terms)
+        attn_tc_decode_kernel<true><<<grid, kThreads, kSmemBytes, s>>>(p);
+    else
+        attn_tc_decode_kernel<false><<<grid, kThreads, kSmemBytes, s>>>(p);
     return cudaGetLastError();
 }
 

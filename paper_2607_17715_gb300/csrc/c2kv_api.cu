@@ -1372,16 +1372,21 @@ c2kv_status c2kv_decode(c2kv_ctx* c, c2kv_cache* cache, int32_t layer, const voi
         // bf16, d 128: the tensor-core attention kernel with the new token as a one-row
         // suffix at suffix index steps[r] (its 128-row query tile holds G live rows: the MMA
         // has time to spare, and its pipeline streams K and V at the rate of HBM) when its
-        // one CTA per SM covers the units in one wave or their key ranges are long; otherwise
-        // (short contexts over more units than SMs: its per-CTA start would be paid twice)
-        // the CUDA-core decode kernel, two CTAs per SM.  Measured on a GB300: Llama-3-8B
-        // layer, 32 layers x 1 request, 1360 keys: 45 us CUDA cores, 52 us tensor cores;
-        // 16 requests x 1160 keys: 31 / 28 us; 2 x 2300 keys, G = 8: 26 / 19 us; 8 x 32900
-        // keys: 212 / 192 us.
+        // one CTA per SM covers the units in one wave or their key ranges are long.  Otherwise
+        // (short contexts over more units than SMs: its per-CTA start is paid again each wave)
+        // the CUDA-core decode kernel, two CTAs per SM, while a group is small: its time grows with
+        // the G queries that each key meets, the tensor cores' does not, so at G = 8 these take it
+        // from 3 key tiles as well, with weights of two bf16 terms in place of its fp32 ones.
+        // Measured, CUDA cores / tensor cores with two terms (us a call, one layer, 8 KV heads; key
+        // tiles 3, 9, 18): G = 8, 32 requests 30 / 24, 71 / 43, 123 / 69, 128 requests 88 / 76, 226 /
+        // 136, 405 / 226, but one tile 53 / 59; G = 4, 32 requests 9 tiles 39 / 43, 18 65 / 69 (with one
+        // term 36 and 57).  One term, one wave: 16 requests x 1160 keys 30 / 18, 8 x 32900 212 / 190.
         const int64_t tiles_max = (n_keys_max + 127) / 128;
-        const bool use_tc = c->cfg.attn_impl != C2KV_ATTN_SIMT &&
-                            c2kv::attn_tc_supported(c->cfg.dtype, d, hq, hkv) &&
-                            (c->cfg.attn_impl == C2KV_ATTN_TC || units <= c->sms || tiles_max >= 32);
+        const int32_t group = hq / hkv;
+        const bool tc = c->cfg.attn_impl != C2KV_ATTN_SIMT && c2kv::attn_tc_supported(c->cfg.dtype, d, hq, hkv);
+        const bool one_term = c->cfg.attn_impl == C2KV_ATTN_TC || units <= c->sms || tiles_max >= 32;
+        const bool two_terms = tc && !one_term && group >= 8 && tiles_max >= 3;
+        const bool use_tc = tc && (one_term || two_terms);
         int32_t n_split = 1;
         if (use_tc) {
             // splits per (layer, request, KV head): the fewest waves of one-CTA-per-SM work,
@@ -1497,6 +1502,7 @@ c2kv_status c2kv_decode(c2kv_ctx* c, c2kv_cache* cache, int32_t layer, const voi
                 ap.v_new = v_new;
                 ap.pos = cache->pos;
                 ap.rope = c->turns;
+                ap.two_terms = two_terms ? 1 : 0;
                 for (int32_t i = 0; i < nb; ++i)
                     if (pad_from[b0 + i] < edge[b0 + i]) ap.pad_mask[i / 32] |= 1u << (i % 32);
                 ProfScope prof_decode(c, C2KV_PROF_DECODE, true);
