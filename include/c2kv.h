@@ -59,7 +59,7 @@ typedef int32_t c2kv_status;
 #define C2KV_MODE_HOST     3  /* stored-form slots that stay in pinned host memory (no copy)   */
 
 /* c2kv_attend kernel choice */
-#define C2KV_ATTN_AUTO   0    /* tensor-core kernel where it applies, SIMT otherwise */
+#define C2KV_ATTN_AUTO   0    /* tensor-core kernels where they apply (also d = 64), else SIMT */
 #define C2KV_ATTN_SIMT   1    /* CUDA-core fp32-accumulate kernel (any dtype)        */
 #define C2KV_ATTN_TC     2    /* tcgen05 / TMEM tensor-core kernel (bf16, d = 128)    */
 
@@ -95,13 +95,13 @@ typedef struct c2kv_config {
     int32_t attn_impl;         /* C2KV_ATTN_AUTO / _SIMT / _TC                                */
     int32_t attn_split;        /* tensor-core attention key-range splits per work unit:
                                   0 = chosen per call (split only when the units would leave
-                                  most SMs idle), 1 = never, n <= 16 = always n (partials
+                                  SMs idle), 1 = never, n <= 16 = always n (partials
                                   merged by an exact log-sum-exp combine)                     */
     int32_t fuse;              /* C2KV_FUSE_AUTO / _NEVER / _ALWAYS (c2kv_compose_attend)     */
     int32_t storage;           /* C2KV_STORAGE_LOCAL_ROPE (0) or C2KV_STORAGE_PRE_ROPE          */
     int32_t attn_pairs;        /* pairs of 128-row query tiles one tensor-core attention CTA
-                                  runs in turn: 0 = chosen per launch (several only when the
-                                  launch is many waves of CTAs), n >= 1 = n (fewer where a
+                                  runs in turn: 0 = chosen per launch (several only where
+                                  that saves a wave of CTAs), n >= 1 = n (fewer where a
                                   (layer, request, KV head) has fewer pairs)                  */
 } c2kv_config;
 
@@ -272,7 +272,9 @@ c2kv_status c2kv_attend(c2kv_ctx* ctx, c2kv_cache* cache, int32_t layer, const v
  * that reading one group over the host link overlaps the attention of the previous one (on
  * a second stream).  Either way the call's work ends on the context's stream.  The context's `fuse` setting chooses (C2KV_FUSE_*): by
  * default the fused kernel runs when each (layer, request, KV head) has one pair of query
- * tiles.  The cache is returned as by c2kv_compose (release it with c2kv_cache_release) and
+ * tiles, unless chunks that do not fill 128-row tiles leave a boundary in so many of them
+ * that the other route is faster (the same bits either way where the keys are not split).
+ * The cache is returned as by c2kv_compose (release it with c2kv_cache_release) and
  * serves later c2kv_decode / c2kv_attend calls.
  *
  *   batch, req_ptr, chunk_ids, positions, suffix_capacity : as c2kv_compose.
@@ -349,7 +351,8 @@ c2kv_status c2kv_attend_noalloc(c2kv_ctx* ctx, c2kv_cache* cache, int32_t layer,
  * kernel); the split buffer comes from the context's memory pool.  With bf16
  * and d = 128 the step runs on the tensor-core attention kernel (the new token as a one-row
  * query tile) when (layers x requests x KV heads) fits one CTA per SM or a request holds
- * 4096 keys or more, else on a CUDA-core decode kernel (C2KV_ATTN_TC forces the former,
+ * more than 31 x 128 keys, or, with each softmax weight as two bf16 terms, when G = 8 and a
+ * request holds more than 2 x 128; else on a CUDA-core decode kernel (C2KV_ATTN_TC forces the former,
  * C2KV_ATTN_SIMT the latter).
  * The tensor-core route reads whole 128-row key tiles, so it zeroes the rows after the new
  * one up to the next 128-row boundary that no earlier call on this cache has written or
@@ -375,7 +378,7 @@ c2kv_status c2kv_decode(c2kv_ctx* ctx, c2kv_cache* cache, int32_t layer, const v
  * The sink block, B(0) in the paper's 1-based numbering, is read as the first block
  * [0, min(k, n)).  The trained C2 embeddings and QKV projections that produce q, k, v for
  * the C2 tokens are the caller's; this is the attention operator they feed.  On the
- * tensor-core route (bf16, d 128) the C2 rows' launch runs on the context's second stream
+ * tensor-core route (bf16) the C2 rows' launch runs on the context's second stream
  * beside the document rows' attention; the call's work ends on the context's stream.
  *
  *   n_layers : layers in the tensors (each processed independently).

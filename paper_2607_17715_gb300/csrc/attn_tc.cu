@@ -53,6 +53,10 @@
 // with the rows' positions, so the cache is complete for later decode steps.  The pool is
 // read once per (layer, request, KV head) and the composed cache written once, rather than
 // written by compose and read back by attention.
+//
+// Other forms: heads of 64 channels (Geo<64>); one query tile a CTA (attn_solo_kernel); a decode step
+// (attn_tc_decode_kernel: one query row, its key tiles split between the two halves of tensor memory,
+// the new token's rows appended by the kernel).
 #include <cuda.h>
 #include <cudaTypedefs.h>
 

@@ -15,7 +15,7 @@
 // context dtype like every cached activation), or extract_rope_k_kernel K alone where the attention
 // turns the queries itself.  The masked attention then takes one of two routes.
 //
-// Tensor cores (bf16, the group sizes attn_tc_kernel takes).  The mask splits into
+// Tensor cores (bf16, the group sizes the tensor-core kernels take).  The mask splits into
 // pieces the suffix-attention kernel already computes:
 //   1. document rows: plain causal attention over document keys 0..t, i.e. a "suffix" of n
 //      tokens over an empty prefix;
@@ -23,7 +23,7 @@
 //      c_0 .. c_j causally; the kernel's SIF mode (sif_k = k) masks every document key but
 //      those of the sink block and B(j), and visits only the key tiles that hold them (for
 //      a pair of 2 x 128 packed rows: its blocks' tiles, tile 0, the C2 tiles).
-// Both are launches of attn_tc_kernel with a token pitch of n + m, so they read and write
+// Both are launches of attn_solo_kernel (or the pair kernel) with a token pitch of n + m, so they read and write
 // the extraction layout in place.
 //
 // CUDA cores (fp32, other group sizes): extract_attn_kernel runs every row with fp32
@@ -81,8 +81,9 @@ __global__ void __launch_bounds__(256) extract_rope_kernel(const __grid_constant
 // K alone, and the table of every token's (cos, sin) from which the solo attention kernel turns its
 // query tiles in shared memory.  Turning Q here read and wrote four fifths of the tensors' bytes
 // (Q is Hq / Hkv times K): 68 us of the 32-layer call on 512 + 128 tokens, against 49 us for those
-// bytes at the rate of HBM; the call went from 226 to 200 us.  A CTA takes kRopeTokens tokens of one layer, each thread one (token, head,
-// vector pair) at a time, its loads issued before the angles are formed.
+// bytes at the rate of HBM; the call went from 226 to 200 us.  A CTA takes kRopeTokens tokens of one
+// layer, each thread one (token, head, vector pair) at a time, its loads issued before the angles are
+// formed.
 constexpr int kRopeTokens = 4;
 template <typename T, int VPH>
 __global__ void __launch_bounds__(256) extract_rope_k_kernel(const __grid_constant__ ExtractParams P) {
