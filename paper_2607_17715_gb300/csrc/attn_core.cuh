@@ -131,7 +131,11 @@ template <typename T, int D, int RT, class Job>
 __device__ __forceinline__ void attention_core(const Job& job, int row0, int ns, int rank, uint8_t* sm) {
     using L = Core<D, RT>;
     constexpr int H = D / 32;                              // 4-channel groups a lane
-    constexpr int kBlk = 32;                               // channels per folded partial
+    // channels per folded partial sum.  (16, and the scale in the exponent's fused multiply-add: the
+    // error against 64 bits is that of the earlier kernel's four interleaved sums, 2e-7 to 5e-7 of the
+    // largest output over 32 to 8192 keys; with 32 and a rounded product it was up to a third above it,
+    // and no faster.)
+    constexpr int kBlk = 16;
     const int tid = threadIdx.x, lane = tid & 31, ty = lane >> 3, tx = lane & 7;
     const int r0 = (tid >> 5) * 4 * RT + ty;               // this lane's rows r0 + 4 i
     const int tiles = (job.nkeys + kCoreKeys - 1) / kCoreKeys;
@@ -218,8 +222,6 @@ __device__ __forceinline__ void attention_core(const Job& job, int row0, int ns,
         float alpha[RT];
 #pragma unroll
         for (int i = 0; i < RT; ++i) {
-#pragma unroll
-            for (int j = 0; j < 8; ++j) s[i][j] *= job.scale_log2;
             if (!whole) {
                 const auto row = job.row(row0 + r0 + 4 * i);
 #pragma unroll
@@ -233,12 +235,12 @@ __device__ __forceinline__ void attention_core(const Job& job, int row0, int ns,
             for (int j = 1; j < 8; ++j) mx = fmaxf(mx, s[i][j]);
 #pragma unroll
             for (int off = 4; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-            const float mn = fmaxf(m[i], mx);
+            const float mn = fmaxf(m[i], mx * job.scale_log2);
             const float ms = mn == -CUDART_INF_F ? 0.f : mn;      // nothing visible yet
             alpha[i] = exp2f(m[i] - ms);
             m[i] = mn;
 #pragma unroll
-            for (int j = 0; j < 8; ++j) s[i][j] = exp2f(s[i][j] - ms);
+            for (int j = 0; j < 8; ++j) s[i][j] = exp2f(fmaf(s[i][j], job.scale_log2, -ms));
             l[i] = l[i] * alpha[i] + (((s[i][0] + s[i][1]) + (s[i][2] + s[i][3])) +
                                       ((s[i][4] + s[i][5]) + (s[i][6] + s[i][7])));   // this lane's keys
         }
