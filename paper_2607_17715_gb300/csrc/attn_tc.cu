@@ -2894,7 +2894,9 @@ cudaError_t launch_plain(const AttnParams& a, cudaStream_t s, Hook before) {
 // 60 % from 512 to 4096 tokens; suffixes of 64 and 200 tokens over 5 to 17 key tiles solo by 2 to
 // 24 % while the pairs are at most half the SMs, or a (layer, request, KV head) has a single query
 // tile, or few key tiles (256 pairs of 3: 38 / 36, of 5: 44 / 42), and the pair kernel by 2 to 7 %
-// (and 13 % over 257 key tiles) when 77 pairs or more share their K/V tiles.
+// (and 13 % over 257 key tiles) when 77 pairs or more share their K/V tiles, unless two tiles an SM
+// take fewer rounds than a pair an SM (an odd number of tiles a head: 640 pairs of 7 tiles 131 / 114, 512
+// of 3 tiles 92.6 / 82.2; with as many rounds, 384 of 7 tiles 83.6 / 82.4, 256 of 3 tiles 60 / 64).
 enum class SoloChoice { kPair, kShared, kAlone };
 SoloChoice solo_choice(const AttnParams& a) {
     if (a.key_pingpong || a.pairs_per_cta != 0 || a.tickets != nullptr) return SoloChoice::kPair;
@@ -2914,7 +2916,10 @@ SoloChoice solo_choice(const AttnParams& a) {
     for (int i = 0; i < a.batch; ++i) slots = std::max(slots, a.req[i].n_slots);
     const int tiles = (slots + a.sq + BN - 1) / BN;
     const bool causal_only = slots == 0;             // extraction document rows
-    if (causal_only || tiles <= 6 || 2 * ((per_head + 1) / 2 * heads) <= sms) return SoloChoice::kShared;
+    const int64_t pairs = (per_head + 1) / 2 * heads;
+    if (causal_only || tiles <= 6 || 2 * pairs <= sms) return SoloChoice::kShared;
+    // an odd number of query tiles: half of each head's last pair is empty
+    if ((units + 2 * sms - 1) / (2 * sms) < (pairs + sms - 1) / sms) return SoloChoice::kShared;
     return SoloChoice::kPair;
 }
 template <bool kSif, int D>

@@ -1,5 +1,5 @@
-"""How many query-tile pairs a CTA of the pair kernel runs in turn (chosen by the rounds of CTAs that
-it saves) does not change a bit of the result."""
+"""How many query-tile pairs a CTA of the pair kernel runs in turn, or two CTAs of one tile an SM
+(chosen by the rounds of CTAs that they save), does not change a bit of the result."""
 import pytest
 import torch
 
@@ -15,6 +15,7 @@ L8B = synth.scaled(synth.workload("llama8b"), layers=1, chunks_per_request=1)
     (32, 16, 128),     # 256 pairs: both of a head in turn
     (32, 24, 100),     # 384: one a CTA, the last with one part-full tile
     (64, 8, 120),      # 256, four a head: two in turn
+    (32, 20, 200),     # 7 tiles a head, 640 pairs: 5 rounds; one tile a CTA, 4
 ])
 def test_same_bits_for_any_number_in_turn(hq, batch, sq):
     c2kv = H.lib()
