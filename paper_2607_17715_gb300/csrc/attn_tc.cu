@@ -2830,10 +2830,13 @@ cudaError_t prepare_tc(const AttnParams& a, TcParams& p, dim3& grid) {
         const int64_t cols = (int64_t)a.hkv * a.lq * a.batch;
         int slots = 0;
         for (int i = 0; i < a.batch; ++i) slots = std::max(slots, a.req[i].n_slots + a.req[i].t0);
-        const double pair_us = 8.0 + 1.6 * ((slots + a.sq + BN - 1) / BN);
+        const int key_tiles = (slots + a.sq + BN - 1) / BN;
+        const double pair_us = 8.0 + 1.6 * key_tiles;
+        const double short_us = ((a.sq + tq - 1) / tq) % 2 == 1 ? 0.6 * key_tiles : 0.0;   // the last pair's one tile
         double best = 0.0;
         for (int64_t n = 1; n <= std::min<int64_t>(pairs, 16); ++n) {
-            const double us = (double)(((pairs + n - 1) / n * cols + sms - 1) / sms) * (1.5 + (double)n * pair_us);
+            const double us = (double)(((pairs + n - 1) / n * cols + sms - 1) / sms) *
+                              (1.5 + (double)n * pair_us - (n == pairs && n > 1 ? short_us : 0.0));
             if (n == 1 || us < 0.985 * best) {
                 best = us;
                 pg = n;
