@@ -495,10 +495,13 @@ def extract_line(wl, world, ms, kernel_ms, hbm, bf16, src):
 
 def decode_on_tensor_cores(wl, keys_per_request, sms=152):
     """The decode route c2kv_decode takes for this shape (its rule: the tensor-core kernel for
-    bf16 at head_dim 128 when the (layer, request, KV head) units fit in one wave of SMs or a
-    request has at least 32 key tiles; the CUDA-core kernel otherwise)."""
+    bf16 at head_dim 128 when the (layer, request, KV head) units fit in one wave of SMs, or a
+    request has at least 32 key tiles, or 3 with eight queries a KV head; the CUDA-core kernel
+    otherwise)."""
     units = wl.layers * wl.batch * wl.n_kv_heads
-    return wl.dtype == "bf16" and wl.head_dim == 128 and (units <= sms or keys_per_request >= 32 * 128)
+    tiles = -(-int(keys_per_request) // 128)
+    return wl.dtype == "bf16" and wl.head_dim == 128 and (
+        units <= sms or tiles >= 32 or (wl.n_q_heads // wl.n_kv_heads >= 8 and tiles >= 3))
 
 
 def decode_line(wl, world, dec_ms, dec_kernel_ms, dec_keys, hbm, src):
