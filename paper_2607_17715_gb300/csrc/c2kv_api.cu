@@ -777,11 +777,13 @@ cudaError_t suffix_run(c2kv_ctx* c, const c2kv_cache* cache, int32_t layer0, int
 
 // Key-range splits of an attend launch on the tensor cores (`merge_launch`: partials merged by a
 // launch of their own rather than in the kernel).  When the query tiles leave SMs idle, each one's
-// key tiles may be split, as far as the SMs go, by a model of the call (us): a key tile takes about
-// 1, a CTA 8 to start and end, the merge launch 5 and its partials' bytes both ways at 5 TB/s.
+// key tiles may be split, as far as two CTAs an SM go, by a model of the call (us): a key tile takes
+// about 1 for a CTA alone on its SM and 1.95 for two sharing it, a CTA 8 to start and end, the merge
+// launch 5 and its partials' bytes both ways at 5 TB/s.
 // (The merge in the kernel, by the last CTA of a unit alone, costs about 0.25 a row: with 256 rows a
 // unit it had made 2 requests x 200 tokens over 16 chunks 103 us a call, now 29.)  Measured, one
-// layer, 32 / 8 heads: 64 tokens over 10 chunks 28.9 -> 16 us, over 64 chunks 43 -> 24.
+// layer, 32 / 8 heads: 64 tokens over 10 chunks 28.9 -> 16 us, over 64 chunks 43 -> 24; 96 query tiles
+// of 257 key tiles, three splits two an SM, 260 -> 181 (two splits 255).
 int32_t attn_splits(const c2kv_ctx* c, const c2kv_cache* cache, int32_t lq, int32_t n_suffix, bool fused,
                     bool* merge_launch) {
     *merge_launch = fused;
@@ -800,8 +802,8 @@ int32_t attn_splits(const c2kv_ctx* c, const c2kv_cache* cache, int32_t lq, int3
     const double rows = (double)lq * cache->batch * n_suffix * c->cfg.n_q_heads;
     int32_t best = 1;
     double cost = tiles * 1.0 + 8.0;
-    for (int32_t n = 2; n <= 16 && n * units <= c->sms && n <= tiles; ++n) {
-        const double t = (tiles + n - 1) / n * 1.0 + 8.0 + 5.0 + n * rows * (c->cfg.head_dim + 1) * 8.0 / 5.0e6;
+    for (int32_t n = 2; n <= 16 && n * units <= 2 * c->sms && n <= tiles; ++n) {
+        const double t = (tiles + n - 1) / n * (n * units <= c->sms ? 1.0 : 1.95) + 8.0 + 5.0 + n * rows * (c->cfg.head_dim + 1) * 8.0 / 5.0e6;
         if (t < 0.95 * cost) {
             cost = t;
             best = n;
