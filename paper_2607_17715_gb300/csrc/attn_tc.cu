@@ -133,21 +133,28 @@ static_assert(kSmemBytes <= 232448, "shared memory budget of one sm_100 CTA");
 
 // What depends on the head dimension D (128, or 64 in the plain kernel's instantiations
 // attn_tc64_*): a tile's bytes, its 64-channel swizzle blocks, the shared memory of a CTA.
-// kSplitP: P enters P.V as two bf16 terms, the rounded weight over the first 64 columns of
-// S_x and what the rounding left over the last 64 (relative error 2^-16 rather than 2^-8).
-// Heads of 64 channels were computed with fp32 weights on the CUDA cores and keep that
-// precision; at N = 64 the second term's MMAs cost as much as one tile's P.V does at 128.
-// Measured on 4 requests x 100 tokens x 1000 slots, 32 / 8 heads: the attend call 400 us on the
-// CUDA cores, 30.2 us here, 0.0017 off the 64-bit result either way (64 CTAs of 9 key tiles:
-// bound by the softmax chain of a CTA and its start, not by the tensor cores).
+// kTerms: the bf16 terms that a weight enters P.V as.  Heads of 64 channels keep fp32 weights, as
+// the CUDA cores take them: the weight's leading 8 bits (over the first 64 columns of S_x), the
+// next 8 (over the last 64) and the last 8 (over 64 columns of their own, kThirdTerm): each term
+// is a bf16 value, and the sum of the three is the fp32 weight itself.  At N = 64 the three terms'
+// MMAs cost 1.5 times one tile's P.V at 128.
+// Measured on 4 requests x 100 tokens x 1000 slots, 32 / 8 heads (64 query tiles of 9 key tiles):
+// the attend call 400 us on the CUDA cores, 25 us here (20.9 with two terms, 16 bits: the third's
+// MMAs and stores are 2 us each), 0.0017 off the 64-bit result either way.  A CTA is bound by the
+// chain softmax, P.V, S of its tiles and its start, not by the tensor cores' rate.
 template <int D>
 struct Geo {
     static constexpr int kTile = BN * D * 2;
     static constexpr int kBlocks = D / 64;
-    static constexpr bool kSplitP = D == 64;
+    static constexpr int kTerms = D == 64 ? 3 : 1;
     static constexpr size_t kSmem = 1024 + (size_t)kTile * kSmemTiles + 8 * NBAR + 16;
 };
 static_assert(Geo<HD>::kTile == TILE && Geo<HD>::kSmem == kSmemBytes, "the fused kernel's layout");
+// The third term's columns, 64 for each S block (two, or the shared solo kernel's one), after the
+// O blocks of 64 columns that begin at column kO.
+template <uint32_t kO>
+constexpr uint32_t kThirdTerm = kO + (kO == kColO ? 128 : 64);
+static_assert(kThirdTerm<kColO> + 2 * 64 <= kTmemCols, "tensor memory of the 64-channel kernels");
 
 struct TcParams {                // CUtensorMap members carry their own alignment
     CUtensorMap tm_q;        // q_rot   [Lq*Btot][Sq'][Hq][128] box {64, G, TQ, 1}; Sq' = sq_pitch
@@ -320,6 +327,12 @@ __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&v)[8])
                  : "memory");
 }
 
+__device__ __forceinline__ void tmem_st4(uint32_t taddr, const uint32_t (&v)[4]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr), "r"(v[0]), "r"(v[1]),
+                 "r"(v[2]), "r"(v[3])
+                 : "memory");
+}
+
 __device__ __forceinline__ void tmem_ld_wait() {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
@@ -361,6 +374,13 @@ __device__ __forceinline__ void fadd2(float& d0, float& d1, float a0, float a1) 
         "mov.b64 {%0, %1}, pd;\n\t}"
         : "+f"(d0), "+f"(d1)
         : "f"(a0), "f"(a1));
+}
+
+// The leading 8 significant bits of (a0, a1) as packed bf16; a0 and a1 keep the rest (exactly).
+__device__ __forceinline__ uint32_t cut_bf16(float& a0, float& a1) {
+    const uint32_t u0 = __float_as_uint(a0), u1 = __float_as_uint(a1);
+    fadd2(a0, a1, -__uint_as_float(u0 & 0xffff0000u), -__uint_as_float(u1 & 0xffff0000u));
+    return __byte_perm(u0, u1, 0x7632);
 }
 
 __device__ __forceinline__ float fmax3(float a, float b, float c) {
@@ -566,10 +586,10 @@ __device__ __forceinline__ PairSpan tile_span(const TcParams& P, int qt, int sp,
 // kO: the first TMEM column of O_A.  kDbl (x = 0): S and P alternate between two column blocks and
 // their barriers (B_SF, B_PF and the next ones); P.V(j - 1) may then still run when S(j) is read,
 // so a rescale of O waits for it (B_OE, one phase per P.V).
-// kTwo: the weights as two bf16 terms (Geo::kSplitP; also a decode step that the CUDA cores would
+// kTerms: bf16 terms of a weight (Geo::kTerms; two for a decode step that the CUDA cores would
 // compute with fp32 weights).
 template <bool kMerge, bool kSif = false, bool kKpp = false, int D = HD, uint32_t kO = kColO, bool kDbl = false,
-          bool kTwo = Geo<D>::kSplitP>
+          int kTerms = Geo<D>::kTerms>
 __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, uint32_t sBar, int x,
                                             int quad, int lane, int t0, int l, int bl, int b,
                                             int hk, int sp, const PairSpan& span, uint32_t sf_base,
@@ -669,11 +689,11 @@ __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, u
         // P_j (bf16, keys 2c and 2c+1 packed in column c) over the first half of S_x
         const uint32_t p_addr = tmem + lane_addr + colS + dbl * BN;
         const float neg_m = -m_sub;
-        // (kTwo: 16 keys at a time, their second terms over the last 64 columns)
-        constexpr int PW = kTwo ? 8 : 16;       // packed words per store
+        // (several terms: 16 keys at a time, the second over the last 64 columns)
+        constexpr int PW = kTerms == 3 ? 4 : kTerms == 2 ? 8 : 16;       // packed words per store
 #pragma unroll
         for (int c = 0; c < 64 / PW; ++c) {
-            uint32_t pk[PW], pl[kTwo ? PW : 1];
+            uint32_t pk[PW], p2[kTerms > 1 ? PW : 1], p3[kTerms > 2 ? PW : 1];
 #pragma unroll
             for (int w = 0; w < PW; ++w) {
                 const int e = 2 * (c * PW + w);            // key of the tile
@@ -682,13 +702,23 @@ __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, u
                 a0 = ex2(a0);
                 a1 = ex2(a1);
                 if (e & 2) fadd2(ps[2], ps[3], a0, a1); else fadd2(ps[0], ps[1], a0, a1);
-                pk[w] = pack_bf16(a0, a1);
-                if constexpr (kTwo)      // what the rounding left (exact differences)
-                    pl[w] = pack_bf16(a0 - __uint_as_float(pk[w] << 16), a1 - __uint_as_float(pk[w] & 0xffff0000u));
+                if constexpr (kTerms == 3) {     // the top 8 bits of what is left, three times
+                    pk[w] = cut_bf16(a0, a1);
+                    p2[w] = cut_bf16(a0, a1);
+                    p3[w] = cut_bf16(a0, a1);
+                } else {
+                    pk[w] = pack_bf16(a0, a1);
+                    if constexpr (kTerms == 2)   // what the rounding left (exact differences)
+                        p2[w] = pack_bf16(a0 - __uint_as_float(pk[w] << 16), a1 - __uint_as_float(pk[w] & 0xffff0000u));
+                }
             }
-            if constexpr (kTwo) {
+            if constexpr (kTerms == 3) {
+                tmem_st4(p_addr + (uint32_t)(c * PW), pk);
+                tmem_st4(p_addr + 64u + (uint32_t)(c * PW), p2);
+                tmem_st4(tmem + lane_addr + kThirdTerm<kO> + ((uint32_t)x + dbl) * 64u + (uint32_t)(c * PW), p3);
+            } else if constexpr (kTerms == 2) {
                 tmem_st8(p_addr + (uint32_t)(c * PW), pk);
-                tmem_st8(p_addr + 64u + (uint32_t)(c * PW), pl);
+                tmem_st8(p_addr + 64u + (uint32_t)(c * PW), p2);
             } else {
                 tmem_st16(p_addr + (uint32_t)(c * PW), pk);
             }
@@ -912,17 +942,22 @@ __device__ __forceinline__ void mma_issuer(const TcParams& P, uint32_t tmem, uin
         }
     };
     // O += P V with P (bf16 pairs) from TMEM: 16 keys (8 columns) per step; the first step
-    // of the first block overwrites O
+    // of the first block overwrites O.  p3: the third term's columns (64 channels)
     constexpr int kKeyStep = 16 * 128;      // bytes of 16 keys' rows in a 64-channel block
-    auto pv_block = [&](uint32_t p, uint64_t dv, uint32_t o, uint32_t acc0) {
+    const uint32_t tP3_a = tmem + kThirdTerm<kColO>, tP3_b = tP3_a + 64u;
+    auto pv_block = [&](uint32_t p, uint32_t p3, uint64_t dv, uint32_t o, uint32_t acc0) {
 #pragma unroll
         for (int kk = 0; kk < BN / 16; ++kk)
             mma_bf16_ts(o, p + (uint32_t)kk * 8u, dv + (uint64_t)((kk * kKeyStep) >> 4), idO,
                         kk > 0 ? 1u : acc0);
-        if constexpr (Geo<D>::kSplitP)      // the weights' second term, over the same V
+        if constexpr (Geo<D>::kTerms == 3) {      // the weights' other terms, over the same V
 #pragma unroll
             for (int kk = 0; kk < BN / 16; ++kk)
                 mma_bf16_ts(o, p + 64u + (uint32_t)kk * 8u, dv + (uint64_t)((kk * kKeyStep) >> 4), idO, 1u);
+#pragma unroll
+            for (int kk = 0; kk < BN / 16; ++kk)
+                mma_bf16_ts(o, p3 + (uint32_t)kk * 8u, dv + (uint64_t)((kk * kKeyStep) >> 4), idO, 1u);
+        }
     };
     auto wait = [&](int i, uint32_t parity) {
         mbar_wait(bar(i), parity, P.err, abort);
@@ -948,13 +983,13 @@ __device__ __forceinline__ void mma_issuer(const TcParams& P, uint32_t tmem, uin
         wait(B_PF + 0, ppa);
         wait(B_VF + st.vs, st.vph);
         if (oe) wait(B_OE, oe_par);
-        pv_block(tS_a, dv, tO_a, acc0);
+        pv_block(tS_a, tP3_a, dv, tO_a, acc0);
         wait(B_KF + st.ks, st.kph);
         s_block(dQa, dk, tS_a);
         mma_commit(bar(B_SF + 0));
         if (kHasB) {
             wait(B_PF + 1, ppb);
-            pv_block(tS_b, dv, tO_b, acc0);
+            pv_block(tS_b, tP3_b, dv, tO_b, acc0);
         }
         mma_commit(bar(B_VE + st.vs));
         if (kHasB) {
@@ -990,10 +1025,10 @@ __device__ __forceinline__ void mma_issuer(const TcParams& P, uint32_t tmem, uin
     wait(B_PF + 0, (st.pa + (uint32_t)n_kv - 1u) & 1u);
     wait(B_VF + st.vs, st.vph);
     if (wait_oe && n_kv == 1) wait(B_OE, oe_par);
-    pv_block(tS_a, dvl, tO_a, acc0);
+    pv_block(tS_a, tP3_a, dvl, tO_a, acc0);
     if (kHasB) {
         wait(B_PF + 1, (st.pb + (uint32_t)n_kv - 1u) & 1u);
-        pv_block(tS_b, dvl, tO_b, acc0);
+        pv_block(tS_b, tP3_b, dvl, tO_b, acc0);
     }
     mma_commit(bar(B_VE + st.vs));
     next_v();
@@ -2061,7 +2096,7 @@ __device__ __forceinline__ void decode_append(const DecodeTcParams& X, int lane,
 // (TcParams::sif_k), a kernel of its own (attn_tc_sif_kernel) so that the plain kernel's code
 // stays as it is.
 // D: head dimension (64 in the plain and the SIF kernel only).
-template <bool kFused, bool kMulti, bool kSif, bool kKpp = false, int D = HD, bool kTwo = Geo<D>::kSplitP>
+template <bool kFused, bool kMulti, bool kSif, bool kKpp = false, int D = HD, int kTerms = Geo<D>::kTerms>
 __device__ __forceinline__ void attn_tc_body(const typename KernelParams<kFused, kKpp>::type& KP) {
     static_assert(D == HD || (!kFused && !kKpp), "64 channels: the plain and SIF kernels");
     constexpr int kTile = Geo<D>::kTile;
@@ -2222,7 +2257,7 @@ __device__ __forceinline__ void attn_tc_body(const typename KernelParams<kFused,
                     if (ps.has_b)
                         mma_issuer<true, D>(P, tmem, sQ, sK, sV, sBar, ps.n_kv, B_Q, q_par, st, pi > 0, oe_par, abort);
                     else if (kKpp)                                        // key tiles ping-pong (one pair)
-                        mma_issuer_kpp<kTwo>(P, tmem, sQ, sK, sV, sBar, ps.n_kv, B_QR, q_par, st, pi > 0, oe_par, abort);
+                        mma_issuer_kpp<(kTerms > 1)>(P, tmem, sQ, sK, sV, sBar, ps.n_kv, B_QR, q_par, st, pi > 0, oe_par, abort);
                     else
                         mma_issuer<false, D>(P, tmem, sQ, sK, sV, sBar, ps.n_kv, B_Q, q_par, st, pi > 0, oe_par, abort);
                 }
@@ -2288,7 +2323,7 @@ __device__ __forceinline__ void attn_tc_body(const typename KernelParams<kFused,
                         decode_turn_queries(KP, (int)threadIdx.x - 128, (int64_t)P.req[bl].l_req + P.req[bl].t0, sQ,
                                             reinterpret_cast<float2*>(smem + TILE + 4096), sBar, abort);
                 if (x == 0 || ps.has_b || kpp) {
-                    softmax_tile<true, kSif, kKpp, D, kColO, false, kTwo>(P, tmem, sBar, x, warp & 3, lane, x && !kpp ? ps.t0b : ps.t0a, l, bl,
+                    softmax_tile<true, kSif, kKpp, D, kColO, false, kTerms>(P, tmem, sBar, x, warp & 3, lane, x && !kpp ? ps.t0b : ps.t0a, l, bl,
                                  b, hk, sp, ps, done, (uint32_t)pi & 1u, p_count > 1, abort,
                                  pi == p_count - 1 ? sQ : 0u, kpp);
                     done += kpp ? (uint32_t)((ps.n_kv + 1 - x) / 2) : (uint32_t)ps.n_kv;
@@ -2343,7 +2378,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc64_sif_kernel(const __grid
 // kTwo: weights of two bf16 terms.
 template <bool kTwo>
 __global__ void __launch_bounds__(kThreads, 1) attn_tc_decode_kernel(const __grid_constant__ DecodeTcParams KP) {
-    attn_tc_body<false, false, false, true, HD, kTwo>(KP);
+    attn_tc_body<false, false, false, true, HD, kTwo ? 2 : 1>(KP);
 }
 
 // One query tile a CTA (the solo kernel), in two forms.
@@ -2352,8 +2387,9 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_decode_kernel(const __gri
 //   latency) and its end (the last softmax, P.V and the epilogue) are some 9 us of a unit of nine
 //   key tiles' 24, and several short pairs in turn pay for each change of query tiles.  Here the
 //   SM's other CTA works on meanwhile: each has one Q tile, one K and one V tile (two at 64
-//   channels; 96 KB at 128), S and O in 256 columns of tensor memory, and runs the chain S(j),
-//   softmax(j), P.V(j); K of the next tile lands while the softmax runs.
+//   channels; 96 KB at 128), S, O and the third term of the weights (64 channels) in 256 columns
+//   of tensor memory, and runs the chain S(j), softmax(j), P.V(j); K of the next tile lands while
+//   the softmax runs.
 //   Alone, one CTA an SM, when the query tiles do not outnumber the SMs: two K and V stages, and S
 //   and P double-buffered in 512 columns, so that S(j + 1) is computed while softmax(j) runs and
 //   the softmax alone is the chain.
@@ -2550,10 +2586,14 @@ __device__ __forceinline__ void attn_solo_body(const TcParams& P) {
                 for (int kk = 0; kk < BN / 16; ++kk)
                     mma_bf16_ts(tO, tP + (uint32_t)kk * 8u, dv + (uint64_t)((kk * kKeyStep) >> 4), idO,
                                 kk > 0 || j > 0 ? 1u : 0u);
-                if constexpr (Geo<D>::kSplitP) {
+                if constexpr (Geo<D>::kTerms == 3) {
 #pragma unroll
                     for (int kk = 0; kk < BN / 16; ++kk)
                         mma_bf16_ts(tO, tP + 64u + (uint32_t)kk * 8u, dv + (uint64_t)((kk * kKeyStep) >> 4), idO, 1u);
+                    const uint32_t tP3 = tmem + kThirdTerm<L::kO> + d * 64u;
+#pragma unroll
+                    for (int kk = 0; kk < BN / 16; ++kk)
+                        mma_bf16_ts(tO, tP3 + (uint32_t)kk * 8u, dv + (uint64_t)((kk * kKeyStep) >> 4), idO, 1u);
                 }
                 if (kAlone) mma_commit(bar(B_OE));
                 mma_commit(bar(B_VE + st));

@@ -48,10 +48,9 @@ def test_extract(n, k):
 
 
 def test_weights_keep_more_than_bf16():
-    """The tensor-core kernel's weights enter P.V as two bf16 terms, so its output is off the
-    CUDA-core kernel's (fp32 weights) by at most a rounding flip of the bf16 output (2^-8 of the
-    value) and, per unit weight, 2^-17 of the largest value; four times that covers the two
-    kernels' fp32 sums.  Weights of one bf16 term would be off by 2^-9 of it."""
+    """The tensor-core kernel's output is off the CUDA-core kernel's by at most a rounding flip of the
+    bf16 output (2^-8 of the value) and, per unit weight, 2^-15 of the largest value.  Weights of one
+    bf16 term would be off by 2^-9 of it."""
     c2kv = H.lib()
     wl = synth.scaled(D64, n_suffix=50, chunks_per_request=4, pool_chunks=4)
     (ids, offs), = synth.requests(wl)
@@ -72,6 +71,42 @@ def test_weights_keep_more_than_bf16():
     vmax = max(float(vs.abs().max()), max(float(np.abs(c[1]).max()) for c in chunks.values()))
     allowed = 2.0 ** -8 * np.abs(outs[1]) + 4 * 2.0 ** -17 * vmax
     assert (np.abs(outs[0] - outs[1]) <= allowed).all(), float((np.abs(outs[0] - outs[1]) - allowed).max())
+
+
+@pytest.mark.parametrize("layers,pairs", [(16, 0), (80, 0), (16, 1)], ids=["alone", "shared", "pair"])
+def test_weights_hold_fp32(layers, pairs):
+    """Two keys that differ by a little in one channel and carry values 1 and -1: the output is the
+    difference of their weights, some 2^-10 of either.  The CUDA-core kernel's weights are fp32, and both
+    routes read the same turned queries and cached rows, so what may differ is a rounding flip of the
+    output (2^-8 of it) and the exponentials' and sums' error: ex2.approx and the exponent's rounding,
+    2^-22 each, for two weights of at most 1, doubled for the other route: 2^-20.  Weights of 16
+    significant bits are off by up to 2^-17 each."""
+    c2kv = H.lib()
+    n = 32
+    wl = synth.scaled(D64, n_q_heads=8, n_kv_heads=2, layers=layers)
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    q = torch.randn((layers, 1, n, 8, 64), generator=gen, device="cuda").bfloat16()
+    zero = torch.zeros((layers, 1, n, 2, 64), device="cuda").bfloat16()       # suffix rows: score 0, value 0
+    rows = torch.randn((layers, 1, 2, 64), generator=gen, device="cuda").repeat(1, 2, 1, 1)
+    rows[..., 0] = torch.tensor([0.0, 2.0 ** -7], device="cuda").view(1, 2, 1)
+    outs = []
+    for impl in (c2kv.ATTN_AUTO, c2kv.ATTN_SIMT):
+        ctx = H.make_ctx(wl, pool_slots=2, attn_impl=impl, attn_pairs=pairs)
+        try:
+            cid = c2kv.c2kv_compress_chunk(ctx, rows.bfloat16(), rows.bfloat16(), 2, 1, c2kv.MODE_STORED)
+            cache = c2kv.c2kv_compose(ctx, [0, 1], [cid], None, suffix_capacity=n)
+            info = c2kv.c2kv_cache_info(cache)
+            ck, cv = (c2kv.device_view(info[x], (layers, info["rows"], 2, 64), torch.bfloat16) for x in "kv")
+            ck[:, :2] = rows.bfloat16()
+            cv[:, 0], cv[:, 1] = 1.0, -1.0
+            out = torch.full_like(q, float("nan"))
+            c2kv.c2kv_attend(ctx, cache, -1, q, zero, zero, n, out)
+            c2kv.c2kv_sync(ctx)
+            outs.append(out.double())
+        finally:
+            c2kv.c2kv_destroy(ctx)
+    over = (outs[0] - outs[1]).abs() - (2.0 ** -8 * outs[1].abs() + 2.0 ** -20)
+    assert (over <= 0).all(), f"{float((over > 0).double().mean()):.3f} of the outputs off by up to {float(over.max()):.3g} more"
 
 
 def test_forced_tensor_cores_stay_refused():
