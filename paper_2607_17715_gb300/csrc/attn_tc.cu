@@ -2622,13 +2622,13 @@ __global__ void __launch_bounds__(kSoloThreads, kAlone ? 1 : 2) attn_solo_kernel
 }
 
 // The kernel of an instantiation.
-// kSolo: 0, or the solo kernel shared (1) or alone (2).
-template <bool kFused, bool kMulti, bool kSif, bool kKpp = false, int D = HD, int kSolo = 0>
+// kSolo: 0, or the solo kernel shared (1) or alone (2).  kTwo (decode): weights of two bf16 terms.
+template <bool kFused, bool kMulti, bool kSif, bool kKpp = false, int D = HD, int kSolo = 0, bool kTwo = false>
 const void* tc_kernel_fn() {
     if constexpr (kSolo != 0) return reinterpret_cast<const void*>(&attn_solo_kernel<kSif, D, kSolo == 2>);
     else if constexpr (D == 64) return reinterpret_cast<const void*>(kSif ? &attn_tc64_sif_kernel : &attn_tc64_kernel);
     else if constexpr (kSif) return reinterpret_cast<const void*>(&attn_tc_sif_kernel);
-    else if constexpr (kKpp) return reinterpret_cast<const void*>(&attn_tc_decode_kernel<false>);
+    else if constexpr (kKpp) return reinterpret_cast<const void*>(&attn_tc_decode_kernel<kTwo>);
     else return reinterpret_cast<const void*>(&attn_tc_kernel<kFused, kMulti>);
 }
 
@@ -2777,19 +2777,23 @@ namespace {
 
 // Host-side preparation shared by the plain and the fused launch: function attributes once
 // per process, the register-split guard, the tensor maps and the scalar parameters.
-template <bool kFused, bool kMulti = false, bool kSif = false, bool kKpp = false, int D = HD, int kSolo = 0>
+template <bool kFused, bool kMulti = false, bool kSif = false, bool kKpp = false, int D = HD, int kSolo = 0,
+          bool kTwo = false>
 cudaError_t prepare_tc(const AttnParams& a, TcParams& p, dim3& grid) {
     constexpr int threads = kFused ? kThreadsFused : kThreads;
     constexpr int high = kFused ? kRegsHighFused : kRegsHigh;
     constexpr int low_total = kFused ? 128 * (kRegsLowFused + kRegsLoadFused) : 128 * kRegsLow;
     // once per process (one device per context; function-local statics: thread-safe)
     static const cudaError_t smem_err = cudaFuncSetAttribute(
-        tc_kernel_fn<kFused, kMulti, kSif, kKpp, D, kSolo>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSolo ? Solo<D, kSolo == 2>::kSmem : Geo<D>::kSmem));
+        tc_kernel_fn<kFused, kMulti, kSif, kKpp, D, kSolo, kTwo>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
+        (int)(kSolo ? Solo<D, kSolo == 2>::kSmem : Geo<D>::kSmem));
     if (smem_err != cudaSuccess) return smem_err;
     if constexpr (!kSolo) {   // the register split must not ask for more than the launch holds
         static const int launch_regs = []() {
             cudaFuncAttributes fa{};
-            return cudaFuncGetAttributes(&fa, tc_kernel_fn<kFused, kMulti, kSif, kKpp, D, kSolo>()) == cudaSuccess ? fa.numRegs : -1;
+            return cudaFuncGetAttributes(&fa, tc_kernel_fn<kFused, kMulti, kSif, kKpp, D, kSolo, kTwo>()) == cudaSuccess
+                       ? fa.numRegs
+                       : -1;
         }();
         if (launch_regs < 0) return cudaErrorInvalidDeviceFunction;
         if (launch_regs * threads < low_total + 256 * high) return cudaErrorInvalidConfiguration;
@@ -2987,14 +2991,10 @@ cudaError_t launch_attn_tc(const AttnParams& a, cudaStream_t s, Hook before) {
 cudaError_t launch_attn_tc_decode(const AttnParams& a, const DecodeAppend& d, cudaStream_t s, Hook before) {
     (void)cudaGetLastError();   // report this launch's error only, not a stale one
     if (!d.k_new || !d.v_new || !d.pos || a.d != HD) return cudaErrorInvalidValue;
-    if (d.two_terms) {
-        static const cudaError_t smem_err = cudaFuncSetAttribute(
-            attn_tc_decode_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
-        if (smem_err != cudaSuccess) return smem_err;
-    }
     DecodeTcParams p;
     dim3 grid;
-    cudaError_t e = prepare_tc<false, false, false, true>(a, p.t, grid);
+    const cudaError_t e = d.two_terms ? prepare_tc<false, false, false, true, HD, 0, true>(a, p.t, grid)
+                                      : prepare_tc<false, false, false, true, HD, 0, false>(a, p.t, grid);
     if (e != cudaSuccess) return e;
     p.k_new = d.k_new;
     p.v_new = d.v_new;

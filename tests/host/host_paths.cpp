@@ -1,0 +1,119 @@
+// The library's host code over the stand-in runtime: one scenario a run (its name is the argument).
+#include <c2kv.h>
+
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+#include <numeric>
+
+#include "fake_cudart.h"
+
+namespace {
+
+#define CHECK(cond, ...)                                                \
+    do {                                                                \
+        if (!(cond)) {                                                  \
+            std::printf("%s:%d: %s: ", __FILE__, __LINE__, #cond);      \
+            std::printf(__VA_ARGS__);                                   \
+            std::printf("\n");                                          \
+            std::exit(1);                                               \
+        }                                                               \
+    } while (0)
+
+alignas(256) char buffer[256];          // every tensor: its address is checked, nothing is read
+
+struct Shape {
+    int dtype, hq, hkv, d, layers = 1;
+};
+
+struct Context {
+    Shape s;
+    c2kv_ctx* ctx = nullptr;
+    explicit Context(Shape shape, int split = 0, int pairs = 0, int fuse = 0, int impl = 0) : s(shape) {
+        c2kv_config cfg{};
+        cfg.layers = s.layers;
+        cfg.n_q_heads = s.hq;
+        cfg.n_kv_heads = s.hkv;
+        cfg.head_dim = s.d;
+        cfg.rope_theta = 1e4;
+        cfg.dtype = s.dtype;
+        cfg.pool_slots = 65536;
+        cfg.attn_impl = impl;
+        cfg.attn_split = split;
+        cfg.attn_pairs = pairs;
+        cfg.fuse = fuse;
+        const c2kv_status st = c2kv_create(&cfg, nullptr, &ctx);
+        CHECK(st == C2KV_OK, "create: %s", c2kv_last_error(nullptr));
+    }
+    ~Context() { c2kv_destroy(ctx); }
+    int chunk(int slots) {
+        int32_t id = -1;
+        CHECK(c2kv_compress_chunk(ctx, buffer, buffer, slots, 1, C2KV_MODE_STORED, &id) == C2KV_OK, "compress");
+        return id;
+    }
+    // `batch` requests of one chunk each
+    c2kv_cache* compose(int batch, int slots, int suffix) {
+        std::vector<int32_t> ptr(batch + 1), ids(batch, chunk(slots));
+        std::iota(ptr.begin(), ptr.end(), 0);
+        c2kv_cache* cache = nullptr;
+        CHECK(c2kv_compose(ctx, batch, ptr.data(), ids.data(), nullptr, suffix, &cache) == C2KV_OK, "compose: %s",
+              c2kv_last_error(ctx));
+        return cache;
+    }
+    c2kv_status attend(c2kv_cache* cache, int suffix) {
+        return c2kv_attend(ctx, cache, -1, buffer, buffer, buffer, suffix, buffer, nullptr);
+    }
+    c2kv_status decode(c2kv_cache* cache, int batch) {
+        std::vector<int32_t> steps(batch, 0);
+        return c2kv_decode(ctx, cache, -1, buffer, buffer, buffer, steps.data(), buffer, nullptr);
+    }
+    c2kv_status extract(int tokens, int ratio) {
+        return c2kv_extract_attention(ctx, 1, buffer, buffer, buffer, tokens, ratio, buffer, nullptr);
+    }
+    c2kv_status step(int chunks, int slots, int suffix, c2kv_cache** cache) {
+        std::vector<int32_t> ids;
+        for (int i = 0; i < chunks; ++i) ids.push_back(chunk(slots));
+        const int32_t ptr[2] = {0, chunks};
+        return c2kv_compose_attend(ctx, 1, ptr, ids.data(), nullptr, suffix, buffer, buffer, buffer, suffix, buffer,
+                                   nullptr, cache);
+    }
+};
+
+constexpr int kBf16 = C2KV_DTYPE_BF16, kF32 = C2KV_DTYPE_F32;
+
+// The kernels whose warps trade registers (setmaxnreg) wait forever when the launch holds fewer than
+// the split hands out, so none of them may be launched with a smaller compiled count.  One kernel a run
+// (the library reads the counts once a process), under the calls that launch them.
+void registers(const std::string& part) {
+    fake::registers = [&](const std::string& name) { return name.find(part) != std::string::npos ? 64 : 168; };
+    int refused = 0;
+    auto call = [&](c2kv_status st) { refused += st == C2KV_ERR_CUDA; };
+    c2kv_cache* cache = nullptr;
+    for (int d : {128, 64}) {
+        Context pairs({kBf16, 32, 8, d}, 1, 1);
+        call(pairs.attend(pairs.compose(1, 1000, 300), 300));
+        call(pairs.extract(600, 4));
+    }
+    Context step({kBf16, 32, 8, 128});
+    call(step.step(4, 128, 32, &cache));
+    Context forced({kBf16, 32, 8, 128}, 0, 0, C2KV_FUSE_ALWAYS);
+    call(forced.step(4, 128, 200, &cache));
+    call(step.decode(step.compose(1, 1000, 8), 1));
+    Context groups({kBf16, 64, 8, 128});                  // eight queries a KV head, more units than SMs
+    call(groups.decode(groups.compose(20, 400, 8), 20));
+    CHECK(!fake::launched(part), "%s launched with too few registers", part.c_str());
+    CHECK(refused > 0, "no call reaches %s", part.c_str());
+}
+
+}  // namespace
+
+int main(int argc, char** argv) {
+    const std::string name = argc > 1 ? argv[1] : "";
+    if (name == "kernels") {
+        for (const std::string& k : fake::kernel_names()) std::printf("%s\n", k.c_str());
+        return 0;
+    }
+    if (name == "registers") registers(argv[2]);
+    else CHECK(false, "unknown scenario '%s'", name.c_str());
+    std::printf("ok\n");
+}
