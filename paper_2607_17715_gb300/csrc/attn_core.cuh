@@ -32,6 +32,7 @@
 #include <algorithm>
 
 #include "internal.cuh"
+#include "per_device.cuh"
 #include "ptx.cuh"
 #include "vec16.cuh"
 
@@ -413,8 +414,7 @@ inline CorePlan core_plan(int64_t nrows, int64_t units, int64_t nkeys, int d, co
     return best;
 }
 
-// CTAs of a kernel with `smem` bytes in clusters of ns that the device holds at once; the answer
-// is kept per (kernel, ns, alone) by the caller's table.
+// CTAs of a kernel with `smem` bytes in clusters of ns that the device holds at once.
 inline int core_capacity(const void* kernel, int ns, size_t smem, int sms) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)ns);
@@ -439,12 +439,12 @@ inline int core_capacity(const void* kernel, int ns, size_t smem, int sms) {
     return n;
 }
 
-// The shared memory opt-in of a kernel instantiation and its table of capacities, filled once per
-// process (function-local statics: thread-safe).
+// The shared memory opt-in of a kernel instantiation on a device, and its table of capacities there.
 template <int D, int RT>
 struct CoreKernel {
-    cudaError_t err;
-    int slots[2][kCoreMaxSplit + 1];       // [alone][ns]
+    cudaError_t err = cudaSuccess;
+    int slots[2][kCoreMaxSplit + 1] = {};  // [alone][ns]
+    CoreKernel() = default;
     CoreKernel(const void* kernel, int sms) {
         err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    std::max(Core<D, RT>::kSmem, kCoreAlone));
@@ -454,18 +454,6 @@ struct CoreKernel {
         }
     }
 };
-
-// SMs of the current device, read once per process.
-inline int core_sms() {
-    static const int sms = []() {
-        int dev = 0, n = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1)
-            return 1;
-        return n;
-    }();
-    return sms;
-}
 
 }  // namespace
 }  // namespace c2kv

@@ -62,9 +62,9 @@ __global__ void __launch_bounds__(kCoreThreads, core_ctas(D, RT)) attn_simt_kern
 }
 
 template <typename T, int D, int RT>
-const CoreKernel<D, RT>& ready() {
-    static const CoreKernel<D, RT> k(reinterpret_cast<const void*>(&attn_simt_kernel<T, D, RT>), core_sms());
-    return k;
+CoreKernel<D, RT> ready() {
+    static PerDevice<CoreKernel<D, RT>> kept;
+    return kept.get([] { return CoreKernel<D, RT>(reinterpret_cast<const void*>(&attn_simt_kernel<T, D, RT>), device_sms()); });
 }
 
 template <typename T, int D, int RT>
@@ -97,8 +97,8 @@ cudaError_t launch_typed(const AttnParams& a, cudaStream_t s) {
     int64_t nkeys = 0;
     for (int i = 0; i < a.batch; ++i) nkeys = std::max<int64_t>(nkeys, (int64_t)a.req[i].n_slots + a.sq);
     const int64_t nrows = (int64_t)a.sq * (a.hq / a.hkv);
-    const CoreKernel<D, 4>& large = ready<T, D, 4>();
-    const CoreKernel<D, 1>& small = ready<T, D, 1>();
+    const CoreKernel<D, 4> large = ready<T, D, 4>();
+    const CoreKernel<D, 1> small = ready<T, D, 1>();
     if (large.err != cudaSuccess || small.err != cudaSuccess) return large.err != cudaSuccess ? large.err : small.err;
     const CorePlan plan = core_plan(nrows, (int64_t)a.hkv * a.lq * a.batch, nkeys, D, [&](bool sm, int ns, bool alone) {
         return sm ? small.slots[alone][ns] : large.slots[alone][ns];

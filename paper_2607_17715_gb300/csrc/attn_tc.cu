@@ -67,6 +67,7 @@
 #include <cstring>
 
 #include "internal.cuh"
+#include "per_device.cuh"
 #include "ptx.cuh"
 #include "rope.cuh"
 #include "vec16.cuh"
@@ -2776,25 +2777,23 @@ bool attn_tc_takes(int dtype, int d, int hq, int hkv) {
 namespace {
 
 // Host-side preparation shared by the plain and the fused launch: function attributes once
-// per process, the register-split guard, the tensor maps and the scalar parameters.
+// per device, the register-split guard, the tensor maps and the scalar parameters.
 template <bool kFused, bool kMulti = false, bool kSif = false, bool kKpp = false, int D = HD, int kSolo = 0,
           bool kTwo = false>
 cudaError_t prepare_tc(const AttnParams& a, TcParams& p, dim3& grid) {
     constexpr int threads = kFused ? kThreadsFused : kThreads;
     constexpr int high = kFused ? kRegsHighFused : kRegsHigh;
     constexpr int low_total = kFused ? 128 * (kRegsLowFused + kRegsLoadFused) : 128 * kRegsLow;
-    // once per process (one device per context; function-local statics: thread-safe)
-    static const cudaError_t smem_err = cudaFuncSetAttribute(
-        tc_kernel_fn<kFused, kMulti, kSif, kKpp, D, kSolo, kTwo>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
-        (int)(kSolo ? Solo<D, kSolo == 2>::kSmem : Geo<D>::kSmem));
+    const void* const kernel = tc_kernel_fn<kFused, kMulti, kSif, kKpp, D, kSolo, kTwo>();
+    static PerDevice<cudaError_t> smem;
+    const cudaError_t smem_err = opt_in_smem(smem, kernel, kSolo ? Solo<D, kSolo == 2>::kSmem : Geo<D>::kSmem);
     if (smem_err != cudaSuccess) return smem_err;
     if constexpr (!kSolo) {   // the register split must not ask for more than the launch holds
-        static const int launch_regs = []() {
+        static PerDevice<int> regs;
+        const int launch_regs = regs.get([&] {
             cudaFuncAttributes fa{};
-            return cudaFuncGetAttributes(&fa, tc_kernel_fn<kFused, kMulti, kSif, kKpp, D, kSolo, kTwo>()) == cudaSuccess
-                       ? fa.numRegs
-                       : -1;
-        }();
+            return cudaFuncGetAttributes(&fa, kernel) == cudaSuccess ? fa.numRegs : -1;
+        });
         if (launch_regs < 0) return cudaErrorInvalidDeviceFunction;
         if (launch_regs * threads < low_total + 256 * high) return cudaErrorInvalidConfiguration;
     }
@@ -2864,13 +2863,7 @@ cudaError_t prepare_tc(const AttnParams& a, TcParams& p, dim3& grid) {
         if (p.n_split != 1) return cudaErrorInvalidValue;
         pg = pairs;
     } else if (!kFused && p.n_split == 1) {
-        static const int sms = []() {
-            int dev = 0, n = 0;
-            if (cudaGetDevice(&dev) != cudaSuccess ||
-                cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1)
-                return 1;
-            return n;
-        }();
+        const int sms = device_sms();
         const int64_t cols = (int64_t)a.hkv * a.lq * a.batch;
         int slots = 0;
         for (int i = 0; i < a.batch; ++i) slots = std::max(slots, a.req[i].n_slots + a.req[i].t0);
@@ -2947,13 +2940,7 @@ cudaError_t launch_plain(const AttnParams& a, cudaStream_t s, Hook before) {
 enum class SoloChoice { kPair, kShared, kAlone };
 SoloChoice solo_choice(const AttnParams& a) {
     if (a.key_pingpong || a.pairs_per_cta != 0 || a.tickets != nullptr) return SoloChoice::kPair;
-    static const int sms = []() {
-        int dev = 0, n = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1)
-            return 1;
-        return n;
-    }();
+    const int sms = device_sms();
     const int tq = BM / (a.hq / a.hkv);
     const int64_t per_head = (a.sq + tq - 1) / tq, heads = (int64_t)a.hkv * a.lq * a.batch;
     const int64_t units = per_head * heads * std::max(1, a.n_split);

@@ -18,6 +18,7 @@
 #include <cstring>
 
 #include "internal.cuh"
+#include "per_device.cuh"
 #include "ptx.cuh"
 #include "vec16.cuh"
 
@@ -407,9 +408,8 @@ cudaError_t launch_g(const DecodeParams& p, cudaStream_t s, Hook before) {
         if (!encode_tensor_map(&x.tm_v, ty, 3, p.cache_v, dims, str, box, CU_TENSOR_MAP_SWIZZLE_NONE))
             return cudaErrorInvalidValue;
     }
-    // once per instantiation (a function-local static: thread-safe)
-    static const cudaError_t smem_err = cudaFuncSetAttribute(
-        decode_kernel<T, D, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecSmem);
+    static PerDevice<cudaError_t> smem;
+    const cudaError_t smem_err = opt_in_smem(smem, reinterpret_cast<const void*>(&decode_kernel<T, D, G>), kDecSmem);
     if (smem_err != cudaSuccess) return smem_err;
     cudaError_t e = cudaSuccess;
     const dim3 grid((unsigned)p.n_split, (unsigned)p.hkv, (unsigned)(p.lq * p.batch));

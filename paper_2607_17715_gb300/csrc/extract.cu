@@ -260,9 +260,9 @@ cudaError_t launch_tc(const ExtractParams& p, cudaStream_t s, cudaStream_t s2, c
 }
 
 template <typename T, int D, int RT>
-const CoreKernel<D, RT>& ready() {
-    static const CoreKernel<D, RT> k(reinterpret_cast<const void*>(&extract_attn_kernel<T, D, RT>), core_sms());
-    return k;
+CoreKernel<D, RT> ready() {
+    static PerDevice<CoreKernel<D, RT>> kept;
+    return kept.get([] { return CoreKernel<D, RT>(reinterpret_cast<const void*>(&extract_attn_kernel<T, D, RT>), device_sms()); });
 }
 
 template <typename T, int D, int RT>
@@ -292,8 +292,8 @@ cudaError_t launch_typed(const ExtractParams& p, cudaStream_t s) {
     extract_rope_kernel<T, VPH><<<dim3((unsigned)p.n_all, (unsigned)p.lq), 256, 0, s>>>(p);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const CoreKernel<D, 4>& large = ready<T, D, 4>();
-    const CoreKernel<D, 1>& small = ready<T, D, 1>();
+    const CoreKernel<D, 4> large = ready<T, D, 4>();
+    const CoreKernel<D, 1> small = ready<T, D, 1>();
     if (large.err != cudaSuccess || small.err != cudaSuccess) return large.err != cudaSuccess ? large.err : small.err;
     // (the causal rows see half of the keys on average)
     const CorePlan plan = core_plan((int64_t)p.n_all * (p.hq / p.hkv), (int64_t)p.hkv * p.lq, (p.n_all + 1) / 2, D,

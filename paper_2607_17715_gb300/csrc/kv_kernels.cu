@@ -9,9 +9,9 @@
 // once to a float in [-1/2, 1/2) turns and handed to sincospif.  The error is about
 // 1e-7 rad at any position, where forming p * inv_freq in fp32 would lose p * 2^-24 rad.
 #include <algorithm>
-#include <atomic>
 
 #include "internal.cuh"
+#include "per_device.cuh"
 #include "ptx.cuh"
 #include "rope.cuh"
 #include "vec16.cuh"
@@ -617,12 +617,6 @@ __global__ void __launch_bounds__(256) suffix_kernel(const __grid_constant__ Suf
     }
 }
 
-int sm_count() {
-    int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return sms;
-}
-
 int vph_of(int dtype, int d) { return d / 2 / (dtype == kDtypeBf16 ? 8 : 4); }
 
 }  // namespace
@@ -648,17 +642,10 @@ cudaError_t preload_suffix_kernels(int dtype, int d) {
 
 template <typename T, int VPH, int N>
 cudaError_t launch_bulk_n(const ComposeParams& p, int layers, cudaStream_t s, Hook pre) {
-    static std::atomic<uint64_t> attr_set{0};     // per instantiation: devices 0..63 done
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    const uint64_t bit = dev < 64 ? (uint64_t)1 << dev : 0;
-    if (!(attr_set.load() & bit)) {
-        e = cudaFuncSetAttribute(compose_bulk_kernel<T, VPH, N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kBulkSmem);
-        if (e != cudaSuccess) return e;
-        attr_set.fetch_or(bit);
-    }
+    static PerDevice<cudaError_t> smem;
+    const cudaError_t smem_err =
+        opt_in_smem(smem, reinterpret_cast<const void*>(&compose_bulk_kernel<T, VPH, N>), kBulkSmem);
+    if (smem_err != cudaSuccess) return smem_err;
     BulkParams<N> bp;
     static_cast<ComposeHead&>(bp) = p;
     for (int i = 0; i < p.n_occ; ++i) bp.occ[i] = p.occ[i];
@@ -667,7 +654,7 @@ cudaError_t launch_bulk_n(const ComposeParams& p, int layers, cudaStream_t s, Ho
     const int nst = (int)std::min<int64_t>(kBulkMaxStages, kBulkSmem / stage);
     if (nst < 2) return cudaErrorInvalidValue;
     const int64_t items = (int64_t)p.n_tiles * layers;
-    const int grid = (int)std::min<int64_t>(items, sm_count());
+    const int grid = (int)std::min<int64_t>(items, device_sms());
     pre();
     compose_bulk_kernel<T, VPH, N><<<grid, kBulkThreads, (size_t)(nst * stage), s>>>(bp, layers, nst);
     return cudaGetLastError();

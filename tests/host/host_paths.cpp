@@ -105,6 +105,45 @@ void registers(const std::string& part) {
     CHECK(refused > 0, "no call reaches %s", part.c_str());
 }
 
+// What a process sets up on its first device is set up again on its second: every kernel that needs more
+// than 48 KB of dynamic shared memory launches there too, and the rules count that device's SMs.
+void second_device() {
+    fake::sms = [](int device) { return device == 0 ? 152 : 16; };
+    for (fake::device = 0; fake::device < 2; ++fake::device) {
+        auto ok = [](c2kv_ctx* ctx, c2kv_status st, const char* what) {
+            CHECK(st == C2KV_OK, "device %d, %s: %s", fake::device, what, c2kv_last_error(ctx));
+        };
+        for (const Shape& s : {Shape{kF32, 4, 2, 64}, Shape{kF32, 16, 4, 128}, Shape{kBf16, 24, 8, 64},
+                               Shape{kBf16, 24, 8, 128}, Shape{kBf16, 32, 8, 64}, Shape{kBf16, 32, 8, 128}}) {
+            Context one(s);
+            for (int batch : {1, 40}) {                              // one row tile or key split a CTA; many
+                c2kv_cache* cache = one.compose(batch, 700, 100);
+                ok(one.ctx, one.attend(cache, 3), "attend");
+                ok(one.ctx, one.attend(cache, 100), "attend");
+                if (s.hq / s.hkv != 3) ok(one.ctx, one.decode(cache, batch), "decode");
+            }
+            ok(one.ctx, one.extract(600, 4), "extract");
+            if (s.dtype == kBf16 && s.hq == 32) {
+                Context pairs(s, 1, 1);
+                ok(pairs.ctx, pairs.attend(pairs.compose(1, 700, 100), 100), "attend, pairs");
+                ok(pairs.ctx, pairs.extract(600, 4), "extract, pairs");
+            }
+        }
+        Context groups({kBf16, 64, 8, 128});
+        ok(groups.ctx, groups.decode(groups.compose(20, 400, 8), 20), "decode of groups of eight");
+        for (int fuse : {C2KV_FUSE_AUTO, C2KV_FUSE_ALWAYS}) {
+            c2kv_cache* cache = nullptr;
+            Context step({kBf16, 32, 8, 128}, 0, 0, fuse);
+            ok(step.ctx, step.step(4, 128, fuse == C2KV_FUSE_AUTO ? 32 : 200, &cache), "step");
+        }
+        // 64 query tiles: one an SM on the first device, more than the SMs on the second
+        fake::launches.clear();
+        Context tiles({kBf16, 32, 8, 128}, 1);
+        ok(tiles.ctx, tiles.attend(tiles.compose(2, 300, 100), 100), "attend, 64 tiles");
+        CHECK(fake::launched("attn_solo_kernelILb0ELi128ELb1E") == (fake::device == 0), "device %d", fake::device);
+    }
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
@@ -114,6 +153,7 @@ int main(int argc, char** argv) {
         return 0;
     }
     if (name == "registers") registers(argv[2]);
+    else if (name == "second_device") second_device();
     else CHECK(false, "unknown scenario '%s'", name.c_str());
     std::printf("ok\n");
 }

@@ -35,3 +35,8 @@ def test_register_splits_are_guarded(program):
     assert len(kernels) == 8
     for k in kernels:
         _run(program, "registers", k)
+
+
+@pytest.mark.parametrize("scenario", ["second_device"])
+def test_scenario(program, scenario):
+    _run(program, scenario)
