@@ -351,7 +351,7 @@ c2kv_status c2kv_attend_noalloc(c2kv_ctx* ctx, c2kv_cache* cache, int32_t layer,
  * kernel); the split buffer comes from the context's memory pool.  With bf16
  * and d = 128 the step runs on the tensor-core attention kernel (the new token as a one-row
  * query tile) when (layers x requests x KV heads) fits one CTA per SM or a request holds
- * more than 31 x 128 keys, or, with each softmax weight as two bf16 terms, when G = 8 and a
+ * more than 31 x 128 keys, or, with fp32 softmax weights (three bf16 terms each), when G = 8 and a
  * request holds more than 2 x 128; else on a CUDA-core decode kernel (C2KV_ATTN_TC forces the former,
  * C2KV_ATTN_SIMT the latter).
  * The tensor-core route reads whole 128-row key tiles, so it zeroes the rows after the new

@@ -322,12 +322,6 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&v)[16
         : "memory");
 }
 
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&v)[8]) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr),
-                 "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
-                 : "memory");
-}
-
 __device__ __forceinline__ void tmem_st4(uint32_t taddr, const uint32_t (&v)[4]) {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr), "r"(v[0]), "r"(v[1]),
                  "r"(v[2]), "r"(v[3])
@@ -403,6 +397,15 @@ __device__ __forceinline__ void stg256(void* p, const uint32_t* w) {
                  "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
                  : "memory");
 }
+__device__ __forceinline__ uint4 lds128(uint32_t a) {
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "r"(a)
+                 : "memory");
+    return v;
+}
+__device__ __forceinline__ uint32_t word_of(const uint4& v, int i) { return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w; }
 __device__ __forceinline__ void sts128_(uint32_t a, const uint4& v) {
     asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
                  : "memory");
@@ -587,8 +590,11 @@ __device__ __forceinline__ PairSpan tile_span(const TcParams& P, int qt, int sp,
 // kO: the first TMEM column of O_A.  kDbl (x = 0): S and P alternate between two column blocks and
 // their barriers (B_SF, B_PF and the next ones); P.V(j - 1) may then still run when S(j) is read,
 // so a rescale of O waits for it (B_OE, one phase per P.V).
-// kTerms: bf16 terms of a weight (Geo::kTerms; two for a decode step that the CUDA cores would
-// compute with fp32 weights).
+// kTerms: bf16 terms of a weight (Geo::kTerms; three for a decode step that the CUDA cores would
+// compute with fp32 weights).  A decode step's three are in rows, not columns: its one query token
+// fills at most 16 rows of the tile's 128, so decode_turn_queries repeats them at rows 32 and 64,
+// every quad of warps finds the same scores and weights, and quad i's rows hold term i.  One P.V then
+// multiplies all three, at no MMA more, and warpgroup A adds the three rows of O at the end.
 template <bool kMerge, bool kSif = false, bool kKpp = false, int D = HD, uint32_t kO = kColO, bool kDbl = false,
           int kTerms = Geo<D>::kTerms>
 __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, uint32_t sBar, int x,
@@ -690,11 +696,13 @@ __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, u
         // P_j (bf16, keys 2c and 2c+1 packed in column c) over the first half of S_x
         const uint32_t p_addr = tmem + lane_addr + colS + dbl * BN;
         const float neg_m = -m_sub;
-        // (several terms: 16 keys at a time, the second over the last 64 columns)
-        constexpr int PW = kTerms == 3 ? 4 : kTerms == 2 ? 8 : 16;       // packed words per store
+        // (terms in columns: 8 keys at a time, the second over the last 64 columns)
+        constexpr bool kCols = kTerms > 1 && !kKpp, kRows = kTerms > 1 && kKpp;
+        constexpr int PW = kCols ? 4 : 16;      // packed words per store
 #pragma unroll
         for (int c = 0; c < 64 / PW; ++c) {
-            uint32_t pk[PW], p2[kTerms > 1 ? PW : 1], p3[kTerms > 2 ? PW : 1];
+            uint32_t pk[PW], p2[kCols ? PW : 1], p3[kCols ? PW : 1];
+            float ar[kRows ? 2 * PW : 1];
 #pragma unroll
             for (int w = 0; w < PW; ++w) {
                 const int e = 2 * (c * PW + w);            // key of the tile
@@ -703,23 +711,29 @@ __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, u
                 a0 = ex2(a0);
                 a1 = ex2(a1);
                 if (e & 2) fadd2(ps[2], ps[3], a0, a1); else fadd2(ps[0], ps[1], a0, a1);
-                if constexpr (kTerms == 3) {     // the top 8 bits of what is left, three times
+                if constexpr (kCols) {           // the top 8 bits of what is left, three times
                     pk[w] = cut_bf16(a0, a1);
                     p2[w] = cut_bf16(a0, a1);
                     p3[w] = cut_bf16(a0, a1);
+                } else if constexpr (kRows) {
+                    ar[2 * w] = a0;
+                    ar[2 * w + 1] = a1;
                 } else {
                     pk[w] = pack_bf16(a0, a1);
-                    if constexpr (kTerms == 2)   // what the rounding left (exact differences)
-                        p2[w] = pack_bf16(a0 - __uint_as_float(pk[w] << 16), a1 - __uint_as_float(pk[w] & 0xffff0000u));
                 }
             }
-            if constexpr (kTerms == 3) {
+            if constexpr (kRows) {               // quad i: what is left after i cuts
+                for (int i = 0; i < min(quad, 2); ++i)
+#pragma unroll
+                    for (int w = 0; w < PW; ++w) cut_bf16(ar[2 * w], ar[2 * w + 1]);
+#pragma unroll
+                for (int w = 0; w < PW; ++w)
+                    pk[w] = __byte_perm(__float_as_uint(ar[2 * w]), __float_as_uint(ar[2 * w + 1]), 0x7632);
+            }
+            if constexpr (kCols) {
                 tmem_st4(p_addr + (uint32_t)(c * PW), pk);
                 tmem_st4(p_addr + 64u + (uint32_t)(c * PW), p2);
                 tmem_st4(tmem + lane_addr + kThirdTerm<kO> + ((uint32_t)x + dbl) * 64u + (uint32_t)(c * PW), p3);
-            } else if constexpr (kTerms == 2) {
-                tmem_st8(p_addr + (uint32_t)(c * PW), pk);
-                tmem_st8(p_addr + 64u + (uint32_t)(c * PW), p2);
             } else {
                 tmem_st16(p_addr + (uint32_t)(c * PW), pk);
             }
@@ -759,6 +773,10 @@ __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, u
         const float w_a = l_run > 0.f ? ex2(m_run - m) : 0.f;
         const float w_b = l_b > 0.f ? ex2(m_b - m) : 0.f;
         const uint32_t colO_b = kColO + HD;
+        // (terms in rows: quads 1 and 2 leave their terms' O in the Q_B tile, 132 floats a row, and
+        // quad 0 adds them to its own)
+        constexpr bool kRows = kTerms > 1 && kKpp;
+        const uint32_t terms = stage + (uint32_t)TILE + 12288u + (uint32_t)(lane & 15) * 528u;
 #pragma unroll 1
         for (int c = 0; c < 8; ++c) {
             uint32_t oa[16], ob[16];
@@ -771,9 +789,43 @@ __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, u
                 const float vb = w_b != 0.f ? w_b * __uint_as_float(ob[e]) : 0.f;   //  is never read)
                 oa[e] = __float_as_uint(va + vb);
             }
-            tmem_st16(tmem + lane_addr + colO + c * 16, oa);
+            if (kRows && quad > 0) {
+                if (quad < 3 && lane < 16)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        sts128_(terms + (uint32_t)((quad - 1) * 16 * 528 + c * 64 + k * 16),
+                                make_uint4(oa[4 * k], oa[4 * k + 1], oa[4 * k + 2], oa[4 * k + 3]));
+            } else {
+                tmem_st16(tmem + lane_addr + colO + c * 16, oa);
+            }
         }
         tmem_st_wait();
+        if constexpr (kRows) {
+            asm volatile("bar.sync 2, 128;" ::: "memory");
+            if (quad == 0) {
+#pragma unroll 1
+                for (int c = 0; c < 8; ++c) {
+                    uint32_t oa[16];
+                    uint4 t2[4], t3[4];
+                    tmem_ld16(tmem + lane_addr + colO + c * 16, oa);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        t2[k] = lds128(terms + (uint32_t)(c * 64 + k * 16));
+                        t3[k] = lds128(terms + (uint32_t)(16 * 528 + c * 64 + k * 16));
+                    }
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) {
+                        // (a value beyond fp32 is in the first term; 0 in the others times it is not)
+                        const float o1 = __uint_as_float(oa[e]);
+                        const float rest = __uint_as_float(word_of(t2[e / 4], e % 4)) + __uint_as_float(word_of(t3[e / 4], e % 4));
+                        oa[e] = __float_as_uint(fabsf(o1) < CUDART_INF_F ? o1 + rest : o1);
+                    }
+                    tmem_st16(tmem + lane_addr + colO + c * 16, oa);
+                }
+                tmem_st_wait();
+            }
+        }
         l_run = w_a * l_run + w_b * l_b;
         m_run = m;
     }
@@ -1044,7 +1096,6 @@ __device__ __forceinline__ void mma_issuer(const TcParams& P, uint32_t tmem, uin
 // that one half's softmax overlaps the other's MMAs as two query tiles' do (warpgroup A merges
 // the halves at the end).  Issue order: S(0), S(1), then per key tile j: P(j).V(j), S(j + 2)
 // on the same half (in issue order after the P.V that reads the P it overwrites).
-template <bool kTwo>
 __device__ __forceinline__ void mma_issuer_kpp(const TcParams& P, uint32_t tmem, uint32_t sQ, uint32_t sK,
                                                uint32_t sV, uint32_t sBar, int n_kv, int q_ready,
                                                uint32_t q_par, RingState& st, bool wait_oe, uint32_t oe_par,
@@ -1094,11 +1145,6 @@ __device__ __forceinline__ void mma_issuer_kpp(const TcParams& P, uint32_t tmem,
         for (int kk = 0; kk < BN / 16; ++kk)
             mma_bf16_ts(x ? tO_b : tO_a, (x ? tS_b : tS_a) + (uint32_t)kk * 8u,
                         dv + (uint64_t)((kk * 2048) >> 4), idO, kk > 0 || j >= 2 ? 1u : 0u);
-        if constexpr (kTwo)               // the weights' second term, over the same V
-#pragma unroll
-            for (int kk = 0; kk < BN / 16; ++kk)
-                mma_bf16_ts(x ? tO_b : tO_a, (x ? tS_b : tS_a) + 64u + (uint32_t)kk * 8u,
-                            dv + (uint64_t)((kk * 2048) >> 4), idO, 1u);
         mma_commit(bar(B_VE + vs));
         vph ^= vs == VSTAGES - 1 ? 1u : 0u;
         vs = vs == VSTAGES - 1 ? 0 : vs + 1;
@@ -1127,14 +1173,6 @@ __device__ __forceinline__ void cp_async_wait() {
 // generic-proxy writes to shared memory become visible to the tensor core's (async) reads
 __device__ __forceinline__ void fence_proxy_async() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-__device__ __forceinline__ uint4 lds128(uint32_t a) {
-    uint4 v;
-    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-                 : "r"(a)
-                 : "memory");
-    return v;
 }
 __device__ __forceinline__ void sts128(uint32_t a, const uint4& v) {
     asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z),
@@ -1983,8 +2021,10 @@ __global__ void __launch_bounds__(256) suffix_angles_kernel(const __grid_constan
 }
 
 // A decode CTA's queries: the softmax warps (ts = 0..255) form the angles of the new token's
-// position in `tab` and turn the G live rows of the query tile in shared memory, then tell the MMA
-// issuer (B_QR).  The suffix kernel's angles and rounding.
+// position in `tab` and turn the G live rows of the query tile in shared memory (kTerms > 1: and
+// repeat them at rows 32 and 64, softmax_tile), then tell the MMA issuer (B_QR).  The suffix kernel's
+// angles and rounding.
+template <int kTerms>
 __device__ __forceinline__ void decode_turn_queries(const DecodeTcParams& X, int ts, int64_t pos, uint32_t sQ,
                                                     float2* tab, uint32_t sBar, volatile uint32_t* abort) {
     const TcParams& P = X.t;
@@ -2005,8 +2045,11 @@ __device__ __forceinline__ void decode_turn_queries(const DecodeTcParams& X, int
             xo[w] = f2_to_bf2(gx.x, gx.y);
             yo[w] = f2_to_bf2(gy.x, gy.y);
         }
-        sts128(a0, make_uint4(xo[0], xo[1], xo[2], xo[3]));
-        sts128(a0 + HALF_TILE, make_uint4(yo[0], yo[1], yo[2], yo[3]));
+#pragma unroll
+        for (int i = 0; i < kTerms; ++i) {
+            sts128(a0 + (uint32_t)(i * 32 * 128), make_uint4(xo[0], xo[1], xo[2], xo[3]));
+            sts128(a0 + (uint32_t)(i * 32 * 128) + HALF_TILE, make_uint4(yo[0], yo[1], yo[2], yo[3]));
+        }
     }
     fence_proxy_async();
     mbar_arrive(sBar + 8u * B_QR);
@@ -2016,9 +2059,13 @@ __device__ __forceinline__ void decode_turn_queries(const DecodeTcParams& X, int
 // and written to the cache (with the row's position, and zeros after it up to the tile's edge when
 // nothing finite is there yet), and, once the tile has landed, written into it in shared memory (the
 // copy engine may have read the cache before or after): the tile's loads complete barriers of their
-// own (B_KL, B_VL), and this warp then fills the stage's for the MMA issuer.  It takes a kernel of
+// own (B_KL, B_VL), and this warp then fills the stage's for the MMA issuer.  kTerms > 1: the tile's
+// V rows after the new one are zeros whatever the cache holds there (an earlier call may have written
+// a value beyond fp32, and a masked key's weight of 0 times that is not 0; the CUDA cores read no row
+// after the new one).  It takes a kernel of
 // its own (3.5 us, then the attention's start behind it) out of every step: 16 requests of 1163 keys
 // 20.7 -> 18.5 us, one of 131k keys 91.8 -> 89.6.
+template <int kTerms>
 __device__ __forceinline__ void decode_append(const DecodeTcParams& X, int lane, int l, int bl, int b, int hk, int n_kv,
                                               int64_t pos, uint32_t sK, uint32_t sV, float2* tab, uint32_t sBar,
                                               volatile uint32_t* abort) {
@@ -2075,7 +2122,7 @@ __device__ __forceinline__ void decode_append(const DecodeTcParams& X, int lane,
         } else if (!is_k && lane >= 8 && c < 16) {
             sts128(tile + (uint32_t)((c >> 3) * HALF_TILE) + sw_off(rt, c & 7), a);
         }
-        if (pad)
+        if (pad || (kTerms > 1 && !is_k))
             for (int i = lane; i < (BN - 1 - rt) * 16; i += 32)
                 sts128(tile + (uint32_t)(((i >> 3) & 1) * HALF_TILE) + sw_off(rt + 1 + (i >> 4), i & 7), z);
         fence_proxy_async();
@@ -2258,7 +2305,7 @@ __device__ __forceinline__ void attn_tc_body(const typename KernelParams<kFused,
                     if (ps.has_b)
                         mma_issuer<true, D>(P, tmem, sQ, sK, sV, sBar, ps.n_kv, B_Q, q_par, st, pi > 0, oe_par, abort);
                     else if (kKpp)                                        // key tiles ping-pong (one pair)
-                        mma_issuer_kpp<(kTerms > 1)>(P, tmem, sQ, sK, sV, sBar, ps.n_kv, B_QR, q_par, st, pi > 0, oe_par, abort);
+                        mma_issuer_kpp(P, tmem, sQ, sK, sV, sBar, ps.n_kv, B_QR, q_par, st, pi > 0, oe_par, abort);
                     else
                         mma_issuer<false, D>(P, tmem, sQ, sK, sV, sBar, ps.n_kv, B_Q, q_par, st, pi > 0, oe_par, abort);
                 }
@@ -2271,7 +2318,7 @@ __device__ __forceinline__ void attn_tc_body(const typename KernelParams<kFused,
             // ------------------------------------------------------------ new row (decode)
             if constexpr (kKpp)
                 if (append)
-                    decode_append(KP, lane, l, bl, b, hk, n_kv, (int64_t)P.req[bl].l_req + P.req[bl].t0, sK, sV,
+                    decode_append<kTerms>(KP, lane, l, bl, b, hk, n_kv, (int64_t)P.req[bl].l_req + P.req[bl].t0, sK, sV,
                                   reinterpret_cast<float2*>(smem + TILE + 8192), sBar, abort);
             // ------------------------------------------------------------ V loader (fused)
             if constexpr (kFused)
@@ -2321,7 +2368,7 @@ __device__ __forceinline__ void attn_tc_body(const typename KernelParams<kFused,
                 const bool kpp = kKpp && ps.n_kv >= 1;
                 if constexpr (kKpp)
                     if (kpp)
-                        decode_turn_queries(KP, (int)threadIdx.x - 128, (int64_t)P.req[bl].l_req + P.req[bl].t0, sQ,
+                        decode_turn_queries<kTerms>(KP, (int)threadIdx.x - 128, (int64_t)P.req[bl].l_req + P.req[bl].t0, sQ,
                                             reinterpret_cast<float2*>(smem + TILE + 4096), sBar, abort);
                 if (x == 0 || ps.has_b || kpp) {
                     softmax_tile<true, kSif, kKpp, D, kColO, false, kTerms>(P, tmem, sBar, x, warp & 3, lane, x && !kpp ? ps.t0b : ps.t0a, l, bl,
@@ -2376,10 +2423,10 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc64_sif_kernel(const __grid
 
 // Decode steps (AttnParams::key_pingpong): the plain kernel whose last pair, when it has one
 // query tile, splits its key tiles between the two softmax warpgroups.
-// kTwo: weights of two bf16 terms.
-template <bool kTwo>
+// kExact: fp32 weights, as three bf16 terms.
+template <bool kExact>
 __global__ void __launch_bounds__(kThreads, 1) attn_tc_decode_kernel(const __grid_constant__ DecodeTcParams KP) {
-    attn_tc_body<false, false, false, true, HD, kTwo ? 2 : 1>(KP);
+    attn_tc_body<false, false, false, true, HD, kExact ? 3 : 1>(KP);
 }
 
 // One query tile a CTA (the solo kernel), in two forms.
@@ -2623,13 +2670,13 @@ __global__ void __launch_bounds__(kSoloThreads, kAlone ? 1 : 2) attn_solo_kernel
 }
 
 // The kernel of an instantiation.
-// kSolo: 0, or the solo kernel shared (1) or alone (2).  kTwo (decode): weights of two bf16 terms.
-template <bool kFused, bool kMulti, bool kSif, bool kKpp = false, int D = HD, int kSolo = 0, bool kTwo = false>
+// kSolo: 0, or the solo kernel shared (1) or alone (2).  kExact (decode): fp32 weights.
+template <bool kFused, bool kMulti, bool kSif, bool kKpp = false, int D = HD, int kSolo = 0, bool kExact = false>
 const void* tc_kernel_fn() {
     if constexpr (kSolo != 0) return reinterpret_cast<const void*>(&attn_solo_kernel<kSif, D, kSolo == 2>);
     else if constexpr (D == 64) return reinterpret_cast<const void*>(kSif ? &attn_tc64_sif_kernel : &attn_tc64_kernel);
     else if constexpr (kSif) return reinterpret_cast<const void*>(&attn_tc_sif_kernel);
-    else if constexpr (kKpp) return reinterpret_cast<const void*>(&attn_tc_decode_kernel<kTwo>);
+    else if constexpr (kKpp) return reinterpret_cast<const void*>(&attn_tc_decode_kernel<kExact>);
     else return reinterpret_cast<const void*>(&attn_tc_kernel<kFused, kMulti>);
 }
 
@@ -2779,12 +2826,12 @@ namespace {
 // Host-side preparation shared by the plain and the fused launch: function attributes once
 // per device, the register-split guard, the tensor maps and the scalar parameters.
 template <bool kFused, bool kMulti = false, bool kSif = false, bool kKpp = false, int D = HD, int kSolo = 0,
-          bool kTwo = false>
+          bool kExact = false>
 cudaError_t prepare_tc(const AttnParams& a, TcParams& p, dim3& grid) {
     constexpr int threads = kFused ? kThreadsFused : kThreads;
     constexpr int high = kFused ? kRegsHighFused : kRegsHigh;
     constexpr int low_total = kFused ? 128 * (kRegsLowFused + kRegsLoadFused) : 128 * kRegsLow;
-    const void* const kernel = tc_kernel_fn<kFused, kMulti, kSif, kKpp, D, kSolo, kTwo>();
+    const void* const kernel = tc_kernel_fn<kFused, kMulti, kSif, kKpp, D, kSolo, kExact>();
     static PerDevice<cudaError_t> smem;
     const cudaError_t smem_err = opt_in_smem(smem, kernel, kSolo ? Solo<D, kSolo == 2>::kSmem : Geo<D>::kSmem);
     if (smem_err != cudaSuccess) return smem_err;
@@ -2980,8 +3027,8 @@ cudaError_t launch_attn_tc_decode(const AttnParams& a, const DecodeAppend& d, cu
     if (!d.k_new || !d.v_new || !d.pos || a.d != HD) return cudaErrorInvalidValue;
     DecodeTcParams p;
     dim3 grid;
-    const cudaError_t e = d.two_terms ? prepare_tc<false, false, false, true, HD, 0, true>(a, p.t, grid)
-                                      : prepare_tc<false, false, false, true, HD, 0, false>(a, p.t, grid);
+    const cudaError_t e = d.exact_weights ? prepare_tc<false, false, false, true, HD, 0, true>(a, p.t, grid)
+                                            : prepare_tc<false, false, false, true, HD, 0, false>(a, p.t, grid);
     if (e != cudaSuccess) return e;
     p.k_new = d.k_new;
     p.v_new = d.v_new;
@@ -2991,7 +3038,7 @@ cudaError_t launch_attn_tc_decode(const AttnParams& a, const DecodeAppend& d, cu
     std::memcpy(p.pad_mask, d.pad_mask, sizeof(p.pad_mask));
     p.rope = d.rope;
     before();
-    if (d.two_terms)
+    if (d.exact_weights)
         attn_tc_decode_kernel<true><<<grid, kThreads, kSmemBytes, s>>>(p);
     else
         attn_tc_decode_kernel<false><<<grid, kThreads, kSmemBytes, s>>>(p);

@@ -1378,17 +1378,18 @@ c2kv_status c2kv_decode(c2kv_ctx* c, c2kv_cache* cache, int32_t layer, const voi
         // (short contexts over more units than SMs: its per-CTA start is paid again each wave)
         // the CUDA-core decode kernel, two CTAs per SM, while a group is small: its time grows with
         // the G queries that each key meets, the tensor cores' does not, so at G = 8 these take it
-        // from 3 key tiles as well, with weights of two bf16 terms in place of its fp32 ones.
-        // Measured, CUDA cores / tensor cores with two terms (us a call, one layer, 8 KV heads; key
-        // tiles 3, 9, 18): G = 8, 32 requests 30 / 24, 71 / 43, 123 / 69, 128 requests 88 / 76, 226 /
-        // 136, 405 / 226, but one tile 53 / 59; G = 4, 32 requests 9 tiles 39 / 43, 18 65 / 69 (with one
-        // term 36 and 57).  One term, one wave: 16 requests x 1160 keys 30 / 18, 8 x 32900 212 / 190.
+        // from 3 key tiles as well, its fp32 weights kept (as three bf16 terms).
+        // Measured, CUDA cores / tensor cores with fp32 weights (us a call, one layer, 8 KV heads; key
+        // tiles 3, 9, 18): G = 8, 32 requests 30 / 26, 71 / 40, 123 / 62, 128 requests 88 / 81, 226 /
+        // 128, 405 / 210, but one tile 53 / 63.  G = 4 with two terms of the weights, 32 requests: 9
+        // tiles 39 / 43, 18 65 / 69.  bf16 weights, one wave: 16 requests x 1160 keys 30 / 18, 8 x
+        // 32900 212 / 190.
         const int64_t tiles_max = (n_keys_max + 127) / 128;
         const int32_t group = hq / hkv;
         const bool tc = c->cfg.attn_impl != C2KV_ATTN_SIMT && c2kv::attn_tc_supported(c->cfg.dtype, d, hq, hkv);
-        const bool one_term = c->cfg.attn_impl == C2KV_ATTN_TC || units <= c->sms || tiles_max >= 32;
-        const bool two_terms = tc && !one_term && group >= 8 && tiles_max >= 3;
-        const bool use_tc = tc && (one_term || two_terms);
+        const bool bf16_weights = c->cfg.attn_impl == C2KV_ATTN_TC || units <= c->sms || tiles_max >= 32;
+        const bool exact_weights = tc && !bf16_weights && group >= 8 && tiles_max >= 3;
+        const bool use_tc = tc && (bf16_weights || exact_weights);
         int32_t n_split = 1;
         if (use_tc) {
             // splits per (layer, request, KV head): the fewest waves of one-CTA-per-SM work,
@@ -1504,7 +1505,7 @@ c2kv_status c2kv_decode(c2kv_ctx* c, c2kv_cache* cache, int32_t layer, const voi
                 ap.v_new = v_new;
                 ap.pos = cache->pos;
                 ap.rope = c->turns;
-                ap.two_terms = two_terms ? 1 : 0;
+                ap.exact_weights = exact_weights ? 1 : 0;
                 for (int32_t i = 0; i < nb; ++i)
                     if (pad_from[b0 + i] < edge[b0 + i]) ap.pad_mask[i / 32] |= 1u << (i % 32);
                 ProfScope prof_decode(c, C2KV_PROF_DECODE, true);

@@ -272,7 +272,7 @@ struct DecodeAppend {
     int32_t* pos;            // [rows]
     uint32_t pad_mask[kMaxReq / 32];   // request i of the launch: zero the rows after the new one up
                                        // to the next 128-row boundary
-    int32_t two_terms;       // 1: the weights as two bf16 terms (relative error 2^-16, not 2^-8)
+    int32_t exact_weights;   // 1: fp32 weights (as three bf16 terms), not bf16 ones
     RopeTurns rope;
 };
 cudaError_t launch_attn_tc_decode(const AttnParams& a, const DecodeAppend& d, cudaStream_t s, Hook before = {});
