@@ -10,7 +10,11 @@
 //   S:   per 4 channels RT + 8 16-byte shared loads feed 32 RT FMAs; every 32 channels the
 //        partial dot products are folded, so no sum is a chain of more than 32 terms.
 //   P.V: 32 keys at a time the weights pass through shared memory within the warp; the
-//        products of 32 keys are summed apart and then folded into O.
+//        products of 32 keys are summed apart and then folded into O.  The keys that a row does
+//        not see have a weight of 0 there; where 32 keys' sums are not finite in a tile that some
+//        row does not see whole, they are formed again without such keys (0 times a value of
+//        infinity or NaN, which may be another row's to see, is not 0).  Looking for them takes
+//        1 to 4 % of a call, leaving every such key out by a test a weight took 8 to 10 %.
 // A 16-byte shared load costs a wavefront per half-warp and 128 bytes of different addresses:
 // with 4 x 8 lanes every load above costs the least, two, so 128 FMAs take 20 to 24 (with lanes
 // 2 x 16 the loads of K and V cost four, and shared memory bound the kernel).
@@ -30,6 +34,7 @@
 #include <math_constants.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "internal.cuh"
 #include "per_device.cuh"
@@ -223,12 +228,16 @@ __device__ __forceinline__ void attention_core(const Job& job, int row0, int ns,
         float alpha[RT];
 #pragma unroll
         for (int i = 0; i < RT; ++i) {
+            uint32_t hidden = 0u;                          // bit j: the row does not see key tx + 8 j
             if (!whole) {
                 const auto row = job.row(row0 + r0 + 4 * i);
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     const int key = k0 + tx + 8 * j;
-                    if (key >= job.nkeys || !job.sees(row, key)) s[i][j] = -CUDART_INF_F;
+                    if (key >= job.nkeys || !job.sees(row, key)) {
+                        s[i][j] = -CUDART_INF_F;
+                        hidden |= 1u << j;
+                    }
                 }
             }
             float mx = s[i][0];
@@ -241,7 +250,10 @@ __device__ __forceinline__ void attention_core(const Job& job, int row0, int ns,
             alpha[i] = exp2f(m[i] - ms);
             m[i] = mn;
 #pragma unroll
-            for (int j = 0; j < 8; ++j) s[i][j] = exp2f(fmaf(s[i][j], job.scale_log2, -ms));
+            for (int j = 0; j < 8; ++j) {
+                s[i][j] = exp2f(fmaf(s[i][j], job.scale_log2, -ms));
+                if (hidden >> j & 1u) s[i][j] = -0.f;
+            }
             l[i] = l[i] * alpha[i] + (((s[i][0] + s[i][1]) + (s[i][2] + s[i][3])) +
                                       ((s[i][4] + s[i][5]) + (s[i][6] + s[i][7])));   // this lane's keys
         }
@@ -250,19 +262,14 @@ __device__ __forceinline__ void attention_core(const Job& job, int row0, int ns,
 #pragma unroll
         for (int half = 0; half < 2; ++half) {
             float4 pv[RT][H];
+            auto clear = [&] {
 #pragma unroll
-            for (int i = 0; i < RT; ++i)
+                for (int i = 0; i < RT; ++i)
 #pragma unroll
-                for (int h = 0; h < H; ++h) pv[i][h] = make_float4(0.f, 0.f, 0.f, 0.f);
-            __syncwarp();                                  // the weights before these are read
-#pragma unroll
-            for (int i = 0; i < RT; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    *reinterpret_cast<float*>(pb + 4 * i * kCorePPitch + (tx + 8 * j) * 4) = s[i][4 * half + j];
-            __syncwarp();
-#pragma unroll 2
-            for (int u = 0; u < 32; u += 4) {              // keys 32 half + u .. + 3
+                    for (int h = 0; h < H; ++h) pv[i][h] = make_float4(0.f, 0.f, 0.f, 0.f);
+            };
+            // keys 32 half + u .. + 3; `masked`: a hidden key's weight, -0, is left out
+            auto weigh = [&](int u, auto masked) {
                 float4 p[RT];
 #pragma unroll
                 for (int i = 0; i < RT; ++i) p[i] = ld4(pb + 4 * i * kCorePPitch + u * 4);
@@ -274,6 +281,7 @@ __device__ __forceinline__ void attention_core(const Job& job, int row0, int ns,
 #pragma unroll
                     for (int i = 0; i < RT; ++i) {
                         const float w = e == 0 ? p[i].x : e == 1 ? p[i].y : e == 2 ? p[i].z : p[i].w;
+                        if (decltype(masked)::value && __float_as_uint(w) == 0x80000000u) continue;
 #pragma unroll
                         for (int h = 0; h < H; ++h) {
                             pv[i][h].x = fmaf(w, v[h].x, pv[i][h].x);
@@ -282,6 +290,30 @@ __device__ __forceinline__ void attention_core(const Job& job, int row0, int ns,
                             pv[i][h].w = fmaf(w, v[h].w, pv[i][h].w);
                         }
                     }
+                }
+            };
+            clear();
+            __syncwarp();                                  // the weights before these are read
+#pragma unroll
+            for (int i = 0; i < RT; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    *reinterpret_cast<float*>(pb + 4 * i * kCorePPitch + (tx + 8 * j) * 4) = s[i][4 * half + j];
+            __syncwarp();
+#pragma unroll 2
+            for (int u = 0; u < 32; u += 4) weigh(u, std::false_type{});
+            if (!whole) {
+                float4 z = make_float4(0.f, 0.f, 0.f, 0.f);      // zeros, or NaN when some sum is not finite
+#pragma unroll
+                for (int i = 0; i < RT; ++i)
+#pragma unroll
+                    for (int h = 0; h < H; ++h)
+                        z = make_float4(fmaf(pv[i][h].x, 0.f, z.x), fmaf(pv[i][h].y, 0.f, z.y),
+                                        fmaf(pv[i][h].z, 0.f, z.z), fmaf(pv[i][h].w, 0.f, z.w));
+                if (__any_sync(0xffffffffu, (z.x + z.y) + (z.z + z.w) != 0.f)) {
+                    clear();
+#pragma unroll 1
+                    for (int u = 0; u < 32; u += 4) weigh(u, std::true_type{});
                 }
             }
 #pragma unroll
