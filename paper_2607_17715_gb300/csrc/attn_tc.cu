@@ -176,6 +176,9 @@ struct TcParams {                // CUtensorMap members carry their own alignmen
     uint32_t* tickets;       // null, or per-unit counters: the last split merges (plain kernel)
     int32_t sif_k;           // 0, or extraction C2 rows with ratio k (plain kernel, one split)
     const float2* q_cs;      // null, or (solo kernel) the queries are before RoPE: AttnParams::q_cs
+    const void* q;           // what tm_q, tm_k and tm_v cover (64 channels: redo_rows reads them)
+    const void* k;
+    const void* v;
     ReqParam req[kMaxReq];
 };
 
@@ -575,6 +578,72 @@ __device__ __forceinline__ PairSpan tile_span(const TcParams& P, int qt, int sp,
 
 // ------------------------------------------------------------------ kernel
 
+// Rows of a 64-channel tile whose O is not finite (`bad`: of a warp's 32 rows), formed again by the
+// warp in fp32: O = sum_j w_j V_j over the keys of its span that the row sees, w_j against the row's
+// final maximum m, times inv.  A value of infinity or NaN gives NaN in the tensor cores' sums where it
+// should not: in rows that do not see it (their weight of 0 times it), and in rows that do (the second
+// and third term of a weight may be 0).  The CUDA cores, which these heads ran on, give the sums'
+// own result, and so does this.  It takes a warp some 0.1 us a key and row, for such values only.
+// sbase: the tile in shared memory, or 0: the row goes to out or to its split's partial.
+template <bool kSif>
+__device__ __noinline__ void redo_rows(const TcParams& P, uint32_t bad, int quad, int lane, int t0, int l, int bl, int b,
+                                       int hk, int sp, const PairSpan span, float m_run, float inv, uint32_t sbase) {
+    using bf = __nv_bfloat16;
+    auto ld = [](const void* p, int64_t i) {
+        return __uint_as_float((uint32_t)__ldcg(static_cast<const unsigned short*>(p) + i) << 16);
+    };
+    const int G = P.group, s_r = P.req[bl].n_slots + P.req[bl].t0;
+    const int64_t kv0 = (((int64_t)(P.layer0 + l) * P.rows + P.req[bl].row_base) * P.hkv + hk) * 64 + lane;
+    for (; bad != 0u; bad &= bad - 1u) {
+        const int i = __ffs(bad) - 1, r = quad * 32 + i;
+        const int t = t0 + r / G, g = r - (r / G) * G;
+        const float m = __shfl_sync(0xffffffffu, m_run, i), iv = __shfl_sync(0xffffffffu, inv, i);
+        const int64_t row_id = (((int64_t)l * P.batch_total + b) * P.sq_pitch + t) * P.hq + hk * G + g;
+        // lane: channels lane and lane + 32, a RoPE pair
+        float q0 = ld(P.q, row_id * 64 + lane), q1 = ld(P.q, row_id * 64 + lane + 32);
+        if (P.q_cs != nullptr) {
+            float x, y;
+            rotate1(q0, q1, P.q_cs[(int64_t)t * 32 + lane], x, y);
+            q0 = __bfloat162float(__float2bfloat16_rn(x));
+            q1 = __bfloat162float(__float2bfloat16_rn(y));
+        }
+        const int lim = s_r + t;
+        const int64_t blo = kSif ? (int64_t)t * P.sif_k : 0;
+        float o0 = 0.f, o1 = 0.f;
+        for (int j = 0; j < span.n_kv; ++j) {
+            const int k0 = (kSif ? span_tile(span, j) : span.j_base + j) * BN, k1 = min(k0 + BN, lim + 1);
+#pragma unroll 4
+            for (int key = k0; key < k1; ++key) {
+                if (kSif && key < s_r && key >= P.sif_k && (key < blo || key >= blo + P.sif_k)) continue;
+                const int64_t at = kv0 + (int64_t)key * P.hkv * 64;
+                float s = fmaf(q0, ld(P.k, at), q1 * ld(P.k, at + 32));
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+                const float w = ex2(fmaf(s, P.scale_log2, -m));
+                o0 = fmaf(w, ld(P.v, at), o0);
+                o1 = fmaf(w, ld(P.v, at + 32), o1);
+            }
+        }
+        o0 *= iv;
+        o1 *= iv;
+        if (P.n_split > 1) {
+            float* dst = P.part_o + ((int64_t)sp * P.lq * P.batch_total * P.sq * P.hq + row_id) * 64 + lane;
+            dst[0] = o0;
+            dst[32] = o1;
+        } else if (sbase != 0u) {
+            const uint32_t at = sbase + (uint32_t)(r * 128 + (((lane >> 3) ^ (r & 7)) << 4) + (lane & 7) * 2);
+            const unsigned short h0 = __bfloat16_as_ushort(__float2bfloat16_rn(o0));
+            const unsigned short h1 = __bfloat16_as_ushort(__float2bfloat16_rn(o1));
+            asm volatile("st.shared.u16 [%0], %1;" ::"r"(at), "h"(h0) : "memory");
+            asm volatile("st.shared.u16 [%0], %1;" ::"r"(at ^ 64u), "h"(h1) : "memory");   // chunk + 4
+        } else {
+            bf* dst = static_cast<bf*>(P.out) + row_id * 64 + lane;
+            dst[0] = __float2bfloat16_rn(o0);
+            dst[32] = __float2bfloat16_rn(o1);
+        }
+    }
+}
+
 // One softmax thread's work on tile x (A or B) for every key tile of a pair, then its
 // epilogue.  r = TMEM lane (row within the tile), t0 = first suffix token of the tile.
 // sf_base: S_x tiles completed in earlier pairs (phase count); od_par: the phase of B_OD that
@@ -841,6 +910,24 @@ __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, u
     const float inv = any ? 1.0f / l_run : 0.f;
     const int64_t row_id = (((int64_t)l * P.batch_total + b) * P.sq_pitch + t) * P.hq + hk * G + g;
     const int64_t lse_id = (((int64_t)l * P.batch_total + b) * P.hq + hk * G + g) * P.sq_pitch + t;
+    // 64 channels: rows whose O is not finite though their sum of weights is (after the row is written)
+    constexpr bool kRedo = D == 64;
+    float fin[2] = {0.f, 0.f};                    // zeros, or NaN
+    auto look = [&](const uint32_t (&ov)[32]) {
+        if constexpr (kRedo)
+#pragma unroll
+            for (int e = 0; e < 32; ++e) fin[e & 1] = fmaf(__uint_as_float(ov[e]), 0.f, fin[e & 1]);
+    };
+    auto redo = [&](uint32_t sbase) {
+        if constexpr (kRedo) {
+            const bool row = t < P.sq && l_run > 0.f && l_run < CUDART_INF_F && fin[0] + fin[1] != 0.f;
+            const uint32_t bad = __ballot_sync(0xffffffffu, row);
+            if (bad != 0u) {
+                __syncwarp();                     // (the rows have been written by their own threads)
+                redo_rows<kSif>(P, bad, quad, lane, t0, l, bl, b, hk, sp, span, m_run, inv, sbase);
+            }
+        }
+    };
     if (P.n_split == 1 && stage != 0u && n_kv > 0) {
         const uint32_t sbase = stage + (uint32_t)(x * Geo<D>::kTile);
 #pragma unroll
@@ -848,6 +935,7 @@ __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, u
             uint32_t ov[32];
             tmem_ld32(tmem + lane_addr + colO + c * 32, ov);
             tmem_ld_wait();
+            look(ov);
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 uint4 w;
@@ -865,6 +953,7 @@ __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, u
             tc_fence_before();
             mbar_arrive(bar(B_OE));
         }
+        redo(sbase);
         // the rows visible to the TMA engine, every row of the tile written, then one store per
         // 64-column block (tokens past the suffix fall outside the map and are dropped)
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -893,6 +982,7 @@ __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, u
             uint32_t ov[32];
             tmem_ld32(tmem + lane_addr + colO + c * 32, ov);
             tmem_ld_wait();
+            look(ov);
             if (t < P.sq) {
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
@@ -912,6 +1002,7 @@ __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, u
         }
         if (P.lse != nullptr && t < P.sq)
             P.lse[lse_id] = (m_run + log2f(l_run)) * 0.69314718055994531f;
+        redo(0u);
     } else {
         // partial over this split's keys: normalised O (fp32) and its log2-domain lse
         const int64_t part_rows = (int64_t)P.lq * P.batch_total * P.sq * P.hq;
@@ -926,18 +1017,23 @@ __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, u
 #pragma unroll
                 for (int e = 0; e < 32; ++e) ov[e] = 0u;
             }
+            look(ov);
             if (t < P.sq) {
 #pragma unroll
                 for (int q8 = 0; q8 < 4; ++q8) {
                     uint32_t w[8];
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) w[e] = __float_as_uint(__uint_as_float(ov[q8 * 8 + e]) * inv);
+                    for (int e = 0; e < 8; ++e) {
+                        w[e] = __float_as_uint(__uint_as_float(ov[q8 * 8 + e]) * inv);
+                        if (kRedo && l_run == 0.f) w[e] = 0u;    // (none of these keys is seen)
+                    }
                     stg256(orow + c * 32 + q8 * 8, w);
                 }
             }
         }
         if (t < P.sq)
             P.part_lse[(int64_t)sp * part_rows + lse_id] = any ? m_run + log2f(l_run) : -CUDART_INF_F;
+        redo(0u);
         if constexpr (kMerge)
             if (P.tickets != nullptr) split_merge<D>(P, sBar, x, r, t0, l, b, hk);
     }
@@ -2889,6 +2985,9 @@ cudaError_t prepare_tc(const AttnParams& a, TcParams& p, dim3& grid) {
     p.tickets = kFused || p.n_split == 1 || p.n_split > kMaxMergeSplits ? nullptr : a.tickets;
     p.sif_k = a.sif_k;
     p.q_cs = a.q_cs;
+    p.q = a.q_rot;
+    p.k = a.cache_k;
+    p.v = a.cache_v;
     if (a.q_cs != nullptr && !kSolo) return cudaErrorInvalidValue;
 
     if (kSif != (a.sif_k > 0) || a.sif_k < 0 || (kSif && (kFused || p.n_split != 1))) return cudaErrorInvalidValue;

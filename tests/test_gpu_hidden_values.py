@@ -120,3 +120,17 @@ def test_attend_large(dtype, d, hq, hkv):
 @pytest.mark.parametrize("n,k", [(150, 4), (333, 16)])
 def test_extract(dtype, d, hq, hkv, n, k):
     check_extract(dtype, d, hq, hkv, n, k)
+
+
+# bf16 heads of 64 channels on the tensor cores, in each form of the kernel
+@pytest.mark.parametrize("hq,hkv", [(32, 8), (16, 16), (32, 4)])
+@pytest.mark.parametrize("form", [dict(), dict(layers=30), dict(pairs=1), dict(split=3), dict(pairs=2, n=200), dict(split=0, slots=2500)],
+                         ids=["alone", "shared", "pair", "merged", "pairs_in_turn", "split"])
+def test_attend_heads64(hq, hkv, form):
+    check_attend("bf16", 64, hq, hkv, bits=False, **form)
+
+
+@pytest.mark.parametrize("hq,hkv", [(32, 8), (16, 16)])
+@pytest.mark.parametrize("n,k,pairs", [(150, 4, 0), (333, 16, 0), (333, 16, 1)])
+def test_extract_heads64(hq, hkv, n, k, pairs):
+    check_extract("bf16", 64, hq, hkv, n, k, bits=False, pairs=pairs, layers=2)
