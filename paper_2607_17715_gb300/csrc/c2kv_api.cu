@@ -890,8 +890,16 @@ cudaError_t attend_run(c2kv_ctx* c, c2kv_cache* cache, int32_t layer0, int32_t l
             const size_t rows = (size_t)lq * B * n_suffix * c->cfg.n_q_heads;
             e = pool_alloc(c, reinterpret_cast<void**>(&part),
                            (size_t)n_split * rows * (c->cfg.head_dim + 1) * sizeof(float));
+            if (e == cudaErrorMemoryAllocation && c->cfg.attn_split == 0) {
+                // splits that no one asked for are done without
+                (void)cudaGetLastError();
+                part = nullptr;
+                n_split = 1;
+                merge_launch = false;
+                e = cudaSuccess;
+            }
             // the pair kernel merges the splits itself (per-unit counters)
-            if (e == cudaSuccess && !merge_launch && n_split <= c2kv::kMaxMergeSplits)
+            if (e == cudaSuccess && n_split > 1 && !merge_launch && n_split <= c2kv::kMaxMergeSplits)
                 e = tickets_ready(c, (size_t)c2kv::attn_tc_units(c->cfg.n_q_heads, c->cfg.n_kv_heads, n_suffix,
                                                                  lq, std::min<int32_t>(B, c2kv::kMaxReq)));
             if (e != cudaSuccess) {
@@ -1229,6 +1237,7 @@ c2kv_status c2kv_compose_attend(c2kv_ctx* c, int32_t batch, const int32_t* req_p
         // PRE_ROPE slots turn by a position per slot, which the fused loaders' per-occurrence
         // angle tables do not hold: compose, then attend
         fuse = fuse && !host_chunks && c->cfg.storage == C2KV_STORAGE_LOCAL_ROPE;
+        const bool fusable = fuse;
         fuse = fuse && (forced || fused_pays(c, cache, occ, req_ptr, n_suffix));
         cudaError_t e = cudaSuccess;
         // suffix tensors and outputs in pinned host memory: copied through device scratch (the
@@ -1249,7 +1258,7 @@ c2kv_status c2kv_compose_attend(c2kv_ctx* c, int32_t batch, const int32_t* req_p
         const void* v_d = pipelined ? v_suf : io.v;
         void* out_d = pipelined ? out : io.out;
         float* lse_d = pipelined ? lse : io.lse;
-        if (fuse) {
+        auto run_fused = [&]() -> cudaError_t {
             static thread_local c2kv::FusedSpec f;   // 13 KB: kept off the stack
             f.pool_k = c->pool_k;
             f.pool_v = c->pool_v;
@@ -1266,17 +1275,20 @@ c2kv_status c2kv_compose_attend(c2kv_ctx* c, int32_t batch, const int32_t* req_p
             // (cos, sin) per layer, occurrence and frequency, then per suffix token and frequency
             float2* occ_cs = nullptr;
             const size_t n_occ_cs = (size_t)c->cfg.layers * std::max<size_t>(occ.size(), 1) * 64;
-            e = pool_alloc(c, reinterpret_cast<void**>(&occ_cs),
-                           (n_occ_cs + (size_t)batch * n_suffix * 64) * sizeof(float2));
-            if (e == cudaSuccess) {
-                f.occ_cs = occ_cs;
-                f.sfx_cs = occ_cs + n_occ_cs;
-                f.pairs_in_turn = pairs_in_turn ? 1 : 0;
-                f.k_suf = k_d;
-                f.v_suf = v_d;
-                e = attend_run(c, cache, 0, c->cfg.layers, q_d, k_d, v_d, n_suffix, out_d, lse_d, &f);
-                pool_free(c, occ_cs);
-            }
+            const cudaError_t ea = pool_alloc(c, reinterpret_cast<void**>(&occ_cs),
+                                              (n_occ_cs + (size_t)batch * n_suffix * 64) * sizeof(float2));
+            if (ea != cudaSuccess) return ea;
+            f.occ_cs = occ_cs;
+            f.sfx_cs = occ_cs + n_occ_cs;
+            f.pairs_in_turn = pairs_in_turn ? 1 : 0;
+            f.k_suf = k_d;
+            f.v_suf = v_d;
+            const cudaError_t er = attend_run(c, cache, 0, c->cfg.layers, q_d, k_d, v_d, n_suffix, out_d, lse_d, &f);
+            pool_free(c, occ_cs);
+            return er;
+        };
+        if (fuse) {
+            e = run_fused();
         } else if (pipelined) {
             e = compose_attend_pipelined(c, cache, occ, q, k_suf, v_suf, n_suffix, out, lse);
         } else if (!c->prof) {
@@ -1285,6 +1297,11 @@ c2kv_status c2kv_compose_attend(c2kv_ctx* c, int32_t batch, const int32_t* req_p
             e = compose_launch(c, cache, occ);
             if (e == cudaSuccess)
                 e = attend_run(c, cache, 0, c->cfg.layers, q_d, k_d, v_d, n_suffix, out_d, lse_d, nullptr);
+        }
+        if (e == cudaErrorMemoryAllocation && fusable && !fuse) {
+            // no room for the turned queries, which the fused kernel does not need
+            (void)cudaGetLastError();
+            e = run_fused();
         }
         if (e == cudaSuccess && !pipelined) e = suffix_io_out(c, io, out, lse, 0, c->cfg.layers);
         if (!pipelined) pool_free(c, io.scratch);

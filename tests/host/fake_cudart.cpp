@@ -14,7 +14,7 @@
 namespace fake {
 int device = 0;
 std::vector<Launch> launches;
-size_t alloc_limit = SIZE_MAX;
+std::function<bool(size_t)> alloc_fails = [](size_t) { return false; };
 std::function<int(const std::string&)> registers = [](const std::string&) { return 168; };
 std::function<int(int)> sms = [](int) { return 152; };
 
@@ -47,7 +47,7 @@ cudaError_t launch(const void* fn, dim3 grid, dim3 block, size_t smem) {
 }
 cudaError_t allocate(void** p, size_t bytes) {
     *p = nullptr;
-    if (bytes > alloc_limit) return answer(cudaErrorMemoryAllocation);
+    if (alloc_fails(bytes)) return answer(cudaErrorMemoryAllocation);
     *p = std::aligned_alloc(256, (bytes + 511) / 256 * 256);
     return cudaSuccess;
 }

@@ -16,7 +16,7 @@ struct Launch {
 };
 extern int device;                                             // the current device
 extern std::vector<Launch> launches;
-extern size_t alloc_limit;                                     // larger allocations fail
+extern std::function<bool(size_t)> alloc_fails;                // whether an allocation of so many bytes fails
 extern std::function<int(const std::string&)> registers;       // compiled register count of a kernel
 extern std::function<int(int)> sms;                            // SMs of a device
 std::vector<std::string> kernel_names();                       // of every kernel of the library

@@ -144,6 +144,34 @@ void second_device() {
     }
 }
 
+// Scratch that only makes a call faster is done without when it cannot be had: the partials of automatic
+// key-range splits,
+void no_partials() {
+    Context one({kBf16, 32, 8, 128}), forced({kBf16, 32, 8, 128}, 4);
+    c2kv_cache* cache = one.compose(1, 8192, 64);
+    c2kv_cache* cache4 = forced.compose(1, 8192, 64);
+    CHECK(one.attend(cache, 64) == C2KV_OK, "attend");
+    CHECK(fake::launched("attn_combine_kernel"), "the call is split when there is memory");
+    fake::launches.clear();
+    fake::alloc_fails = [](size_t bytes) { return bytes > 64 * 32 * 128 * 2; };          // the turned queries fit
+    CHECK(one.attend(cache, 64) == C2KV_OK, "attend without partials: %s", c2kv_last_error(one.ctx));
+    CHECK(fake::launched("attn_solo_kernel") && !fake::launched("attn_combine_kernel"), "one split");
+    CHECK(forced.attend(cache4, 64) == C2KV_ERR_NOMEM, "splits that were asked for");
+}
+
+// and the turned queries of a step of ragged chunks, which is composed before it is attended.
+void no_queries() {
+    Context step({kBf16, 32, 8, 128, 32}), never({kBf16, 32, 8, 128, 32}, 0, 0, C2KV_FUSE_NEVER);
+    c2kv_cache* cache = nullptr;
+    CHECK(step.step(10, 125, 64, &cache) == C2KV_OK, "step");
+    CHECK(!fake::launched("14attn_tc_kernelILb1"), "not fused when there is memory");
+    fake::launches.clear();
+    fake::alloc_fails = [](size_t bytes) { return bytes == (size_t)32 * 64 * 32 * 128 * 2; };
+    CHECK(step.step(10, 125, 64, &cache) == C2KV_OK, "step without turned queries: %s", c2kv_last_error(step.ctx));
+    CHECK(fake::launched("14attn_tc_kernelILb1ELb0"), "fused");
+    CHECK(never.step(10, 125, 64, &cache) == C2KV_ERR_NOMEM, "never fused");
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
@@ -154,6 +182,8 @@ int main(int argc, char** argv) {
     }
     if (name == "registers") registers(argv[2]);
     else if (name == "second_device") second_device();
+    else if (name == "no_partials") no_partials();
+    else if (name == "no_queries") no_queries();
     else CHECK(false, "unknown scenario '%s'", name.c_str());
     std::printf("ok\n");
 }
