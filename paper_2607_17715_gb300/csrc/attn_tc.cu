@@ -654,8 +654,8 @@ __device__ __noinline__ void redo_rows(const TcParams& P, uint32_t bad, int quad
 // thread (which touch a separate cache line per thread).
 // kMerge: the plain kernel, whose split partials may be merged in the kernel (split_merge).
 // kSif: the plain kernel over extraction C2 rows (TcParams::sif_k), its own instantiation.
-// kKpp: the plain kernel's decode instantiation, whose pairs with one query tile split their
-// key tiles between the two warpgroups (kpp: this pair does).
+// kKpp: a decode step, whose one query tile's key tiles the two warpgroups share (kpp_pair: false
+// for a split without key tiles).
 // kO: the first TMEM column of O_A.  kDbl (x = 0): S and P alternate between two column blocks and
 // their barriers (B_SF, B_PF and the next ones); P.V(j - 1) may then still run when S(j) is read,
 // so a rescale of O waits for it (B_OE, one phase per P.V).
@@ -827,10 +827,6 @@ __device__ __forceinline__ void softmax_tile(const TcParams& P, uint32_t tmem, u
             asm volatile("bar.sync 4, 256;" ::: "memory");
             if constexpr (kMerge)
                 if (P.n_split > 1 && P.tickets != nullptr) split_merge<D>(P, sBar, x, r, t0, l, b, hk);
-            if (arrive_oe) {
-                tc_fence_before();
-                mbar_arrive(bar(B_OE));
-            }
             return;
         }
         mbar_wait(bar(B_OD), od_par, P.err, abort);
@@ -1186,15 +1182,14 @@ __device__ __forceinline__ void mma_issuer(const TcParams& P, uint32_t tmem, uin
     if (kHasB) st.pb += (uint32_t)n_kv;
 }
 
-// The MMA issuer for a pair with one query tile (tile A) and n_kv >= 1 key tiles, the key tiles
+// The MMA issuer of a decode step: one query tile (tile A) and n_kv >= 1 key tiles, the key tiles
 // split between the two halves of TMEM: tiles 0, 2, 4, ... go to (S_A, O_A), tiles 1, 3, 5, ...
 // to (S_B, O_B), and the two softmax warpgroups each run an online softmax over their half, so
 // that one half's softmax overlaps the other's MMAs as two query tiles' do (warpgroup A merges
 // the halves at the end).  Issue order: S(0), S(1), then per key tile j: P(j).V(j), S(j + 2)
 // on the same half (in issue order after the P.V that reads the P it overwrites).
 __device__ __forceinline__ void mma_issuer_kpp(const TcParams& P, uint32_t tmem, uint32_t sQ, uint32_t sK,
-                                               uint32_t sV, uint32_t sBar, int n_kv, int q_ready,
-                                               uint32_t q_par, RingState& st, bool wait_oe, uint32_t oe_par,
+                                               uint32_t sV, uint32_t sBar, int n_kv,
                                                volatile uint32_t* abort) {
     auto bar = [&](int i) { return sBar + 8u * (uint32_t)i; };
     constexpr uint32_t idS = idesc_bf16(BM, BN, false);
@@ -1209,8 +1204,8 @@ __device__ __forceinline__ void mma_issuer_kpp(const TcParams& P, uint32_t tmem,
         mbar_wait(bar(i), parity, P.err, abort);
         tc_fence_after();
     };
-    int ks = st.ks, vs = st.vs;
-    uint32_t kph = st.kph, vph = st.vph;
+    int ks = 0, vs = 0;
+    uint32_t kph = 0u, vph = 0u;
     auto s_next = [&](int x) {        // S of the next key tile into half x, its K stage released after
         wait(B_KF + ks, kph);
         const uint64_t dk = dK0 + (uint64_t)ks * kTileDesc;
@@ -1224,18 +1219,14 @@ __device__ __forceinline__ void mma_issuer_kpp(const TcParams& P, uint32_t tmem,
         kph ^= ks == KSTAGES - 1 ? 1u : 0u;
         ks = ks == KSTAGES - 1 ? 0 : ks + 1;
     };
-    wait(q_ready, q_par);
+    wait(B_QR, 0u);
     s_next(0);
     if (n_kv > 1) s_next(1);
-    uint32_t pa = st.pa, pb = st.pb;   // P phases of each half completed before this pair
 #pragma unroll 1
     for (int j = 0; j < n_kv; ++j) {
         const int x = j & 1;
-        wait(B_PF + x, (x ? pb : pa) & 1u);
-        pa += x ? 0u : 1u;
-        pb += x ? 1u : 0u;
+        wait(B_PF + x, (uint32_t)(j >> 1) & 1u);
         wait(B_VF + vs, vph);
-        if (wait_oe && j == 0) wait(B_OE, oe_par);
         const uint64_t dv = dV0 + (uint64_t)vs * kTileDesc;
 #pragma unroll
         for (int kk = 0; kk < BN / 16; ++kk)
@@ -1246,14 +1237,7 @@ __device__ __forceinline__ void mma_issuer_kpp(const TcParams& P, uint32_t tmem,
         vs = vs == VSTAGES - 1 ? 0 : vs + 1;
         if (j + 2 < n_kv) s_next(x);
     }
-    mma_commit(bar(B_QF));
     mma_commit(bar(B_OD));
-    st.ks = ks;
-    st.kph = kph;
-    st.vs = vs;
-    st.vph = vph;
-    st.pa = pa;
-    st.pb = pb;
 }
 
 // ------------------------------------------------------------------ fused loaders
@@ -2394,14 +2378,14 @@ __device__ __forceinline__ void attn_tc_body(const typename KernelParams<kFused,
                     else
                         mma_issuer<false>(P, tmem, sQ, sK, sV, sBar, ps.n_kv, B_QR, q_par, st, pi > 0, oe_par, abort);
                 }
+            } else if constexpr (kKpp) {         // a decode step
+                mma_issuer_kpp(P, tmem, sQ, sK, sV, sBar, n_kv, abort);
             } else {
                 for (int pi = 0; pi < p_count; ++pi) {
                     const PairSpan ps = pi == 0 ? ps0 : pair_span(P, p_first + pi, sp, s_r);
                     const uint32_t q_par = (uint32_t)pi & 1u, oe_par = (uint32_t)(pi - 1) & 1u;
                     if (ps.has_b)
                         mma_issuer<true, D>(P, tmem, sQ, sK, sV, sBar, ps.n_kv, B_Q, q_par, st, pi > 0, oe_par, abort);
-                    else if (kKpp)                                        // key tiles ping-pong (one pair)
-                        mma_issuer_kpp(P, tmem, sQ, sK, sV, sBar, ps.n_kv, B_QR, q_par, st, pi > 0, oe_par, abort);
                     else
                         mma_issuer<false, D>(P, tmem, sQ, sK, sV, sBar, ps.n_kv, B_Q, q_par, st, pi > 0, oe_par, abort);
                 }
@@ -2456,21 +2440,21 @@ __device__ __forceinline__ void attn_tc_body(const typename KernelParams<kFused,
                 }
             }
         } else {
+            // (a decode step has one pair and one query tile, whose key tiles the two warpgroups share
+            // (mma_issuer_kpp) and merge at the end)
             uint32_t done = 0u;     // S_x tiles of the earlier pairs
             for (int pi = 0; pi < p_count; ++pi) {
                 const PairSpan ps = pi == 0 ? ps0 : pair_span(P, p_first + pi, sp, s_r);
-                // a decode step's one query tile: the two warpgroups take alternate key tiles
-                // (mma_issuer_kpp) and merge at the end
                 const bool kpp = kKpp && ps.n_kv >= 1;
                 if constexpr (kKpp)
                     if (kpp)
-                        decode_turn_queries<kTerms>(KP, (int)threadIdx.x - 128, (int64_t)P.req[bl].l_req + P.req[bl].t0, sQ,
-                                            reinterpret_cast<float2*>(smem + TILE + 4096), sBar, abort);
+                        decode_turn_queries<kTerms>(KP, (int)threadIdx.x - 128, (int64_t)P.req[bl].l_req + P.req[bl].t0,
+                                                    sQ, reinterpret_cast<float2*>(smem + TILE + 4096), sBar, abort);
                 if (x == 0 || ps.has_b || kpp) {
-                    softmax_tile<true, kSif, kKpp, D, kColO, false, kTerms>(P, tmem, sBar, x, warp & 3, lane, x && !kpp ? ps.t0b : ps.t0a, l, bl,
-                                 b, hk, sp, ps, done, (uint32_t)pi & 1u, p_count > 1, abort,
-                                 pi == p_count - 1 ? sQ : 0u, kpp);
-                    done += kpp ? (uint32_t)((ps.n_kv + 1 - x) / 2) : (uint32_t)ps.n_kv;
+                    softmax_tile<true, kSif, kKpp, D, kColO, false, kTerms>(
+                        P, tmem, sBar, x, warp & 3, lane, x && !kpp ? ps.t0b : ps.t0a, l, bl, b, hk, sp, ps, done,
+                        (uint32_t)pi & 1u, p_count > 1, abort, pi == p_count - 1 ? sQ : 0u, kpp);
+                    done += (uint32_t)ps.n_kv;
                 } else if (p_count > 1) {    // no tile B in this pair: nothing of O to read
                     mbar_arrive(bar(B_OE));
                 } else if (P.tickets != nullptr) {   // a split without tile B: the merge's two
@@ -2517,9 +2501,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc64_sif_kernel(const __grid
     attn_tc_body<false, false, true, false, 64>(KP);
 }
 
-// Decode steps (AttnParams::key_pingpong): the plain kernel whose last pair, when it has one
-// query tile, splits its key tiles between the two softmax warpgroups.
-// kExact: fp32 weights, as three bf16 terms.
+// Decode steps (AttnParams::key_pingpong): one query token, whose key tiles the two softmax
+// warpgroups share.  kExact: fp32 weights, as three bf16 terms.
 template <bool kExact>
 __global__ void __launch_bounds__(kThreads, 1) attn_tc_decode_kernel(const __grid_constant__ DecodeTcParams KP) {
     attn_tc_body<false, false, false, true, HD, kExact ? 3 : 1>(KP);
