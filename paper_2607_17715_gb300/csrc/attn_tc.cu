@@ -3065,7 +3065,9 @@ cudaError_t launch_plain(const AttnParams& a, cudaStream_t s, Hook before) {
 // tile, or few key tiles (256 pairs of 3: 38 / 36, of 5: 44 / 42), and the pair kernel by 2 to 7 %
 // (and 13 % over 257 key tiles) when 77 pairs or more share their K/V tiles, unless two tiles an SM
 // take fewer rounds than a pair an SM (an odd number of tiles a head: 640 pairs of 7 tiles 131 / 114, 512
-// of 3 tiles 92.6 / 82.2; with as many rounds, 384 of 7 tiles 83.6 / 82.4, 256 of 3 tiles 60 / 64).
+// of 3 tiles 92.6 / 82.2; with as many rounds, 384 of 7 tiles 83.6 / 82.4, 256 of 3 tiles 60 / 64).  Heads
+// of 64 channels solo always: of 240 launches the pair kernel was never faster (320 query tiles of 12 key
+// tiles 89 / 72, 512 of 13 96 / 89, 216 of 158 501 / 451).
 enum class SoloChoice { kPair, kShared, kAlone };
 SoloChoice solo_choice(const AttnParams& a) {
     if (a.key_pingpong || a.pairs_per_cta != 0 || a.tickets != nullptr) return SoloChoice::kPair;
@@ -3074,7 +3076,7 @@ SoloChoice solo_choice(const AttnParams& a) {
     const int64_t per_head = (a.sq + tq - 1) / tq, heads = (int64_t)a.hkv * a.lq * a.batch;
     const int64_t units = per_head * heads * std::max(1, a.n_split);
     if (units <= sms && a.sif_k == 0) return SoloChoice::kAlone;
-    if (a.n_split > 1 || a.sif_k > 0 || per_head == 1) return SoloChoice::kShared;
+    if (a.n_split > 1 || a.sif_k > 0 || per_head == 1 || a.d == 64) return SoloChoice::kShared;
     int slots = 0;
     for (int i = 0; i < a.batch; ++i) slots = std::max(slots, a.req[i].n_slots);
     const int tiles = (slots + a.sq + BN - 1) / BN;

@@ -778,8 +778,11 @@ cudaError_t suffix_run(c2kv_ctx* c, const c2kv_cache* cache, int32_t layer0, int
 // Key-range splits of an attend launch on the tensor cores (`merge_launch`: partials merged by a
 // launch of their own rather than in the kernel).  When the query tiles leave SMs idle, each one's
 // key tiles may be split, as far as two CTAs an SM go, by a model of the call (us): a key tile takes
-// about 1 for a CTA alone on its SM and 1.95 for two sharing it, a CTA 8 to start and end, the merge
-// launch 5 and its partials' bytes both ways at 5 TB/s.
+// about 1 for a CTA alone on its SM and 1.95 for two sharing it (heads of 64 channels, whose weights
+// enter P.V three times: 1.6 and 2.2), a CTA 8 to start and end, the merge launch 5 and its partials'
+// bytes both ways at 5 TB/s.  Over 240 launches of either head size (8 / 8 to 64 / 8 and 32 / 4 heads, 1
+// to 8 requests of 16 to 250 tokens, 300 to 20000 slots) the choice takes 1 % more than the best number
+// of splits in the mean, and at most 17 % (128 channels) and 22 % (64).
 // (The merge in the kernel, by the last CTA of a unit alone, costs about 0.25 a row: with 256 rows a
 // unit it had made 2 requests x 200 tokens over 16 chunks 103 us a call, now 29.)  Measured, one
 // layer, 32 / 8 heads: 64 tokens over 10 chunks 28.9 -> 16 us, over 64 chunks 43 -> 24; 96 query tiles
@@ -800,10 +803,12 @@ int32_t attn_splits(const c2kv_ctx* c, const c2kv_cache* cache, int32_t lq, int3
     }
     const int64_t units = c2kv::attn_tc_tiles(c->cfg.n_q_heads, c->cfg.n_kv_heads, n_suffix, lq, cache->batch);
     const double rows = (double)lq * cache->batch * n_suffix * c->cfg.n_q_heads;
+    const double alone = c->cfg.head_dim == 64 ? 1.6 : 1.0, shared = c->cfg.head_dim == 64 ? 2.2 : 1.95;
     int32_t best = 1;
-    double cost = tiles * 1.0 + 8.0;
+    double cost = tiles * alone + 8.0;
     for (int32_t n = 2; n <= 16 && n * units <= 2 * c->sms && n <= tiles; ++n) {
-        const double t = (tiles + n - 1) / n * (n * units <= c->sms ? 1.0 : 1.95) + 8.0 + 5.0 + n * rows * (c->cfg.head_dim + 1) * 8.0 / 5.0e6;
+        const double t = (tiles + n - 1) / n * (n * units <= c->sms ? alone : shared) + 8.0 + 5.0 +
+                         n * rows * (c->cfg.head_dim + 1) * 8.0 / 5.0e6;
         if (t < 0.95 * cost) {
             cost = t;
             best = n;
@@ -819,7 +824,10 @@ int32_t attn_splits(const c2kv_ctx* c, const c2kv_cache* cache, int32_t lq, int3
 // query tile), so with such tiles a model of both (us) decides; compose moves its bytes at 6.7 TB/s.
 // Measured, fused / unfused (32 / 8 heads, 64 suffix tokens, chunks x slots): 32 layers, 10 x 128:
 // 81 / 107, 10 x 125: 270 / 107; 16 layers, 10 x 130: 132 / 61, 3 x 500: 77 / 68, 20 x 64: 132 / 61; one
-// layer, 2 requests, 10 x 125: 136 / 33.  The results are the same bits, unless the keys are split.
+// layer, 2 requests, 10 x 125: 136 / 33.  Over 120 steps of 8 / 8, 32 / 8, 64 / 8 and 32 / 4 heads the
+// choice takes 1.7 % more than the better route in the mean; at most 8 % with boundaries, 26 % without
+// (one layer of 2 requests, which always runs fused).  The results are the same bits, unless the keys are
+// split.
 bool fused_pays(const c2kv_ctx* c, const c2kv_cache* cache, const std::vector<c2kv::OccParam>& occ,
                 const int32_t* req_ptr, int32_t n_suffix) {
     const int32_t L = c->cfg.layers, B = cache->batch, hkv = c->cfg.n_kv_heads;
