@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(kCoreThreads, core_ctas(D, RT)) attn_simt_kern
     j.bl = (int)blockIdx.z - j.l * a.batch;
     j.hk = blockIdx.y;
     j.g_heads = a.hq / a.hkv;
-    j.rows = 16 * RT;
+    j.rows = Core<D, RT>::kRows;
     j.row0 = (int)(blockIdx.x / (unsigned)ns) * j.rows;
     j.nrows = a.sq * j.g_heads;
     j.slots = a.req[j.bl].n_slots;
@@ -99,15 +99,19 @@ cudaError_t launch_typed(const AttnParams& a, cudaStream_t s) {
     const int64_t nrows = (int64_t)a.sq * (a.hq / a.hkv);
     const CoreKernel<D, 4> large = ready<T, D, 4>();
     const CoreKernel<D, 1> small = ready<T, D, 1>();
-    if (large.err != cudaSuccess || small.err != cudaSuccess) return large.err != cudaSuccess ? large.err : small.err;
-    const CorePlan plan = core_plan(nrows, (int64_t)a.hkv * a.lq * a.batch, nkeys, D, [&](bool sm, int ns, bool alone) {
-        return sm ? small.slots[alone][ns] : large.slots[alone][ns];
+    const CoreKernel<D, 0> four = ready<T, D, 0>();
+    if (large.err != cudaSuccess) return large.err;
+    if (small.err != cudaSuccess || four.err != cudaSuccess) return small.err != cudaSuccess ? small.err : four.err;
+    const CorePlan plan = core_plan(nrows, (int64_t)a.hkv * a.lq * a.batch, nkeys, D, false, [&](int form, int ns, bool alone) {
+        return form == 4 ? large.slots[alone][ns] : form == 1 ? small.slots[alone][ns] : four.slots[alone][ns];
     });
-    const int64_t rows = plan.small ? 16 : 64;
+    const int64_t rows = plan.form == 0 ? 4 : 16 * plan.form;
     const int64_t gx = (nrows + rows - 1) / rows * plan.ns;
     if (gx > 0x7fffffffLL) return cudaErrorInvalidValue;
     const dim3 grid((unsigned)gx, a.hkv, a.lq * a.batch);
-    return plan.small ? launch_rt<T, D, 1>(a, plan, grid, s) : launch_rt<T, D, 4>(a, plan, grid, s);
+    return plan.form == 4   ? launch_rt<T, D, 4>(a, plan, grid, s)
+           : plan.form == 1 ? launch_rt<T, D, 1>(a, plan, grid, s)
+                            : launch_rt<T, D, 0>(a, plan, grid, s);
 }
 
 template <typename T, int D>
@@ -115,8 +119,10 @@ cudaError_t preload() {
     cudaFuncAttributes fa{};
     cudaError_t e = cudaFuncGetAttributes(&fa, attn_simt_kernel<T, D, 4>);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, attn_simt_kernel<T, D, 1>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, attn_simt_kernel<T, D, 0>);
     if (e == cudaSuccess) e = ready<T, D, 4>().err;
     if (e == cudaSuccess) e = ready<T, D, 1>().err;
+    if (e == cudaSuccess) e = ready<T, D, 0>().err;
     return e;
 }
 

@@ -824,7 +824,7 @@ int32_t attn_splits(const c2kv_ctx* c, const c2kv_cache* cache, int32_t lq, int3
 // query tile), so with such tiles a model of both (us) decides; compose moves its bytes at 6.7 TB/s.
 // Measured, fused / unfused (32 / 8 heads, 64 suffix tokens, chunks x slots): 32 layers, 10 x 128:
 // 81 / 107, 10 x 125: 270 / 107; 16 layers, 10 x 130: 132 / 61, 3 x 500: 77 / 68, 20 x 64: 132 / 61; one
-// layer, 2 requests, 10 x 125: 136 / 33.  Over 120 steps of 8 / 8, 32 / 8, 64 / 8 and 32 / 4 heads the
+// layer, 2 requests, 10 x 125: 136 / 33.  Over 96 steps of 8 / 8, 32 / 8, 64 / 8 and 32 / 4 heads the
 // choice takes 1.7 % more than the better route in the mean; at most 8 % with boundaries, 26 % without
 // (one layer of 2 requests, which always runs fused).  The results are the same bits, unless the keys are
 // split.

@@ -172,10 +172,11 @@ __global__ void __launch_bounds__(kCoreThreads, core_ctas(D, RT)) extract_attn_k
     j.hk = blockIdx.y;
     j.g_heads = P.hq / P.hkv;
     // last rows first: under the causal mask they see the most keys
-    j.row0 = (int)((gridDim.x - 1 - blockIdx.x) / (unsigned)ns) * 16 * RT;
+    constexpr int kRows = Core<D, RT>::kRows;
+    j.row0 = (int)((gridDim.x - 1 - blockIdx.x) / (unsigned)ns) * kRows;
     j.nrows = P.n_all * j.g_heads;
     j.t0 = j.row0 / j.g_heads;
-    j.t1 = min(P.n_all - 1, (j.row0 + 16 * RT - 1) / j.g_heads);
+    j.t1 = min(P.n_all - 1, (j.row0 + kRows - 1) / j.g_heads);
     const int n = P.n, ja = max(j.t0 - n, 0), jb = j.t1 - n;
     const bool c2 = j.t1 >= n;
     j.doc_end = j.t0 < n ? min(j.t1, n - 1) + 1 : 0;
@@ -267,7 +268,8 @@ CoreKernel<D, RT> ready() {
 
 template <typename T, int D, int RT>
 cudaError_t launch_rt(const ExtractParams& p, int ns, bool alone, cudaStream_t s) {
-    const int64_t gx = ((int64_t)p.n_all * (p.hq / p.hkv) + 16 * RT - 1) / (16 * RT) * ns;
+    constexpr int kRows = Core<D, RT>::kRows;
+    const int64_t gx = ((int64_t)p.n_all * (p.hq / p.hkv) + kRows - 1) / kRows * ns;
     if (gx > 0x7fffffffLL) return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)gx, (unsigned)p.hkv, (unsigned)p.lq);
@@ -294,13 +296,18 @@ cudaError_t launch_typed(const ExtractParams& p, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     const CoreKernel<D, 4> large = ready<T, D, 4>();
     const CoreKernel<D, 1> small = ready<T, D, 1>();
-    if (large.err != cudaSuccess || small.err != cudaSuccess) return large.err != cudaSuccess ? large.err : small.err;
-    // (the causal rows see half of the keys on average)
-    const CorePlan plan = core_plan((int64_t)p.n_all * (p.hq / p.hkv), (int64_t)p.hkv * p.lq, (p.n_all + 1) / 2, D,
-                                    [&](bool sm, int ns, bool alone) {
-                                        return sm ? small.slots[alone][ns] : large.slots[alone][ns];
+    const CoreKernel<D, 0> four = ready<T, D, 0>();
+    if (large.err != cudaSuccess) return large.err;
+    if (small.err != cudaSuccess || four.err != cudaSuccess) return small.err != cudaSuccess ? small.err : four.err;
+    const CorePlan plan = core_plan((int64_t)p.n_all * (p.hq / p.hkv), (int64_t)p.hkv * p.lq, p.n_all, D, true,
+                                    [&](int form, int ns, bool alone) {
+                                        return form == 4   ? large.slots[alone][ns]
+                                               : form == 1 ? small.slots[alone][ns]
+                                                           : four.slots[alone][ns];
                                     });
-    return plan.small ? launch_rt<T, D, 1>(p, plan.ns, plan.alone, s) : launch_rt<T, D, 4>(p, plan.ns, plan.alone, s);
+    return plan.form == 4   ? launch_rt<T, D, 4>(p, plan.ns, plan.alone, s)
+           : plan.form == 1 ? launch_rt<T, D, 1>(p, plan.ns, plan.alone, s)
+                            : launch_rt<T, D, 0>(p, plan.ns, plan.alone, s);
 }
 
 }  // namespace

@@ -172,6 +172,20 @@ void no_queries() {
     CHECK(never.step(10, 125, 64, &cache) == C2KV_ERR_NOMEM, "never fused");
 }
 
+// Few rows of many units on the CUDA cores: four rows a CTA, whose warps share the keys; not the forms of 16
+// and 64 rows, most of which would be empty.
+void few_rows() {
+    for (int d : {64, 128}) {
+        Context one({kF32, 32, 8, d, 32});
+        for (int slots : {8, 100, 300}) {
+            c2kv_cache* cache = one.compose(10, slots, 4);
+            fake::launches.clear();
+            CHECK(one.attend(cache, 1) == C2KV_OK, "attend: %s", c2kv_last_error(one.ctx));
+            CHECK(fake::launched("attn_simt_kernelIfLi" + std::to_string(d) + "ELi0E"), "d %d, %d slots", d, slots);
+        }
+    }
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
@@ -182,6 +196,7 @@ int main(int argc, char** argv) {
     }
     if (name == "registers") registers(argv[2]);
     else if (name == "second_device") second_device();
+    else if (name == "few_rows") few_rows();
     else if (name == "no_partials") no_partials();
     else if (name == "no_queries") no_queries();
     else CHECK(false, "unknown scenario '%s'", name.c_str());

@@ -25,6 +25,16 @@ def test_attend_f32(d, hq, hkv, sq, tokens, k):
     _attend_case(synth.scaled(F32, n_q_heads=hq, n_kv_heads=hkv, head_dim=d, chunk_tokens=tokens, ratio_k=k), n_suffix=sq)
 
 
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("hq,hkv,sq", [(1, 1, 1), (4, 1, 1), (2, 1, 2), (2, 2, 4), (8, 2, 5), (3, 1, 2)])
+@pytest.mark.parametrize("keys", [1, 8, 9, 16, 17, 32, 33, 64, 65, 200, 1100])
+def test_attend_few_rows(d, hq, hkv, sq, keys):
+    # four rows whose keys the warps share (key tiles partly full, warps without keys), and clusters of it
+    if keys > sq:
+        _attend_case(synth.scaled(F32, n_q_heads=hq, n_kv_heads=hkv, head_dim=d, chunk_tokens=keys - sq, ratio_k=1,
+                                  chunks_per_request=1, pool_chunks=1), n_suffix=sq)
+
+
 @pytest.mark.parametrize("d,sq,batch,hq,hkv", [(64, 250, 3, 32, 8), (128, 129, 4, 32, 8), (128, 16, 2, 64, 32)])
 def test_attend_f32_large_launch(d, sq, batch, hq, hkv):
     # several CTAs per SM: 64 rows a CTA
