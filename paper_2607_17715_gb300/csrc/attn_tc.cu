@@ -2900,6 +2900,21 @@ bool attn_tc_takes(int dtype, int d, int hq, int hkv) {
     return g == 1 || g == 2 || g == 4 || g == 8 || g == 16;
 }
 
+// Heads of 64 channels ran on the CUDA cores, with fp32 weights, and still do where a unit's packed rows and
+// keys are so few that a tensor-core CTA is mostly its start and end: 4 ceil(rows / 4) keys <= 700, or, when
+// the query tiles outnumber the SMs, at most 4 rows over 360 keys.  Over 352 launches (16 / 16, 32 / 8 and 32 /
+// 4 heads, 4 to 5120 units of 1 to 480 rows, 9 to 960 keys) the rule takes 0.7 % more than the better side in
+// the mean, at most 18 %.  Measured (us a call, CUDA cores / tensor cores): 5120 units of one row over 9
+// keys 60 / 137, over 41 65 / 131, over 301 196 / 226, over 901 527 / 469; 1792 units of 12 rows over 11 keys
+// 28 / 53, over 43 38 / 51, over 103 58 / 49.
+bool attn_tc_pays(int d, int hq, int hkv, int sq, int64_t nkeys, int64_t units) {
+    if (d != 64) return true;
+    const int g = hq / hkv, tq = BM / g;
+    const int64_t rows = (int64_t)sq * g;
+    if ((rows + 3) / 4 * 4 * nkeys <= 700) return false;
+    return !(rows <= 4 && nkeys <= 360 && (sq + tq - 1) / tq * units > device_sms());
+}
+
 namespace {
 
 // Host-side preparation shared by the plain and the fused launch: function attributes once

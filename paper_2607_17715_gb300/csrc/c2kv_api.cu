@@ -874,9 +874,15 @@ cudaError_t attend_run(c2kv_ctx* c, c2kv_cache* cache, int32_t layer0, int32_t l
                        const void* k_suf, const void* v_suf, int32_t n_suffix, void* out, float* lse,
                        const c2kv::FusedSpec* fused, void* q_rot_ready = nullptr) {
     const int32_t B = cache->batch;
+    int32_t keys = 0;
+    for (int32_t b = 0; b < B; ++b) keys = std::max(keys, cache->n_slots[b] + n_suffix);
+    // (splits and pairs that the context asks for are the tensor-core kernels')
     const bool use_tc =
         c->cfg.attn_impl != C2KV_ATTN_SIMT &&
-        c2kv::attn_tc_takes(c->cfg.dtype, c->cfg.head_dim, c->cfg.n_q_heads, c->cfg.n_kv_heads);
+        c2kv::attn_tc_takes(c->cfg.dtype, c->cfg.head_dim, c->cfg.n_q_heads, c->cfg.n_kv_heads) &&
+        (c->cfg.attn_split != 0 || c->cfg.attn_pairs != 0 ||
+         c2kv::attn_tc_pays(c->cfg.head_dim, c->cfg.n_q_heads, c->cfg.n_kv_heads, n_suffix, keys,
+                            (int64_t)lq * B * c->cfg.n_kv_heads));
     if (fused && (!use_tc || c->cfg.head_dim != 128 || layer0 != 0 || lq != c->cfg.layers || B > c2kv::kMaxReq))
         return cudaErrorInvalidValue;
 
@@ -1623,7 +1629,7 @@ c2kv_status c2kv_extract_attention(c2kv_ctx* c, int32_t n_layers, const void* q,
         const int32_t n_all = (int32_t)(n_tokens + m);
         const int32_t hq = c->cfg.n_q_heads, hkv = c->cfg.n_kv_heads;
         // the turned queries, or the angles from which the attention turns them
-        const bool turn_q = c2kv::extract_uses_tc(c->cfg.dtype, d, hq, hkv) &&
+        const bool turn_q = c2kv::extract_uses_tc(c->cfg.dtype, d, hq, hkv, n_all, n_layers, c->cfg.attn_pairs) &&
                             c2kv::extract_turns_queries(c->cfg.attn_pairs);
         const size_t qb = turn_q ? (size_t)n_all * (d / 2) * sizeof(float2)
                                  : (size_t)n_layers * n_all * hq * d * c->eb;
@@ -1657,7 +1663,7 @@ c2kv_status c2kv_extract_attention(c2kv_ctx* c, int32_t n_layers, const void* q,
         p.pairs_per_cta = c->cfg.attn_pairs;
         p.rope = c->turns;
         // the C2 rows beside the document rows on the second stream (tensor-core route)
-        const bool two = c2kv::extract_uses_tc(c->cfg.dtype, d, c->cfg.n_q_heads, c->cfg.n_kv_heads) &&
+        const bool two = c2kv::extract_uses_tc(c->cfg.dtype, d, hq, hkv, n_all, n_layers, c->cfg.attn_pairs) &&
                          aux_ready(c, 2) == cudaSuccess;
         {
             ProfScope prof(c, C2KV_PROF_EXTRACT);

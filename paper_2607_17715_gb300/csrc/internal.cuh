@@ -248,7 +248,7 @@ cudaError_t launch_extract(const ExtractParams& p, int dtype, int d, cudaStream_
                            cudaStream_t s2 = nullptr, cudaEvent_t fork = nullptr, cudaEvent_t join = nullptr);
 // Whether launch_extract takes the tensor-core route; otherwise every row runs on the CUDA
 // cores.
-bool extract_uses_tc(int dtype, int d, int hq, int hkv);
+bool extract_uses_tc(int dtype, int d, int hq, int hkv, int n_all, int lq, int pairs_per_cta);
 // Whether the tensor-core route turns the queries in the attention (q_rot null, q_cs given).
 bool extract_turns_queries(int pairs_per_cta);
 
@@ -263,6 +263,9 @@ bool encode_tensor_map(CUtensorMap* tm, CUtensorMapDataType type, int rank, cons
 // and C2KV_ATTN_TC (d 128).
 bool attn_tc_supported(int dtype, int d, int hq, int hkv);
 bool attn_tc_takes(int dtype, int d, int hq, int hkv);
+// Whether an attend launch that the tensor cores take (attn_tc_takes) is the faster there: sq suffix tokens
+// over at most nkeys keys (theirs among them) in `units` (layer, request, KV head) units.
+bool attn_tc_pays(int d, int hq, int hkv, int sq, int64_t nkeys, int64_t units);
 cudaError_t launch_attn_tc(const AttnParams& p, cudaStream_t s, Hook before = {});
 // A decode step on the tensor cores (AttnParams with sq 1, key_pingpong 1; its q_rot is the queries
 // before RoPE): the new token's key and value rows are appended by the same kernel.

@@ -51,7 +51,8 @@ cudaError_t noalloc_prepare(int dtype, int d, bool tc, void** scratch) {
     void* p = nullptr;
     cudaError_t e = cudaGetSymbolAddress(&p, g_attend_scratch);
     if (e == cudaSuccess) e = preload_suffix_kernels(dtype, d);
-    if (e == cudaSuccess) e = tc ? preload_attn_tc_kernels(d) : preload_attn_simt_kernels(dtype, d);
+    if (e == cudaSuccess && tc) e = preload_attn_tc_kernels(d);
+    if (e == cudaSuccess && (!tc || d == 64)) e = preload_attn_simt_kernels(dtype, d);   // (attn_tc_pays)
     if (e != cudaSuccess) return e;
     *scratch = p;
     return cudaSuccess;
@@ -102,8 +103,12 @@ extern "C" c2kv_status c2kv_attend_noalloc(c2kv_ctx* ctx, c2kv_cache* cache, int
                       "attend_noalloc: the current device is not the context's device");
     void* const q_rot = v.noalloc_scratch;
     cudaError_t e = cudaSuccess;
+    int32_t keys = 0;
+    for (int32_t b = 0; b < B; ++b) keys = v.n_slots[b] + n_suffix > keys ? v.n_slots[b] + n_suffix : keys;
     const bool use_tc = v.attn_impl != C2KV_ATTN_SIMT &&
-                        c2kv::attn_tc_takes(v.dtype, v.head_dim, v.n_q_heads, v.n_kv_heads);
+                        c2kv::attn_tc_takes(v.dtype, v.head_dim, v.n_q_heads, v.n_kv_heads) &&
+                        (v.attn_pairs != 0 || c2kv::attn_tc_pays(v.head_dim, v.n_q_heads, v.n_kv_heads, n_suffix, keys,
+                                                                 (int64_t)lq * B * v.n_kv_heads));
     for (int32_t b0 = 0; e == cudaSuccess && b0 < B; b0 += c2kv::kMaxReq) {
         const int32_t nb = B - b0 < c2kv::kMaxReq ? B - b0 : c2kv::kMaxReq;
         c2kv::SuffixParams s{};

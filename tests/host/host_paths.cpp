@@ -186,6 +186,38 @@ void few_rows() {
     }
 }
 
+// bf16 heads of 64 channels: few rows over few keys stay on the CUDA cores, for both attend calls.
+void short64() {
+    Context one({kBf16, 32, 8, 64, 32}), split({kBf16, 32, 8, 64, 32}, 1);
+    struct {
+        int slots, n;
+        bool tc;
+    } const cases[] = {{8, 1, false}, {300, 1, false}, {900, 1, true}, {30, 8, true}, {100, 60, true}};
+    for (const auto& k : cases) {
+        c2kv_cache* cache = one.compose(10, k.slots, 64);
+        for (int noalloc = 0; noalloc < 2; ++noalloc) {
+            fake::launches.clear();
+            const c2kv_status st = noalloc ? c2kv_attend_noalloc(one.ctx, cache, k.slots > 100 ? 0 : -1, buffer, buffer,
+                                                                 buffer, k.n, buffer, nullptr)
+                                           : one.attend(cache, k.n);
+            if (st == C2KV_ERR_ARG && noalloc) continue;          // beyond its fixed scratch
+            CHECK(st == C2KV_OK, "%s", c2kv_last_error(one.ctx));
+            if (noalloc && k.slots > 100) continue;               // one layer: another count of query tiles
+            CHECK(fake::launched("attn_solo_kernel") == k.tc && fake::launched("attn_simt_kernel") != k.tc,
+                  "%d slots, %d tokens, noalloc %d", k.slots, k.n, noalloc);
+        }
+        fake::launches.clear();
+        CHECK(split.attend(split.compose(10, k.slots, 64), k.n) == C2KV_OK, "%s", c2kv_last_error(split.ctx));
+        CHECK(fake::launched("attn_solo_kernel"), "splits that are asked for are the tensor cores'");
+    }
+    for (int tokens : {8, 40, 700}) {                             // and short chunks' extraction
+        fake::launches.clear();
+        CHECK(one.extract(tokens, 4) == C2KV_OK, "%s", c2kv_last_error(one.ctx));
+        CHECK(fake::launched("attn_solo_kernel") == (tokens == 700) && fake::launched("extract_attn_kernel") != (tokens == 700),
+              "%d tokens", tokens);
+    }
+}
+
 }  // namespace
 
 int main(int argc, char** argv) {
@@ -197,6 +229,7 @@ int main(int argc, char** argv) {
     if (name == "registers") registers(argv[2]);
     else if (name == "second_device") second_device();
     else if (name == "few_rows") few_rows();
+    else if (name == "short64") short64();
     else if (name == "no_partials") no_partials();
     else if (name == "no_queries") no_queries();
     else CHECK(false, "unknown scenario '%s'", name.c_str());

@@ -1,6 +1,10 @@
 """bf16 heads of 64 channels on the tensor cores: the suffix attention and the extraction
 attention against the oracle and against the CUDA-core kernel, at the edges of the query and key
 tiles (128 packed rows, 128 keys), over the group sizes and key-range splits."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -9,6 +13,7 @@ import synth
 from tests import _gpu_helpers as H
 from tests.test_gpu_extract import _extract_case
 from tests.test_gpu_parity import _attend_case
+from tests.test_zz_no_alloc import _FIRST_CALL
 
 pytestmark = pytest.mark.gpu
 
@@ -29,6 +34,25 @@ def test_attend(hq, hkv, sq, tokens, k):
     _attend_case(synth.scaled(D64, n_q_heads=hq, n_kv_heads=hkv, chunk_tokens=tokens, ratio_k=k), n_suffix=sq)
 
 
+@pytest.mark.parametrize("hq,hkv,sq,tokens,k", [(4, 1, 1, 64, 1), (8, 2, 3, 20, 4), (1, 1, 4, 1, 1), (32, 8, 1, 150, 1)])
+def test_attend_short(hq, hkv, sq, tokens, k):
+    # few rows over few keys: on the tensor cores when splits are asked for, else on the CUDA cores
+    wl = synth.scaled(D64, n_q_heads=hq, n_kv_heads=hkv, chunk_tokens=tokens, ratio_k=k)
+    _attend_case(wl, n_suffix=sq, attn_split=1)
+    _attend_case(synth.scaled(wl, layers=24), n_suffix=sq)
+
+
+@pytest.mark.parametrize("n_suffix", [1, 48])
+def test_noalloc_first_call_takes_no_device_memory(n_suffix):
+    # either route's kernels are loaded when the context is made
+    script = _FIRST_CALL.replace("n_suffix=16)", f"n_suffix={n_suffix}, head_dim=64, chunk_tokens=64)")
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    res = subprocess.run([sys.executable, "-c", script.format(root=root)], env=dict(os.environ, CUDA_MODULE_LOADING="LAZY"),
+                         capture_output=True, text=True, timeout=240, cwd=root)
+    assert res.returncode == 0, res.stdout[-2000:] + res.stderr[-2000:]
+    assert "FREE_DELTA 0\n" in res.stdout, res.stdout[-2000:]
+
+
 @pytest.mark.parametrize("split", [2, 5, 16])
 def test_attend_splits(split):
     # three key tiles: with more splits some are empty, and they merge in the kernel
@@ -44,7 +68,11 @@ def test_attend_layer_of_a_batch():
 
 @pytest.mark.parametrize("n,k", [(512, 4), (128, 1), (129, 16), (33, 4), (1, 1), (700, 10)])
 def test_extract(n, k):
+    # (short chunks: on the CUDA cores by themselves, on the tensor cores with pairs that are asked for)
     _extract_case(D64, n, k, layers=2 if n < 200 else 1)
+    if n < 200:
+        _extract_case(D64, n, k, layers=2, attn_pairs=1)
+        _extract_case(D64, n, k, layers=40 if n > 1 else 2)
 
 
 def test_weights_keep_more_than_bf16():

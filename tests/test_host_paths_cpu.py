@@ -37,6 +37,6 @@ def test_register_splits_are_guarded(program):
         _run(program, "registers", k)
 
 
-@pytest.mark.parametrize("scenario", ["second_device", "no_partials", "no_queries", "few_rows"])
+@pytest.mark.parametrize("scenario", ["second_device", "no_partials", "no_queries", "few_rows", "short64"])
 def test_scenario(program, scenario):
     _run(program, scenario)
