@@ -396,21 +396,25 @@ __global__ void __launch_bounds__(kBulkThreads, 1)
 // summed in row order; the angles of the CTA's slots, the same for every head and layer, are formed
 // once in shared memory.  With one row of K and V in flight and eight angles formed per item, a
 // 2000-token chunk of 32 layers took 62 us a call 8 to a slot, 103 us uncompressed; now 50 (5.9 TB/s)
-// and 83 (6.3 TB/s).
+// and 83 (6.3 TB/s).  kBoth (ROWS = 1, one layer: there are no other layers' rows): K and V of the item
+// by one thread instead, in CTAs of which an SM holds four: 4000 uncompressed tokens of one layer 12.3 us
+// in the other form, 10.3 before it, 8.2 so.
 // ---------------------------------------------------------------------------------------
-template <typename T, int VPH, int ROWS>
-__global__ void __launch_bounds__(256, 3) compress_kernel(const __grid_constant__ CompressParams P) {
+template <typename T, int VPH, int ROWS, bool kBoth = false>
+__global__ void __launch_bounds__(256, kBoth ? 4 : 3) compress_kernel(const __grid_constant__ CompressParams P) {
     using V = Vec16<T>;
     constexpr int E = V::N;
     constexpr int HALF = VPH * E;
     constexpr int D = 2 * HALF;
-    constexpr int LPT = 4 / ROWS;
+    static_assert(!kBoth || ROWS == 1, "one row of K and of V");
+    constexpr int LPT = kBoth ? 2 : 4 / ROWS;            // (layer, kBoth: tensor)
+    constexpr int STEP = kBoth ? 1 : LPT;                // layers
     __shared__ float2 cs[(256 + 2 * VPH) * E];           // [slots of the CTA][HALF]
     const int pairs = P.hkv * VPH;                       // items a slot (at least VPH)
     const int64_t per_layer = (int64_t)P.m * pairs;
     const int64_t first = (int64_t)blockIdx.x * blockDim.x;
     const int64_t r = first + threadIdx.x;
-    const bool turn = blockIdx.z == 0 && P.turn;
+    const bool turn = (kBoth || blockIdx.z == 0) && P.turn;
     auto slot_of = [&](int64_t i) { return per_layer <= 0x7fffffffLL ? (int)i / pairs : (int)(i / pairs); };
     const int j_first = slot_of(first);
     const bool live = r < per_layer;
@@ -421,17 +425,19 @@ __global__ void __launch_bounds__(256, 3) compress_kernel(const __grid_constant_
     const int64_t col = (int64_t)(p / VPH) * D + iv * E;
     const int r0 = P.one_row ? j : j * P.k;
     const int cnt = P.one_row ? 1 : min(r0 + P.k, P.n) - r0;
-    const T* const in = static_cast<const T*>(blockIdx.z ? P.in_v : P.in_k) + (int64_t)r0 * row_elems + col;
-    T* const out = static_cast<T*>(blockIdx.z ? P.pool_v : P.pool_k) + ((int64_t)P.slot_base + j) * row_elems + col;
+    const int64_t in_at = (int64_t)r0 * row_elems + col, out_at = ((int64_t)P.slot_base + j) * row_elems + col;
+    const T* const in = static_cast<const T*>(blockIdx.z ? P.in_v : P.in_k) + in_at;
+    T* const out = static_cast<T*>(blockIdx.z ? P.pool_v : P.pool_k) + out_at;
     const int64_t in_layer = (int64_t)P.rows_in * row_elems, out_layer = P.pool_slots * row_elems;
     bool angles = !turn;
-    for (int l0 = blockIdx.y * LPT; l0 < P.layers; l0 += gridDim.y * LPT) {
+    for (int l0 = blockIdx.y * STEP; l0 < P.layers; l0 += gridDim.y * STEP) {
         uint4 x[LPT][ROWS], y[LPT][ROWS];
         auto load = [&](int u, int c) {                  // rows c .. of layer l0 + u
 #pragma unroll
             for (int i = 0; i < ROWS; ++i)
-                if (live && l0 + u < P.layers && c + i < cnt) {
-                    const T* s = in + (int64_t)(l0 + u) * in_layer + (int64_t)(c + i) * row_elems;
+                if (live && (kBoth || l0 + u < P.layers) && c + i < cnt) {
+                    const T* s = kBoth ? static_cast<const T*>(u ? P.in_v : P.in_k) + in_at + (int64_t)l0 * in_layer
+                                       : in + (int64_t)(l0 + u) * in_layer + (int64_t)(c + i) * row_elems;
                     x[u][i] = ld16(s);
                     y[u][i] = ld16(s + HALF);
                 }
@@ -452,7 +458,7 @@ __global__ void __launch_bounds__(256, 3) compress_kernel(const __grid_constant_
         if (!live) continue;
 #pragma unroll
         for (int u = 0; u < LPT; ++u) {
-            if (l0 + u >= P.layers) break;
+            if (!kBoth && l0 + u >= P.layers) break;
             float sx[E], sy[E];
 #pragma unroll
             for (int e = 0; e < E; ++e) sx[e] = sy[e] = 0.f;
@@ -480,7 +486,7 @@ __global__ void __launch_bounds__(256, 3) compress_kernel(const __grid_constant_
                     sy[e] = sy[e] / c;
                 }
             }
-            if (turn) {
+            if (turn && !(kBoth && u == 1)) {
                 float gx[E], gy[E];
                 rotate<E>(sx, sy, cs + (j - j_first) * HALF + iv * E, gx, gy);
 #pragma unroll
@@ -489,7 +495,8 @@ __global__ void __launch_bounds__(256, 3) compress_kernel(const __grid_constant_
                     sy[e] = gy[e];
                 }
             }
-            T* dst = out + (int64_t)(l0 + u) * out_layer;
+            T* dst = kBoth ? static_cast<T*>(u ? P.pool_v : P.pool_k) + out_at + (int64_t)l0 * out_layer
+                           : out + (int64_t)(l0 + u) * out_layer;
             st16(dst, V::pack(sx));
             st16(dst + HALF, V::pack(sy));
         }
@@ -714,7 +721,8 @@ cudaError_t launch_compose(const ComposeParams& p, int dtype, int d, int layers,
 
 template <typename T, int VPH>
 cudaError_t launch_compress_rows(const CompressParams& p, int rows, dim3 grid, cudaStream_t s) {
-    if (rows == 1) compress_kernel<T, VPH, 1><<<grid, 256, 0, s>>>(p);
+    if (rows == 1 && p.layers == 1) compress_kernel<T, VPH, 1, true><<<dim3(grid.x, 1, 1), 256, 0, s>>>(p);
+    else if (rows == 1) compress_kernel<T, VPH, 1><<<grid, 256, 0, s>>>(p);
     else if (rows == 2) compress_kernel<T, VPH, 2><<<grid, 256, 0, s>>>(p);
     else compress_kernel<T, VPH, 4><<<grid, 256, 0, s>>>(p);
     return cudaGetLastError();

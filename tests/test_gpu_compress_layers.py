@@ -16,7 +16,7 @@ TINY = synth.workload("tiny_f32")
 
 @pytest.mark.parametrize("base,hkv,d", [(L8B, 8, 128), (L8B, 1, 64), (L8B, 3, 128), (TINY, 2, 64), (TINY, 1, 128)])
 @pytest.mark.parametrize("layers,n,k", [(1, 1, 1), (4, 37, 1), (5, 70, 1), (3, 71, 2), (2, 50, 3), (2, 301, 4), (3, 90, 7),
-                                        (1, 200, 16), (1, 5, 9)])
+                                        (1, 200, 16), (1, 5, 9), (1, 71, 1), (1, 300, 1)])
 def test_meanpool(base, hkv, d, layers, n, k):
     c2kv = H.lib()
     wl = synth.scaled(base, layers=layers, n_q_heads=4 * hkv, n_kv_heads=hkv, head_dim=d, chunk_tokens=n, ratio_k=k)
@@ -38,7 +38,7 @@ def test_meanpool(base, hkv, d, layers, n, k):
         c2kv.c2kv_destroy(ctx)
 
 
-@pytest.mark.parametrize("layers,m", [(1, 1), (6, 33)])
+@pytest.mark.parametrize("layers,m", [(1, 1), (6, 33), (1, 33)])
 def test_provided(layers, m):
     c2kv = H.lib()
     wl = synth.scaled(L8B, layers=layers, chunk_tokens=4 * m - 1, ratio_k=4)
