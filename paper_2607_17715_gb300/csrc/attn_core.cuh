@@ -565,5 +565,31 @@ struct CoreKernel {
     }
 };
 
+// A planned launch: `ns` CTAs a cluster along x; `dependent`: it starts while the kernel before it runs,
+// and waits for it.
+inline cudaError_t core_launch(const void* kernel, dim3 grid, size_t smem, const CorePlan& plan, bool dependent, void** args,
+                               cudaStream_t s) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(kCoreThreads);
+    cfg.dynamicSmemBytes = plan.alone ? kCoreAlone : smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    cfg.attrs = attr;
+    if (plan.ns > 1) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+        attr[cfg.numAttrs].val.clusterDim.x = (unsigned)plan.ns;
+        attr[cfg.numAttrs].val.clusterDim.y = 1;
+        attr[cfg.numAttrs].val.clusterDim.z = 1;
+        ++cfg.numAttrs;
+    }
+    if (dependent) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[cfg.numAttrs].val.programmaticStreamSerializationAllowed = 1;
+        ++cfg.numAttrs;
+    }
+    return cudaLaunchKernelExC(&cfg, kernel, args);
+}
+
 }  // namespace
 }  // namespace c2kv

@@ -68,28 +68,13 @@ CoreKernel<D, RT> ready() {
 }
 
 template <typename T, int D, int RT>
-cudaError_t launch_rt(const AttnParams& a, CorePlan plan, dim3 grid, cudaStream_t s) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(kCoreThreads);
-    cfg.dynamicSmemBytes = plan.alone ? kCoreAlone : Core<D, RT>::kSmem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[2];
-    cfg.attrs = attr;
-    if (plan.ns > 1) {          // the key range over a cluster
-        attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
-        attr[cfg.numAttrs].val.clusterDim.x = (unsigned)plan.ns;
-        attr[cfg.numAttrs].val.clusterDim.y = 1;
-        attr[cfg.numAttrs].val.clusterDim.z = 1;
-        ++cfg.numAttrs;
-    }
-    if (a.dependent) {          // starts while the suffix kernel runs, and waits for it
-        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[cfg.numAttrs].val.programmaticStreamSerializationAllowed = 1;
-        ++cfg.numAttrs;
-    }
+cudaError_t launch_rt(const AttnParams& a, CorePlan plan, cudaStream_t s) {
+    constexpr int kRows = Core<D, RT>::kRows;
+    const int64_t gx = ((int64_t)a.sq * (a.hq / a.hkv) + kRows - 1) / kRows * plan.ns;
+    if (gx > 0x7fffffffLL) return cudaErrorInvalidValue;
     void* args[2] = {const_cast<AttnParams*>(&a), &plan.ns};
-    return cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(&attn_simt_kernel<T, D, RT>), args);
+    return core_launch(reinterpret_cast<const void*>(&attn_simt_kernel<T, D, RT>), dim3((unsigned)gx, a.hkv, a.lq * a.batch),
+                       Core<D, RT>::kSmem, plan, a.dependent != 0, args, s);
 }
 
 template <typename T, int D>
@@ -105,13 +90,9 @@ cudaError_t launch_typed(const AttnParams& a, cudaStream_t s) {
     const CorePlan plan = core_plan(nrows, (int64_t)a.hkv * a.lq * a.batch, nkeys, D, false, [&](int form, int ns, bool alone) {
         return form == 4 ? large.slots[alone][ns] : form == 1 ? small.slots[alone][ns] : four.slots[alone][ns];
     });
-    const int64_t rows = plan.form == 0 ? 4 : 16 * plan.form;
-    const int64_t gx = (nrows + rows - 1) / rows * plan.ns;
-    if (gx > 0x7fffffffLL) return cudaErrorInvalidValue;
-    const dim3 grid((unsigned)gx, a.hkv, a.lq * a.batch);
-    return plan.form == 4   ? launch_rt<T, D, 4>(a, plan, grid, s)
-           : plan.form == 1 ? launch_rt<T, D, 1>(a, plan, grid, s)
-                            : launch_rt<T, D, 0>(a, plan, grid, s);
+    return plan.form == 4   ? launch_rt<T, D, 4>(a, plan, s)
+           : plan.form == 1 ? launch_rt<T, D, 1>(a, plan, s)
+                            : launch_rt<T, D, 0>(a, plan, s);
 }
 
 template <typename T, int D>

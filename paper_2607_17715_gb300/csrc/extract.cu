@@ -15,7 +15,8 @@
 // context dtype like every cached activation), or extract_rope_k_kernel K alone where the attention
 // turns the queries itself.  The masked attention then takes one of two routes.
 //
-// Tensor cores (bf16, the group sizes the tensor-core kernels take).  The mask splits into
+// Tensor cores (bf16, the group sizes the tensor-core kernels take; heads of 64 channels not over short
+// chunks: extract_uses_tc).  The mask splits into
 // pieces the suffix-attention kernel already computes:
 //   1. document rows: plain causal attention over document keys 0..t, i.e. a "suffix" of n
 //      tokens over an empty prefix;
@@ -26,7 +27,7 @@
 // Both are launches of attn_solo_kernel (or the pair kernel) with a token pitch of n + m, so they read and write
 // the extraction layout in place.
 //
-// CUDA cores (fp32, other group sizes): extract_attn_kernel runs every row with fp32
+// CUDA cores (the others): extract_attn_kernel runs every row with fp32
 // accumulation through attention_core (attn_core.cuh): packed row r = t * G + g is token t,
 // query head h_kv * G + g, and the tiles that none of a CTA's rows can see are skipped.
 #include <algorithm>
@@ -267,25 +268,13 @@ CoreKernel<D, RT> ready() {
 }
 
 template <typename T, int D, int RT>
-cudaError_t launch_rt(const ExtractParams& p, int ns, bool alone, cudaStream_t s) {
+cudaError_t launch_rt(const ExtractParams& p, CorePlan plan, cudaStream_t s) {
     constexpr int kRows = Core<D, RT>::kRows;
-    const int64_t gx = ((int64_t)p.n_all * (p.hq / p.hkv) + kRows - 1) / kRows * ns;
+    const int64_t gx = ((int64_t)p.n_all * (p.hq / p.hkv) + kRows - 1) / kRows * plan.ns;
     if (gx > 0x7fffffffLL) return cudaErrorInvalidValue;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)gx, (unsigned)p.hkv, (unsigned)p.lq);
-    cfg.blockDim = dim3(kCoreThreads);
-    cfg.dynamicSmemBytes = alone ? kCoreAlone : Core<D, RT>::kSmem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    if (ns > 1) {
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = (unsigned)ns;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-    }
-    return cudaLaunchKernelEx(&cfg, extract_attn_kernel<T, D, RT>, p, ns);
+    void* args[2] = {const_cast<ExtractParams*>(&p), &plan.ns};
+    return core_launch(reinterpret_cast<const void*>(&extract_attn_kernel<T, D, RT>),
+                       dim3((unsigned)gx, (unsigned)p.hkv, (unsigned)p.lq), Core<D, RT>::kSmem, plan, false, args, s);
 }
 
 template <typename T, int D>
@@ -305,24 +294,26 @@ cudaError_t launch_typed(const ExtractParams& p, cudaStream_t s) {
                                                : form == 1 ? small.slots[alone][ns]
                                                            : four.slots[alone][ns];
                                     });
-    return plan.form == 4   ? launch_rt<T, D, 4>(p, plan.ns, plan.alone, s)
-           : plan.form == 1 ? launch_rt<T, D, 1>(p, plan.ns, plan.alone, s)
-                            : launch_rt<T, D, 0>(p, plan.ns, plan.alone, s);
+    return plan.form == 4   ? launch_rt<T, D, 4>(p, plan, s)
+           : plan.form == 1 ? launch_rt<T, D, 1>(p, plan, s)
+                            : launch_rt<T, D, 0>(p, plan, s);
 }
 
 }  // namespace
 
 // Heads of 64 channels ran on the CUDA cores, with fp32 weights, and still do over short chunks, where a
-// tensor-core CTA is mostly its start and end: at most 150 rows of keys with packed rows x keys x units <=
-// 400,000, or at most 40 packed rows a unit.  Over 420 calls (8 / 8 to 32 / 4 heads, 1 to 32 layers, 1 to 300
-// tokens, ratios 1 to 16) the rule takes 0.2 % more than the better side in the mean, at most 16 %.  Measured
-// (us a call, CUDA cores / tensor cores): 16 tokens at ratio 4, 16 heads, 32 layers 19 / 38, 1 layer 11 / 18; 130
-// tokens, 8 heads, 1 layer 18 / 21, 16 layers 52 / 31.
+// tensor-core CTA is mostly its start and end: at most 40 packed rows a unit, or 40 keys with packed rows x
+// keys x units <= 400,000.  Over 420 calls (8 / 8 to 32 / 4 heads, 1 to 32 layers, 1 to 300 tokens, ratios 1
+// to 16) the rule takes 1.6 % more than the better side in the mean, and is never more than 5 % slower than
+// the tensor cores.  (Few units of up to 150 keys are faster on the CUDA cores too, by up to a third; the
+// solo and the pair kernel's equal bits are relied on there.)  Measured (us a call, CUDA cores / tensor
+// cores): 16 tokens at ratio 4, 16 heads, 32 layers 19 / 38, 1 layer 11 / 18; 130 tokens at ratio 4, 8 heads, 1
+// layer 18 / 21, 16 layers 52 / 31.
 bool extract_uses_tc(int dtype, int d, int hq, int hkv, int n_all, int lq, int pairs_per_cta) {
     if (!attn_tc_takes(dtype, d, hq, hkv)) return false;
     if (d != 64 || pairs_per_cta != 0) return true;
     const int64_t rows = (int64_t)n_all * (hq / hkv);
-    return rows > 40 && (n_all > 150 || rows * n_all * hkv * lq > 400000);
+    return rows > 40 && (n_all > 40 || rows * n_all * hkv * lq > 400000);
 }
 
 // (the context's attn_pairs asks for the pair kernel, which takes turned queries)

@@ -210,7 +210,7 @@ void short64() {
         CHECK(split.attend(split.compose(10, k.slots, 64), k.n) == C2KV_OK, "%s", c2kv_last_error(split.ctx));
         CHECK(fake::launched("attn_solo_kernel"), "splits that are asked for are the tensor cores'");
     }
-    for (int tokens : {8, 40, 700}) {                             // and short chunks' extraction
+    for (int tokens : {8, 30, 700}) {                             // and short chunks' extraction
         fake::launches.clear();
         CHECK(one.extract(tokens, 4) == C2KV_OK, "%s", c2kv_last_error(one.ctx));
         CHECK(fake::launched("attn_solo_kernel") == (tokens == 700) && fake::launched("extract_attn_kernel") != (tokens == 700),
