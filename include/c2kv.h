@@ -59,7 +59,8 @@ typedef int32_t c2kv_status;
 #define C2KV_MODE_HOST     3  /* stored-form slots that stay in pinned host memory (no copy)   */
 
 /* c2kv_attend kernel choice */
-#define C2KV_ATTN_AUTO   0    /* tensor-core kernels where they apply (also d = 64), else SIMT */
+#define C2KV_ATTN_AUTO   0    /* tensor-core kernels where they apply (also d = 64, unless few
+                                 rows meet few keys), else SIMT                               */
 #define C2KV_ATTN_SIMT   1    /* CUDA-core fp32-accumulate kernel (any dtype)        */
 #define C2KV_ATTN_TC     2    /* tcgen05 / TMEM tensor-core kernel (bf16, d = 128)    */
 
@@ -72,7 +73,8 @@ typedef int32_t c2kv_status;
 /* c2kv_compose_attend: when the fused compose + attention kernel runs */
 #define C2KV_FUSE_AUTO   0    /* when each (layer, request, KV head) has a single pair of
                                  128-row query tiles, n_suffix * Hq / Hkv <= 256: every
-                                 stored slot is then read and turned by exactly one CTA   */
+                                 stored slot is then read and turned by exactly one CTA;
+                                 and it is expected to be the faster (see below)          */
 #define C2KV_FUSE_NEVER  1    /* always compose, then attend                           */
 #define C2KV_FUSE_ALWAYS 2    /* whenever the fused kernel takes the call; with several
                                  pairs of query tiles one CTA runs them in turn, the last
@@ -95,14 +97,19 @@ typedef struct c2kv_config {
     int32_t attn_impl;         /* C2KV_ATTN_AUTO / _SIMT / _TC                                */
     int32_t attn_split;        /* tensor-core attention key-range splits per work unit:
                                   0 = chosen per call (split only when the units would leave
-                                  SMs idle), 1 = never, n <= 16 = always n (partials
-                                  merged by an exact log-sum-exp combine)                     */
+                                  SMs idle, and not when there is no memory for the
+                                  partials), 1 = never, n <= 16 = always n (partials merged by
+                                  an exact log-sum-exp combine)                               */
     int32_t fuse;              /* C2KV_FUSE_AUTO / _NEVER / _ALWAYS (c2kv_compose_attend)     */
     int32_t storage;           /* C2KV_STORAGE_LOCAL_ROPE (0) or C2KV_STORAGE_PRE_ROPE          */
     int32_t attn_pairs;        /* pairs of 128-row query tiles one tensor-core attention CTA
                                   runs in turn: 0 = chosen per launch (several only where
-                                  that saves a wave of CTAs), n >= 1 = n (fewer where a
-                                  (layer, request, KV head) has fewer pairs)                  */
+                                  that saves a wave of CTAs, or one query tile a CTA, in
+                                  another kernel).  n >= 1 asks for the pair kernel, with n in
+                                  turn (fewer where a (layer, request, KV head) has fewer
+                                  pairs), also where heads of 64 channels would run on the CUDA
+                                  cores, and in c2kv_extract_attention for a pass of its own that
+                                  turns the queries                                           */
 } c2kv_config;
 
 /* Chunk metadata (c2kv_chunk_info). */

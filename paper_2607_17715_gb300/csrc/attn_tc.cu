@@ -2999,7 +2999,7 @@ cudaError_t prepare_tc(const AttnParams& a, TcParams& p, dim3& grid) {
     // CTAs: the choice with the least rounds x (1.5 + pairs x (8 + 1.6 a key tile)).  Measured at 1 / 2
     // pairs a CTA (us a call; 32 / 8 heads, 11 key tiles): 256 pairs 63.3 / 61.1, 384 89.7 / 106.4, 640
     // (four a head) 131 / 146, 1024 204 / 220; 64 / 8 heads, 22 key tiles, 512 pairs (16 a head) 170 /
-    // 171, three in turn 228.  The context's attn_pairs setting caps the choice.
+    // 171, three in turn 228.  The context's attn_pairs setting takes the choice's place.
     int64_t pg = 1;
     if (kSolo) {
         if (p.n_split > 1 && (p.tickets || kSif)) return cudaErrorInvalidValue;

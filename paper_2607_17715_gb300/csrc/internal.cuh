@@ -146,8 +146,8 @@ struct AttnParams {
     int32_t n_split;         // key-range splits per work unit (1 = write O directly)
     float* part_o;           // n_split > 1: [n_split][Lq][Btot][Sq][Hq][d] fp32, normalised
     float* part_lse;         // n_split > 1: [n_split][Lq][Btot][Hq][Sq] fp32, log2 domain
-    int32_t pairs_per_cta;   // tensor-core kernel: at most this many pairs of query tiles per
-                             // CTA (0 = chosen per launch)
+    int32_t pairs_per_cta;   // 0, or the pair kernel with this many pairs of query tiles a CTA (at
+                             // most a unit's) in place of the choice per launch
     int32_t dependent;       // tensor-core kernel and its merge: launched as the programmatic
                              // dependent of the kernel before them on the stream (each waits
                              // for that grid before it reads memory)
