@@ -1412,9 +1412,8 @@ c2kv_status c2kv_decode(c2kv_ctx* c, c2kv_cache* cache, int32_t layer, const voi
         // from 3 key tiles as well, its fp32 weights kept (as three bf16 terms).
         // Measured, CUDA cores / tensor cores with fp32 weights (us a call, one layer, 8 KV heads; key
         // tiles 3, 9, 18): G = 8, 32 requests 30 / 26, 71 / 40, 123 / 62, 128 requests 88 / 81, 226 /
-        // 128, 405 / 210, but one tile 53 / 63.  G = 4 with two terms of the weights, 32 requests: 9
-        // tiles 39 / 43, 18 65 / 69.  bf16 weights, one wave: 16 requests x 1160 keys 30 / 18, 8 x
-        // 32900 212 / 190.
+        // 128, 405 / 210, but one tile 53 / 63.  G = 4, 32 requests: 3 tiles 18 / 26, 9 39 / 40, 18 65 /
+        // 62.  bf16 weights, one wave: 16 requests x 1160 keys 30 / 18, 8 x 32900 212 / 190.
         const int64_t tiles_max = (n_keys_max + 127) / 128;
         const int32_t group = hq / hkv;
         const bool tc = c->cfg.attn_impl != C2KV_ATTN_SIMT && c2kv::attn_tc_supported(c->cfg.dtype, d, hq, hkv);
